@@ -20,6 +20,7 @@ namespace {
 constexpr int kSMs = 152;           // GB300: 2 dies x 76 SMs
 constexpr int kGlNodes = 128;       // Gauss-Legendre nodes for the ES transform
 constexpr int kMaxGramCtas = 2 * kSMs;
+constexpr int kMaxGramF64Splits = 256;
 constexpr int kGramTmaMinAssets = 192;  // default switch to the pre-split contraction
 
 struct Prof {
@@ -259,7 +260,6 @@ struct mm_plan_s {
   unsigned long long* gapbits = nullptr;
   void* wsq = nullptr;
   void* partial = nullptr;        // FP64 path: per-split partial tiles
-  size_t partial_bytes = 0;
   float* acc[2] = {nullptr, nullptr};  // mixed path: FP32 accumulators, used alternately
   void* tma_hi = nullptr;         // mixed path, pre-split contraction: operand hi and lo planes
   void* tma_lo = nullptr;         // (Dpad x kpc complex modes, pad rows zero)
@@ -636,20 +636,17 @@ GramParams gram_params(mm_plan p, int N) {
   g.N = N;
   g.ld = N + 1;
   g.Dp = (g.D + 3) / 4 * 4;
-  g.tile = p->fp64 ? 64 : 128;
+  if (p->fp64) {
+    gram_f64_shape(&g, kMaxGramF64Splits);
+    return g;
+  }
+  g.tile = 128;
   g.ntiles = (g.D + g.tile - 1) / g.tile;
   g.npairs = g.ntiles * (g.ntiles + 1) / 2;
-  g.chunk = p->fp64 ? 16 : (p->desc.prec == MM_PREC_MIXED_BF16X3 ? 32 : 16);
+  g.chunk = p->desc.prec == MM_PREC_MIXED_BF16X3 ? 32 : 16;
   g.nchunks = (N + 1 + g.chunk - 1) / g.chunk;
   int S;
-  if (p->fp64) {
-    // split K so that all SMs get work while the partial tiles stay a small
-    // fraction of the operand bytes
-    const double a_bytes = (double)g.D * 2.0 * (N + 1) * 8.0;
-    const double tile_bytes = (double)g.tile * g.tile * 8.0;
-    const int s_traffic = (int)std::max(1.0, ceil(a_bytes / (4.0 * g.npairs * tile_bytes)));
-    S = std::max(1, std::min({g.nchunks, std::max(1, kMaxGramCtas / g.npairs), s_traffic}));
-  } else if (gram_uses_tma(p)) {
+  if (gram_uses_tma(p)) {
     // one CTA per SM (its stage ring fills the shared memory): one wave
     S = std::max(1, std::min((g.nchunks + 1) / 2, std::max(1, kSMs / g.npairs)));
   } else {
@@ -771,7 +768,6 @@ mm_status corr_impl(mm_plan p, const void* coeffs, int N, void* sigma, void* R, 
   if (p->desc.basis == MM_BASIS_FEJER && N < 1) return MM_ERR_CUTOFF;
   p->last = st;
   GramParams g = gram_params(p, N);
-  if (p->fp64 && (size_t)g.npairs * g.splits * g.tile * g.tile * p->rs > p->partial_bytes) return MM_ERR_UNSUPPORTED;
   if (p->w_N != N || p->w_basis != (int)p->desc.basis) {
     StageScope sc(p, MM_STAGE_SETUP, st);
     MM_CUDA(launch_gram_weights(p->desc.basis, N, p->fp64, p->wsq, st));
@@ -1008,10 +1004,8 @@ mm_status plan_create_impl(const mm_plan_desc* desc, int gsize, bool batch, mm_p
   A(&p->wsq, Np1 * p->rs);
   if (!batch) {
     GramParams g = gram_params(p, d.N_max);
-    size_t ctas = std::max<size_t>((size_t)kMaxGramCtas, (size_t)g.npairs);
     if (p->fp64) {
-      p->partial_bytes = ctas * g.tile * g.tile * p->rs;
-      A(&p->partial, p->partial_bytes);
+      A(&p->partial, gram_f64_partial_bytes(d.D));
     } else {
       A((void**)&p->acc[0], D * (size_t)g.Dp * sizeof(float));
       A((void**)&p->acc[1], D * (size_t)g.Dp * sizeof(float));

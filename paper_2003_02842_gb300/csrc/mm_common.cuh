@@ -149,7 +149,7 @@ struct GramParams {
   int D;
   int N;             // modes k = 0..N
   int ld;            // leading dimension (complex elements) of the coefficients
-  int tile;          // output tile edge (128 tensor path, 64 fp64 path)
+  int tile;          // output tile edge (128 tensor path, 4 fp64 path)
   int ntiles;        // ceil(D / tile)
   int npairs;        // ntiles (ntiles+1) / 2
   int splits;        // split-K factor
@@ -233,6 +233,8 @@ cudaError_t launch_spread_fft(const int64_t* off, const int* rb0, const void* rd
 size_t fft_rows_smem(const FftParams& f, bool fp64);
 
 cudaError_t launch_gram_weights(int basis, int N, bool fp64, void* wsq, cudaStream_t s);
+void gram_f64_shape(GramParams* g, int max_splits);  // tile .. splits of the FP64 contraction, from D and N
+size_t gram_f64_partial_bytes(int D);                // partial tiles of any such shape
 cudaError_t launch_gram_f64(const void* coeffs, const GramParams& g, const double* wsq,
                             double* partial, cudaStream_t s);
 cudaError_t launch_gram_tc(int mode, const void* coeffs, const GramParams& g, const float* wsq,

@@ -25,9 +25,11 @@ namespace {
 constexpr int kNaMaxD = 128;
 constexpr int kNaMaxN = 65535;
 constexpr int kNaMaxSplits = 16;
-// partial tiles: FP32 path 1 pair of 128 x 128 floats; FP64 path up to
-// 3 pairs of 64 x 64 doubles (D <= 128 gives at most 2 x 2 tiles of 64)
-constexpr size_t kNaPartialBytes = (size_t)kNaMaxSplits * 3 * 64 * 64 * 8;  // >= the FP32 accumulator
+// partial tiles: FP32 path 1 pair of 128 x 128 floats; FP64 path up to 528
+// pairs of 4 x 4 doubles per split (D <= 128 gives at most 32 tiles of 4),
+// 1.1 MB at 16 splits
+constexpr size_t kNaPartialBytes = (size_t)kNaMaxSplits * 3 * 64 * 64 * 8;
+static_assert((size_t)kNaMaxSplits * (32 * 33 / 2) * 16 * 8 <= kNaPartialBytes, "FP64 partial tiles");
 constexpr size_t kNaWeightBytes = (size_t)(kNaMaxN + 1) * 8;
 constexpr size_t kNaStatusBytes = 256;
 constexpr size_t kNaBytes = kNaPartialBytes + kNaWeightBytes + kNaStatusBytes;
@@ -95,14 +97,18 @@ extern "C" mm_status mm_corr_noalloc(int32_t D, int32_t N, mm_basis basis, mm_pr
   g.N = N;
   g.ld = N + 1;
   g.Dp = (D + 3) / 4 * 4;
-  g.tile = fp64 ? 64 : 128;
-  g.ntiles = (D + g.tile - 1) / g.tile;
-  g.npairs = g.ntiles * (g.ntiles + 1) / 2;
-  g.chunk = fp64 ? 16 : (prec == MM_PREC_MIXED_BF16X3 ? 32 : 16);
-  g.nchunks = (N + 1 + g.chunk - 1) / g.chunk;
-  const int S = g.nchunks < kNaMaxSplits ? g.nchunks : kNaMaxSplits;
-  g.chunks_per_split = (g.nchunks + S - 1) / S;
-  g.splits = (g.nchunks + g.chunks_per_split - 1) / g.chunks_per_split;
+  if (fp64) {
+    gram_f64_shape(&g, kNaMaxSplits);
+  } else {
+    g.tile = 128;
+    g.ntiles = (D + g.tile - 1) / g.tile;
+    g.npairs = g.ntiles * (g.ntiles + 1) / 2;
+    g.chunk = prec == MM_PREC_MIXED_BF16X3 ? 32 : 16;
+    g.nchunks = (N + 1 + g.chunk - 1) / g.chunk;
+    const int S = g.nchunks < kNaMaxSplits ? g.nchunks : kNaMaxSplits;
+    g.chunks_per_split = (g.nchunks + S - 1) / S;
+    g.splits = (g.nchunks + g.chunks_per_split - 1) / g.chunks_per_split;
+  }
 
   cudaStream_t st = (cudaStream_t)stream;
   // the status word and the mixed path's accumulator must start at zero; the
