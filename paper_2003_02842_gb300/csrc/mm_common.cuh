@@ -197,10 +197,14 @@ cudaError_t launch_spread_poly(const int64_t* off, const int* rb0, const void* r
 cudaError_t launch_spread_f64(const int64_t* off, const int* rb0, const void* rd, const void* rv,
                               const SpreadParams& p, double* grid, const int* status, cudaStream_t s);
 
-cudaError_t launch_gl_nodes(int nq, double* x, double* w, cudaStream_t s);
+// Quadrature nodes y and weights f of the ES transform, its Chebyshev series
+// (mixed precision) and the per-cutoff tables (mm_fft.cu).
+constexpr int kEsChebMax = 64;
+cudaError_t launch_es_nodes(int nq, double beta, double* y, double* f, cudaStream_t s);
+cudaError_t launch_es_fit(int nq, int msp, const double* y, const double* f, double* cheb, cudaStream_t s);
 cudaError_t launch_setup_tables(int kernel, int msp, int64_t Mr, int N, int64_t n,
-                                const SpreadParams& sp, double tau, const double* glx,
-                                const double* glw, int nq, void* W, void* U, void* decon,
+                                const SpreadParams& sp, double tau, const double* esy,
+                                const double* esf, int nq, const double* cheb, void* W, void* U, void* decon,
                                 bool fp64, cudaStream_t s);
 cudaError_t launch_fft_cols_f32(float* grid, const FftParams& f, int D, const void* W, const int* status, cudaStream_t s);
 cudaError_t launch_fft_cols_f64(double* grid, const FftParams& f, int D, const void* W, const int* status, cudaStream_t s);

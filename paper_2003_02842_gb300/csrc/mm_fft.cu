@@ -179,8 +179,13 @@ __global__ void __launch_bounds__(kFftThreads) k_fft_rows(const Cplx<T>* __restr
 }
 
 // ------------------------------------------------------------ tables
-// Gauss-Legendre nodes on [-1, 1] by Newton's method on P_nq (one thread per node).
-__global__ void k_gl_nodes(int nq, double* x, double* w) {
+// Quadrature of the ES kernel's transform (steps D.1-D.2 of Algorithm 10):
+//   phihat(k) = 2 alpha I(alpha k), I(theta) = int_0^1 e(y) cos(theta y) dy,
+//   e(y) = exp(beta (sqrt(1 - y^2) - 1)), alpha = 2 pi M_sp / M_r,
+// by nq-point Gauss-Legendre in y: nodes y_q and weights f_q = w_q e(y_q),
+// which depend on the plan's M_sp alone. Legendre roots by Newton's method on
+// P_nq (one thread per node).
+__global__ void k_es_nodes(int nq, double beta, double* y, double* f) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nq) return;
   double zz = cos(kPi * (i + 0.75) / (nq + 0.5));
@@ -204,22 +209,68 @@ __global__ void k_gl_nodes(int nq, double* x, double* w) {
     p1 = p2;
   }
   dp = nq * (zz * p1 - p0) / (zz * zz - 1.0);
-  x[i] = zz;
-  w[i] = 2.0 / ((1.0 - zz * zz) * dp * dp);
+  const double w = 2.0 / ((1.0 - zz * zz) * dp * dp);
+  const double yy = 0.5 * (zz + 1.0);
+  y[i] = yy;
+  f[i] = 0.5 * w * exp(beta * (sqrt(fmax(1.0 - yy * yy, 0.0)) - 1.0));
 }
 
-cudaError_t launch_gl_nodes(int nq, double* x, double* w, cudaStream_t s) {
-  k_gl_nodes<<<(nq + 127) / 128, 128, 0, s>>>(nq, x, w);
+cudaError_t launch_es_nodes(int nq, double beta, double* y, double* f, cudaStream_t s) {
+  k_es_nodes<<<(nq + 31) / 32, 32, 0, s>>>(nq, beta, y, f);
+  return cudaGetLastError();
+}
+
+// Chebyshev coefficients of I(theta) in x = 2 (theta / theta_max)^2 - 1 (I is
+// even and entire in theta; theta = alpha k <= pi M_sp / 2 = theta_max for
+// every mode of every cutoff, because k <= N < M_r / 4). The coefficients
+// decay like the Bessel functions J_2i(theta_max): es_cheb_terms() of them
+// leave an error of a few 1e-14 of I (checked against the quadrature for
+// M_sp = 1..30), far below float32 rounding. So a mixed-precision plan fits
+// once and its per-cutoff tables need some 25 float64 multiply-adds a mode
+// instead of 128 exponentials and cosines (k_setup_tables).
+__global__ void __launch_bounds__(1024) k_es_fit(int nq, const double* __restrict__ y, const double* __restrict__ f,
+                                                 double theta_max, int nt, double* cheb) {
+  __shared__ double val[kEsChebMax];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int m = warp; m < nt; m += 32) {
+    const double theta = theta_max * sqrt(0.5 * (cospi((m + 0.5) / nt) + 1.0));
+    double acc = 0.0;
+    for (int q = lane; q < nq; q += 32) acc = fma(f[q], cos(theta * y[q]), acc);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) val[m] = acc;
+  }
+  __syncthreads();
+  for (int i = warp; i < nt; i += 32) {
+    double acc = 0.0;
+    for (int m = lane; m < nt; m += 32) acc = fma(val[m], cospi(i * (m + 0.5) / nt), acc);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) cheb[i] = (i == 0 ? 1.0 : 2.0) / nt * acc;
+  }
+}
+
+int es_cheb_terms(int msp) { return 12 + (9 * msp + 9) / 10; }  // 18 at M_sp = 6, 39 at 30
+
+cudaError_t launch_es_fit(int nq, int msp, const double* y, const double* f, double* cheb, cudaStream_t s) {
+  const int nt = es_cheb_terms(msp);
+  if (nt > kEsChebMax) return cudaErrorInvalidValue;
+  k_es_fit<<<1, 1024, 0, s>>>(nq, y, f, 0.5 * kPi * msp, nt, cheb);
   return cudaGetLastError();
 }
 
 // W[j] = e^{-2 pi i j / n} (j < n); U[k] = e^{-i pi k / n} (k <= N);
 // decon[k]: the F-convention deconvolution factor of Eq. (14) for the kernel
-// as spread by mm_spread.cu (so F(k) = G(k) decon(k)).
+// as spread by mm_spread.cu (so F(k) = G(k) decon(k)). Bound by the float64
+// pipe. The ES transform is the Chebyshev series of k_es_fit for float32
+// tables and the quadrature itself (its exponentials already in f) for
+// float64 ones. A serving request builds these tables for its own cutoff: with
+// 128 exp and cos a mode they took 421 us a request on the serving
+// workload (eight requests in flight), now 9.4 us.
 template <typename T>
-__global__ void k_setup_tables(int kernel, int msp, int64_t Mr, int N, int64_t n, double es_beta, double kb_b,
-                               double kb_inv_phi0, double tau, const double* __restrict__ glx,
-                               const double* __restrict__ glw, int nq, Cplx<T>* W, Cplx<T>* U, T* decon) {
+__global__ void k_setup_tables(int kernel, int msp, int64_t Mr, int N, int64_t n, double kb_b, double kb_inv_phi0,
+                               double tau, const double* __restrict__ esy, const double* __restrict__ esf, int nq,
+                               const double* __restrict__ cheb, int nt, Cplx<T>* W, Cplx<T>* U, T* decon) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) {
     double s, c;
@@ -241,13 +292,21 @@ __global__ void k_setup_tables(int kernel, int msp, int64_t Mr, int N, int64_t n
       const double arg = (double)msp * sqrt(fmax(kb_b * kb_b - a * a, 0.0));
       v = 1.0 / (2.0 * kPi * kb_inv_phi0 * cyl_bessel_i0(arg));
     } else {
-      // steps D.1-D.2 of Algorithm 10: phihat(k) = 2 alpha int_0^1
-      // exp(beta (sqrt(1-y^2) - 1)) cos(alpha k y) dy, Gauss-Legendre in y
       const double alpha = kPi * 2.0 * msp / (double)Mr;
       double acc = 0.0;
-      for (int q = 0; q < nq; ++q) {
-        const double y = 0.5 * (glx[q] + 1.0);
-        acc += 0.5 * glw[q] * exp(es_beta * (sqrt(fmax(1.0 - y * y, 0.0)) - 1.0)) * cos(alpha * k * y);
+      if constexpr (sizeof(T) == 4) {
+        // Clenshaw's recurrence at x = 2 (theta / theta_max)^2 - 1,
+        // theta / theta_max = 4 k / M_r
+        const double r = 4.0 * k / (double)Mr, x2 = 4.0 * r * r - 2.0;  // 2 x
+        double b1 = 0.0, b2 = 0.0;
+        for (int q = nt - 1; q >= 1; --q) {
+          const double b0 = fma(x2, b1, cheb[q] - b2);
+          b2 = b1;
+          b1 = b0;
+        }
+        acc = fma(0.5 * x2, b1, cheb[0] - b2);
+      } else {
+        for (int q = 0; q < nq; ++q) acc = fma(esf[q], cos(alpha * k * esy[q]), acc);
       }
       const double ph = 2.0 * alpha * acc;
       v = 1.0 / ((double)Mr * ph);
@@ -257,16 +316,18 @@ __global__ void k_setup_tables(int kernel, int msp, int64_t Mr, int N, int64_t n
 }
 
 cudaError_t launch_setup_tables(int kernel, int msp, int64_t Mr, int N, int64_t n, const SpreadParams& sp,
-                                double tau, const double* glx, const double* glw, int nq, void* W, void* U,
-                                void* decon, bool fp64, cudaStream_t s) {
+                                double tau, const double* esy, const double* esf, int nq, const double* cheb,
+                                void* W, void* U, void* decon, bool fp64, cudaStream_t s) {
   const int64_t m = n > (int64_t)N + 1 ? n : (int64_t)N + 1;
-  const int blocks = (int)((m + 255) / 256);
+  const int nth = 128;
+  const int blocks = (int)((m + nth - 1) / nth);
+  const int nt = es_cheb_terms(msp);
   if (fp64)
-    k_setup_tables<double><<<blocks, 256, 0, s>>>(kernel, msp, Mr, N, n, sp.es_beta, sp.kb_b, sp.kb_inv_phi0, tau,
-                                                  glx, glw, nq, (Cplx<double>*)W, (Cplx<double>*)U, (double*)decon);
+    k_setup_tables<double><<<blocks, nth, 0, s>>>(kernel, msp, Mr, N, n, sp.kb_b, sp.kb_inv_phi0, tau, esy, esf, nq,
+                                                  cheb, nt, (Cplx<double>*)W, (Cplx<double>*)U, (double*)decon);
   else
-    k_setup_tables<float><<<blocks, 256, 0, s>>>(kernel, msp, Mr, N, n, sp.es_beta, sp.kb_b, sp.kb_inv_phi0, tau,
-                                                 glx, glw, nq, (Cplx<float>*)W, (Cplx<float>*)U, (float*)decon);
+    k_setup_tables<float><<<blocks, nth, 0, s>>>(kernel, msp, Mr, N, n, sp.kb_b, sp.kb_inv_phi0, tau, esy, esf, nq,
+                                                 cheb, nt, (Cplx<float>*)W, (Cplx<float>*)U, (float*)decon);
   return cudaGetLastError();
 }
 
