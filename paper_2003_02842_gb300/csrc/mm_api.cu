@@ -271,7 +271,9 @@ struct mm_plan_s {
   double* pw_A = nullptr;         // the repair's working matrix and eigenvectors
   double* pw_V = nullptr;         // (allocated on first use)
   int* pw_clip = nullptr;
-  void* pw_sync = nullptr;        // the multi-CTA repair's barrier words
+  void* pw_sync = nullptr;        // the repair's barrier words and results
+  void* pw_part = nullptr;        // split partial sums
+  void* pw_log = nullptr;         // the one-CTA repair's rotations
   int acc_sel = 0;
   bool acc_dirty = true;          // clear both before the next contraction
   int acc_D = -1;                 // D whose D x Dp region the last epilogue cleared
@@ -356,7 +358,7 @@ void free_all(mm_plan p) {
   void* ptrs[] = {p->grid, p->rec_b0, p->rec_d, p->rec_v, p->W, p->atw, p->U, p->decon, p->esy, p->esf, p->es_cheb, p->bounds, p->gscale, p->status, p->gapbits, p->wsq,
                   p->partial, p->acc[0], p->acc[1], p->gram_done, p->pw_N, p->pw_sig, p->pw_A,
                   p->pw_V, p->pw_clip, p->s_off, p->s_t, p->s_p, p->s_coef,
-                  p->s_sigma, p->s_R, p->asset_order, p->tma_hi, p->tma_lo, p->pw_sync};
+                  p->s_sigma, p->s_R, p->asset_order, p->tma_hi, p->tma_lo, p->pw_sync, p->pw_part, p->pw_log};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   if (p->h_status) cudaFreeHost(p->h_status);
@@ -1099,27 +1101,37 @@ mm_status mm_corr_pairwise(mm_plan p, const void* d_coeffs, int32_t N_coeffs, co
   const int lo = p->desc.basis == MM_BASIS_FEJER ? 1 : 0;
   for (int i = 0; i < D; ++i)
     if (h_N[i] < lo || h_N[i] > N_coeffs) return MM_ERR_CUTOFF;
-  if (!p->pw_N) {
-    const size_t dd = (size_t)p->desc.D * p->desc.D * sizeof(double);
-    mm_status a = dalloc(p, (void**)&p->pw_N, (size_t)p->desc.D * sizeof(int));
-    if (a == MM_OK) a = dalloc(p, (void**)&p->pw_sig, dd);
-    if (a == MM_OK && p->desc.D <= pairwise_psd_max_assets()) a = dalloc(p, (void**)&p->pw_A, dd);
-    if (a == MM_OK && p->desc.D <= pairwise_psd_max_assets()) a = dalloc(p, (void**)&p->pw_V, dd);
-    if (a == MM_OK) a = dalloc(p, (void**)&p->pw_clip, sizeof(int));
-    if (a == MM_OK) a = dalloc(p, &p->pw_sync, psd_sync_bytes());
-    if (a != MM_OK) return a;
-  }
   cudaStream_t st = (cudaStream_t)stream;
+  if (!p->pw_part) {  // first use; a failed attempt is resumed by the next call
+    const size_t dd = (size_t)p->desc.D * p->desc.D * sizeof(double);
+    const bool psd = p->desc.D <= pairwise_psd_max_assets();
+    const size_t part = pairwise_part_bytes(p->desc.D);
+    mm_status a = MM_OK;
+    auto need = [&](void** ptr, size_t bytes) {
+      if (a == MM_OK && !*ptr) a = dalloc(p, ptr, bytes);
+    };
+    need((void**)&p->pw_N, (size_t)p->desc.D * sizeof(int));
+    need((void**)&p->pw_sig, dd);
+    if (psd) need((void**)&p->pw_A, dd);
+    if (psd) need((void**)&p->pw_V, dd);
+    need((void**)&p->pw_clip, sizeof(int));
+    need(&p->pw_sync, psd_sync_bytes());
+    need(&p->pw_log, psd_log_bytes(p->fp64, p->desc.D));
+    need(&p->pw_part, part);
+    if (a != MM_OK) return a;
+    MM_CUDA(cudaMemsetAsync(p->pw_part, 0, part, st));
+  }
   p->last = st;
   MM_CUDA(cudaMemcpyAsync(p->pw_N, h_N, (size_t)D * sizeof(int), cudaMemcpyHostToDevice, st));
   {
     StageScope sc(p, MM_STAGE_GRAM, st);
     MM_CUDA(launch_pairwise(p->fp64, p->desc.basis == MM_BASIS_FEJER, d_coeffs, N_coeffs + 1, p->pw_N, D,
-                            p->pw_sig, st));
+                            p->pw_part, p->pw_sig, st));
   }
   StageScope sc(p, MM_STAGE_REDUCE, st, psd_repair ? 2 : 1);
   int* clip = d_clipped_or_null ? (int*)d_clipped_or_null : p->pw_clip;
-  if (psd_repair) MM_CUDA(launch_psd_repair(p->fp64, p->pw_sig, p->pw_A, p->pw_V, D, clip, p->pw_sync, p->status, st));
+  if (psd_repair) MM_CUDA(launch_psd_repair(p->fp64, p->pw_sig, p->pw_A, p->pw_V, D, clip, p->pw_log, p->pw_sync, p->status,
+                                           st));
   else MM_CUDA(cudaMemsetAsync(clip, 0, sizeof(int), st));
   MM_CUDA(launch_pairwise_out(p->fp64, p->pw_sig, D, d_sigma_or_null, d_R, p->status, st));
   return MM_OK;

@@ -269,12 +269,14 @@ cudaError_t launch_epps(int Dg, bool fejer, bool fp64, const void* coef, int ld,
 
 // Pairwise-cutoff covariance (float64 D x D into sig) and its repair to the
 // nearest positive semi-definite matrix (D <= pairwise_psd_max_assets(): one CTA while the
-// matrix and eigenvectors fit its shared memory, else every SM under a cooperative launch).
+// matrix fits its shared memory, else every SM under a cooperative launch).
 int pairwise_psd_max_assets();
 cudaError_t launch_pairwise(bool fp64, bool fejer, const void* coeffs, int ld, const int* Nv, int D,
-                            double* sig, cudaStream_t s);
-cudaError_t launch_psd_repair(bool fp64, double* sig, double* A, double* V, int D, int* clipped, void* sync,
-                              int* status, cudaStream_t s);
+                            void* part, double* sig, cudaStream_t s);
+size_t pairwise_part_bytes(int D);         // split partial sums and zeroed arrival counters
+cudaError_t launch_psd_repair(bool fp64, double* sig, double* A, double* V, int D, int* clipped, void* log,
+                              void* sync, int* status, cudaStream_t s);
+size_t psd_log_bytes(bool fp64, int D);    // the one-CTA iteration's rotation log
 size_t psd_sync_bytes();  // the multi-CTA repair's barrier and reduction words
 cudaError_t launch_pairwise_out(bool fp64, const double* sig, int D, void* sigma, void* R, int* status,
                                 cudaStream_t s);

@@ -9,21 +9,25 @@
 //   Dirichlet  (2 pi)^2 / (2N + 1)      * sum_{k<=N} d_k Re(F_i(k) conj F_j(k)),
 //   Fejer      (2 pi)^2 / ((N + 1) N)   * sum_{k<=N} d_k (N - k) Re(F_i(k) conj F_j(k)),
 // d_0 = 1, d_k = 2 (the -k half folded in); every weight is non-negative.
-// One CTA per 16 x 16 tile of pairs (upper tiles), the two tiles' coefficient
-// rows staged in shared memory 128 modes at a time; a thread owns one pair,
-// sums a chunk in the coefficients' precision and adds it to a float64 sum.
+// A CTA takes a 16 x 16 tile of pairs (upper tiles) and every S-th chunk of 128
+// modes, the two tiles' coefficient rows staged in shared memory; a thread owns
+// one pair, sums a chunk in the coefficients' precision and adds it to a float64
+// sum; the last CTA of a tile adds the S partial sums in order. Latency bound
+// (staging, then dependent adds): with one CTA per tile, 28 CTAs at D = 100,
+// N = 1e4 took 252 us; S filling the SMs takes 34 us.
 //
 // Repair: the matrix closest to Sigma in the Frobenius norm among the positive
 // semi-definite ones is V max(Lambda, 0) V^T (Sigma = V Lambda V^T), the
 // eigenvalue method the paper points to. The eigendecomposition is a cyclic
-// Jacobi iteration in one CTA: each step applies D/2 disjoint
-// rotations in parallel (round-robin pairing), a sweep is D - 1 steps, and
-// the sweeps stop when the off-diagonal norm is below 2 D eps of the matrix
-// norm (eps of the working type: float64 for FP64 plans, float32 for the
-// mixed precisions' float32 Sigma) or after kJacobiSweeps. GB300 issues
-// float64 at a small fraction of the float32 rate, so the mixed path works
-// in float32.
+// Jacobi iteration: each step applies D/2 disjoint rotations (round-robin pairing), a
+// sweep is D - 1 steps, and the sweeps stop when the off-diagonal norm is below
+// 2 D eps of the matrix norm (eps of the working type: float64 for FP64 plans,
+// float32 for the mixed precisions' float32 Sigma) or after kJacobiSweeps. GB300
+// issues float64 at a small fraction of the float32 rate, so the mixed path
+// works in float32.
 #include <math.h>
+
+#include <algorithm>
 
 #include "mm_common.cuh"
 
@@ -33,10 +37,12 @@ namespace {
 
 constexpr int kPT = 16;        // tile edge (pairs per tile: 16 x 16)
 constexpr int kPChunk = 128;   // modes staged per chunk
+constexpr int kPairwiseCtas = 4 * 152;  // CTAs k_pairwise aims at (33 KB of shared memory each in float32)
 constexpr int kJacobiThreads = 1024;
 constexpr int kJacobiSweeps = 40;
-constexpr int kPsdMaxD = 256;  // rotation arrays of the one-CTA repair (it takes what fits 200 KB)
-constexpr size_t kPsdSmemBytes = 200 * 1024;  // the working matrix and eigenvectors in shared memory up to this
+constexpr int kPsdMaxD = 158;      // the one-CTA iteration (at most kPsdRounds blocks a thread); in float64 the
+constexpr int kPsdMaxD64 = 112;    // pipes of all SMs beat those of one beyond this
+constexpr int kPsdRounds = 4;
 
 __device__ __forceinline__ void tile_of(int p, int nt, int& I, int& J) {
   int i = 0;
@@ -58,9 +64,10 @@ __device__ __forceinline__ T2 zero2() {
 
 template <typename T2, typename T, bool FEJER>
 __global__ void __launch_bounds__(256) k_pairwise(const T2* __restrict__ F, int ld, const int* __restrict__ Nv,
-                                                  int D, int nt, double* __restrict__ sig) {
+                                                  int D, int nt, double* __restrict__ part, int* __restrict__ done,
+                                                  double* __restrict__ sig) {
   __shared__ T2 a[kPT][kPChunk + 1], b[kPT][kPChunk + 1];
-  __shared__ int s_nmax;
+  __shared__ int s_nmax, s_last;
   int I, J;
   tile_of(blockIdx.x, nt, I, J);
   const int ti = threadIdx.x / kPT, tj = threadIdx.x % kPT;
@@ -73,7 +80,7 @@ __global__ void __launch_bounds__(256) k_pairwise(const T2* __restrict__ F, int 
   __syncthreads();
   const int nmax = s_nmax;  // the tile's largest pairwise cutoff
   double acc = 0.0;
-  for (int k0 = 0; k0 <= nmax; k0 += kPChunk) {
+  for (int k0 = blockIdx.y * kPChunk; k0 <= nmax; k0 += gridDim.y * kPChunk) {
     for (int e = threadIdx.x; e < kPT * kPChunk; e += blockDim.x) {
       const int r = e / kPChunk, c = e - r * kPChunk;
       const int k = k0 + c;
@@ -82,16 +89,30 @@ __global__ void __launch_bounds__(256) k_pairwise(const T2* __restrict__ F, int 
       b[r][c] = (k <= nmax && rb < D) ? F[(size_t)rb * ld + k] : zero2<T2>();
     }
     __syncthreads();
-    T part = 0;
+    T part_sum = 0;
     const int cend = min(kPChunk - 1, Nij - k0);  // last mode of this pair in the chunk
     for (int c = 0; c <= cend; ++c) {
       const int k = k0 + c;
       T w = k == 0 ? (T)1 : (T)2;
       if (FEJER) w *= (T)(Nij - k);
-      part += w * (a[ti][c].x * b[tj][c].x + a[ti][c].y * b[tj][c].y);
+      part_sum += w * (a[ti][c].x * b[tj][c].x + a[ti][c].y * b[tj][c].y);
     }
-    acc += (double)part;
+    acc += (double)part_sum;
     __syncthreads();
+  }
+  if (gridDim.y > 1) {
+    // partial sums of this split; the tile's last CTA adds all of them in order
+    double* slot = part + (size_t)blockIdx.x * gridDim.y * 256;
+    slot[(size_t)blockIdx.y * 256 + threadIdx.x] = acc;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(done + blockIdx.x, 1) == (int)gridDim.y - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    acc = 0.0;
+    for (int y = 0; y < (int)gridDim.y; ++y) acc += __ldcg(slot + (size_t)y * 256 + threadIdx.x);
+    if (threadIdx.x == 0) done[blockIdx.x] = 0;
   }
   if (valid) {
     const double fp2 = 4.0 * kPi * kPi;
@@ -104,135 +125,365 @@ __global__ void __launch_bounds__(256) k_pairwise(const T2* __restrict__ F, int 
 // The Jacobi iteration (Golub and Van Loan, the cyclic Jacobi algorithm with
 // a parallel ordering): rotation (p, q) with tau = (a_qq - a_pp) / (2 a_pq),
 // t = sign(tau) / (|tau| + sqrt(1 + tau^2)), c = 1 / sqrt(1 + t^2), s = t c
-// zeroes a_pq in J^T A J, J = [[c, s], [-s, c]] on rows and columns p, q;
-// V accumulates V J. A is a float64 copy of Sigma, V the eigenvectors (both
-// in shared memory up to D = 112, else in global scratch); sig is replaced by
-// V max(Lambda, 0) V^T only when an eigenvalue is negative.
+// zeroes a_pq in J^T A J, J = [[c, s], [-s, c]] on rows and columns p, q.
+//
+// V accumulates V J; when an eigenvalue is negative Sigma becomes
+// V max(Lambda, 0) V^T.
+//
+// One CTA up to kPsdMaxD (kPsdMaxD64) assets. It is a serial chain of D - 1
+// steps a sweep, so a step is kept short, with one barrier:
+//  * a step's rotations, i = 0 .. nh-1 on players (u_i, v_i), split J^T A J into
+//    independent 2 x 2 blocks (i, j), of which the upper triangle i <= j is
+//    kept, by position: block e of a folded triangle at index e of four planes
+//    (uu, uv, vu, vv), so a thread reads its own blocks at fixed places without
+//    bank conflicts;
+//  * the players move on by one rotation a step (u_i to i-1, v_i to i+1, around
+//    the ends), so a block's four results go to four fixed places too, in the
+//    other of two copies of the matrix, at a constant distance for neighbouring
+//    threads;
+//  * meanwhile the first warps work out the next step's rotations, each from the
+//    three entries it needs of the matrix that the others are still writing.
+// Shared-memory accesses and issue slots bound float32, the float64 pipe float64.
+// The eigenvectors are not carried along: the rotations go to a log, and
+// k_psd_vectors applies it to the rows of V, which are independent, a warp each
+// over the whole GPU, when there is something to repair. Row and column passes
+// over A and V in one CTA, with three barriers and 4-way conflicts, took 3709 us
+// at D = 100 in float32 and 4328 us at D = 60 in float64; now 670 us and 1780 us
+// (of it the vectors and the product 90 us and 125 us).
 template <typename W>
-__global__ void __launch_bounds__(kJacobiThreads) k_psd_repair(double* __restrict__ sig, W* Ag, W* Vg, int D,
-                                                               int* clipped) {
-  // the working matrix and the eigenvectors in shared memory when both fit,
-  // else in the global scratch
+struct __align__(2 * sizeof(W)) CosSin {
+  W c, s;
+};
+struct PsdInfo {
+  int neg;    // negative eigenvalues
+  int steps;  // steps in the rotation log
+};
+
+// The rotation that zeroes a_pq. Any t gives a rotation when c = 1 / sqrt(1 + t^2)
+// is exact, and a t off by a few 2^-22 leaves as much of a_pq, which the next
+// sweep squares away: so t takes the approximate float32 operations. c does not:
+// its rounding drifts V from orthogonality over the steps (one Newton step in
+// place of the root and division raised the repaired matrix's float32 error 1.6
+// times). In float64 two Newton steps, as small corrections, from the
+// approximate reciprocal root reach rounding (relative error 2^-21, 2^-41).
+__device__ __forceinline__ float tangent(float num, float den) {
+  float tau = __fdividef(num, den);
+  if (!(fabsf(tau) >= 0.0f)) tau = 0.0f;  // both underflow
+  const float r = fmaf(tau, tau, 1.0f);
+  return copysignf(__fdividef(1.0f, fminf(fabsf(tau) + r * rsqrtf(r), 1.0e37f)), tau);
+}
+__device__ __forceinline__ CosSin<float> rotation(float app, float aqq, float apq) {
+  if (apq == 0.0f) return {1.0f, 0.0f};
+  const float t = tangent(aqq - app, 2.0f * apq);
+  const float x = fmaf(t, t, 1.0f);
+  const float c = 1.0f / sqrtf(x);
+  return {c, t * c};
+}
+__device__ __forceinline__ CosSin<double> rotation(double app, double aqq, double apq) {
+  if (apq == 0.0) return {1.0, 0.0};
+  const double t = (double)tangent((float)(aqq - app), (float)(2.0 * apq));
+  const double x = fma(t, t, 1.0);
+  double c = (double)rsqrtf((float)x);
+  c = fma(0.5 * c, fma(-(x * c), c, 1.0), c);
+  c = fma(0.5 * c, fma(-(x * c), c, 1.0), c);
+  return {c, t * c};
+}
+
+// The folded triangle of blocks i <= j < nh: rows of nh + 1, row r holding
+// i = r (nh - r blocks) and then i = nh - 1 - r.
+__host__ __device__ __forceinline__ int fold(int i, int j, int nh) {
+  return 2 * i <= nh - 1 ? i * (nh + 1) + (j - i) : (nh - 1 - i) * (nh + 1) + j + 1;
+}
+__host__ __device__ __forceinline__ int fold_size(int nh) { return (nh + 1) / 2 * (nh + 1); }
+// false for the empty half of the middle row of an odd nh
+__device__ __forceinline__ bool unfold(int e, int nh, int& i, int& j) {
+  const int r = e / (nh + 1), x = e - r * (nh + 1);
+  const bool first = x < nh - r;
+  i = first ? r : nh - 1 - r;
+  j = first ? r + x : x - 1;
+  return first || 2 * r < nh - 1;
+}
+// Rotation and role (0: u, 1: v) of player (role, i) at the next step.
+__device__ __forceinline__ void next_place(int nh, int& i, int& role) {
+  if (role == 0) {
+    if (i > 0) i -= 1;
+    else if (nh > 1) i = 1, role = 1;
+  } else if (i > 0) {
+    if (i < nh - 1) i += 1;
+    else role = 0;
+  }
+}
+// Index in the four planes (each of P entries) of the entry between players
+// (ra, i) and (rb, j).
+__device__ __forceinline__ int entry_at(int nh, int P, int i, int ra, int j, int rb) {
+  if (i > j || (i == j && ra > rb)) {
+    int t = i;
+    i = j;
+    j = t;
+    t = ra;
+    ra = rb;
+    rb = t;
+  }
+  return (2 * ra + rb) * P + fold(i, j, nh);
+}
+
+template <typename W>
+__global__ void __launch_bounds__(kJacobiThreads) k_psd_jacobi(const double* __restrict__ sig, int D,
+                                                               CosSin<W>* __restrict__ log, double* __restrict__ lam,
+                                                               PsdInfo* info, int* clipped) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const bool in_smem = (size_t)2 * D * D * sizeof(W) <= kPsdSmemBytes;
-  W* A = in_smem ? reinterpret_cast<W*>(smem_raw) : Ag;
-  W* V = in_smem ? reinterpret_cast<W*>(smem_raw) + (size_t)D * D : Vg;
-  __shared__ int sp[kPsdMaxD / 2], sq[kPsdMaxD / 2];
-  __shared__ W sc[kPsdMaxD / 2], ss[kPsdMaxD / 2];
-  __shared__ double s_lam[kPsdMaxD];
+  const int m = (D + 1) & ~1;  // players of the round-robin (one idle when D is odd)
+  const int nh = m / 2, P = fold_size(nh);
+  CosSin<W>* rot = reinterpret_cast<CosSin<W>*>(smem_raw);  // this step's, then the next one's
+  W* A = reinterpret_cast<W*>(rot + 2 * nh);                // two copies of four planes
   __shared__ double s_red[kJacobiThreads / 32];
   __shared__ int s_neg;
-  const int tid = threadIdx.x, nth = blockDim.x;
-  const int m = (D + 1) & ~1;  // players of the round-robin (one idle when D is odd)
-  const int nh = m / 2;
-  for (int e = tid; e < D * D; e += nth) {
-    A[e] = (W)sig[e];
-    const int r = e / D;
-    V[e] = (r == e - r * D) ? (W)1 : (W)0;
-  }
-  __syncthreads();
-  auto block_sum = [&](double v) -> double {
+  const int tid = threadIdx.x, nth = kJacobiThreads;
+  auto block_red = [&](double v, bool max) -> double {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int o = 16; o > 0; o >>= 1) {
+      const double u = __shfl_xor_sync(0xffffffffu, v, o);
+      v = max ? fmax(v, u) : v + u;
+    }
     if ((tid & 31) == 0) s_red[tid >> 5] = v;
     __syncthreads();
-    double t = 0.0;
-    for (int w = 0; w < (nth >> 5); ++w) t += s_red[w];
+    double t = s_red[0];
+    for (int w = 1; w < (nth >> 5); ++w) t = max ? fmax(t, s_red[w]) : t + s_red[w];
     __syncthreads();
     return t;
   };
+  // scale by a power of two (exact) to entries of at most 2
+  double big = 0.0;
+  for (int e = tid; e < D * D; e += nth) big = fmax(big, fabs(sig[e]));
+  big = block_red(big, true);
+  int ex = 0;
+  if (big > 0.0 && big < INFINITY) ex = ilogb(big);
+  const double down = ldexp(1.0, -ex), up = ldexp(1.0, ex);
+  // players of rotation i at step 0: u_i = i, v_i = m - 1 - i
   double nrm = 0.0;
-  for (int e = tid; e < D * D; e += nth) nrm += (double)A[e] * (double)A[e];
-  const double norm2 = block_sum(nrm);
+  for (int e = tid; e < 4 * P; e += nth) {
+    const int plane = e / P;
+    int i, j;
+    W a = 0;
+    if (unfold(e - plane * P, nh, i, j)) {
+      const int r = (plane & 2) ? m - 1 - i : i, c = (plane & 1) ? m - 1 - j : j;
+      if (r < D && c < D && !(i == j && plane == 2)) {
+        a = (W)(sig[(size_t)min(r, c) * D + max(r, c)] * down);
+        nrm += (r == c ? 1.0 : 2.0) * (double)a * (double)a;
+      }
+    }
+    A[e] = a;
+  }
+  const double norm2 = block_red(nrm, false);
   // converged when the off-diagonal norm reaches the level rounding leaves in
   // a D x D rotation sequence, 2 D eps of the norm (eps of the working type)
   const double eps = sizeof(W) == 8 ? 1.1102230246251565e-16 : 5.9604644775390625e-8;
   const double rel2 = (2.0 * D * eps) * (2.0 * D * eps);
-  for (int sweep = 0; sweep < kJacobiSweeps; ++sweep) {
-    double off = 0.0;
-    for (int e = tid; e < D * D; e += nth) {
-      const int r = e / D;
-      if (r != e - r * D) off += (double)A[e] * (double)A[e];
+
+  // the first warps own the rotations, thread i < nh rotation i, the others the
+  // blocks: kPsdRounds places of their blocks and of each block's four results
+  const int rot_threads = (nh + 31) & ~31, nwt = nth - rot_threads;
+  const int wt = tid - rot_threads;
+  int src[kPsdRounds], bi[kPsdRounds], bj[kPsdRounds], dst[kPsdRounds][4];
+  int n_uu = 0, n_vv = 0, n_uv = 0, r_uu = 0, r_vv = 0;  // a rotation thread's next entries: index, source
+  int i_uu = 0, i_vv = 0;
+#pragma unroll
+  for (int q = 0; q < kPsdRounds; ++q) src[q] = -1;
+  if (wt >= 0) {
+#pragma unroll
+    for (int q = 0; q < kPsdRounds; ++q) {
+      const int e = wt + q * nwt;
+      int i, j;
+      if (e < P && unfold(e, nh, i, j)) {
+        src[q] = e;
+        bi[q] = i;
+        bj[q] = j;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          int ni = i, nj = j, na = k >> 1, nb = k & 1;
+          next_place(nh, ni, na);
+          next_place(nh, nj, nb);
+          dst[q][k] = entry_at(nh, P, ni, na, nj, nb);
+        }
+      }
     }
-    if (!(block_sum(off) > rel2 * norm2)) break;  // uniform
-    for (int step = 0; step < m - 1; ++step) {
-      // round-robin: player m-1 meets player `step`; the others pair up
-      // symmetrically around it
+  } else if (tid < nh) {
+    // the players of rotation tid at the next step: where they are now
+    for (int i = 0; i < nh; ++i)
+      for (int role = 0; role < 2; ++role) {
+        int ni = i, nr = role;
+        next_place(nh, ni, nr);
+        if (ni == tid && nr == 0) i_uu = i, r_uu = role;
+        if (ni == tid && nr == 1) i_vv = i, r_vv = role;
+      }
+    n_uu = fold(i_uu, i_uu, nh);
+    n_vv = fold(i_vv, i_vv, nh);
+    n_uv = fold(min(i_uu, i_vv), max(i_uu, i_vv), nh);
+    const int e = fold(tid, tid, nh);
+    const CosSin<W> cs = rotation(A[e], A[3 * P + e], A[P + e]);
+    rot[tid] = cs;
+    log[tid] = cs;
+  }
+  __syncthreads();
+  // a result of a block under rotations R (rows) and S (columns)
+  auto entry = [](W auu, W auv, W avu, W avv, CosSin<W> R, int a, CosSin<W> S, int b) -> W {
+    const W x = a ? R.s : R.c, y = a ? R.c : -R.s;
+    const W u = x * auu + y * avu, v = x * auv + y * avv;
+    return (b ? S.s : S.c) * u + (b ? S.c : -S.s) * v;
+  };
+  int steps = 0;
+  for (int sweep = 0; sweep < kJacobiSweeps; ++sweep) {
+    W off = 0;
+    for (int e = tid; e < P; e += nth) {
+      const W* B = A + (steps & 1) * 4 * P + e;
+      int i, j;
+      if (unfold(e, nh, i, j)) off += B[P] * B[P] + (i == j ? (W)0 : B[0] * B[0] + B[2 * P] * B[2 * P] + B[3 * P] * B[3 * P]);
+    }
+    if (!(2.0 * block_red((double)off, false) > rel2 * norm2)) break;  // uniform
+    for (int step = 0; step < m - 1; ++step, ++steps) {
+      const W* __restrict__ B = A + (steps & 1) * 4 * P;
+      W* __restrict__ C = A + ((steps & 1) ^ 1) * 4 * P;
+      const CosSin<W>* cur = rot + (steps & 1) * nh;
       if (tid < nh) {
-        int p, q;
-        if (tid == 0) {
-          p = step;
-          q = m - 1;
-        } else {
-          p = (step + tid) % (m - 1);
-          q = (step - tid + (m - 1)) % (m - 1);
-        }
-        if (p > q) {
-          const int x = p;
-          p = q;
-          q = x;
-        }
-        W c = 1, sn = 0;
-        if (q < D) {
-          const W apq = A[(size_t)p * D + q];
-          if (apq != (W)0) {
-            const W tau = (A[(size_t)q * D + q] - A[(size_t)p * D + p]) / ((W)2 * apq);
-            const W t = (tau >= (W)0 ? (W)1 : (W)-1) / (fabs(tau) + sqrt((W)1 + tau * tau));
-            c = (W)1 / sqrt((W)1 + t * t);
-            sn = t * c;
+        const CosSin<W> R = cur[i_uu], S = cur[i_vv];
+        const W* b = B + n_uu;
+        const W aa = entry(b[0], b[P], b[P], b[3 * P], R, r_uu, R, r_uu);
+        b = B + n_vv;
+        const W bb = entry(b[0], b[P], b[P], b[3 * P], S, r_vv, S, r_vv);
+        b = B + n_uv;
+        W ab;
+        if (i_uu == i_vv) ab = entry(b[0], b[P], b[P], b[3 * P], R, 0, R, 1);
+        else if (i_uu < i_vv) ab = entry(b[0], b[P], b[2 * P], b[3 * P], R, r_uu, S, r_vv);
+        else ab = entry(b[0], b[P], b[2 * P], b[3 * P], S, r_vv, R, r_uu);
+        const CosSin<W> cs = rotation(aa, bb, ab);
+        rot[((steps & 1) ^ 1) * nh + tid] = cs;
+        log[(size_t)(steps + 1) * nh + tid] = cs;
+      } else {
+#pragma unroll
+        for (int q = 0; q < kPsdRounds; ++q) {
+          if (src[q] >= 0) {
+            const CosSin<W> R = cur[bi[q]], S = cur[bj[q]];
+            const W* b = B + src[q];
+            const bool diag = bi[q] == bj[q];
+            const W auu = b[0], auv = b[P], avu = diag ? auv : b[2 * P], avv = b[3 * P];
+            // rows: J_i^T, then columns: J_j (with c and s: a common factor c_i c_j
+            // after four multiply-adds with t rounds all four results alike, which
+            // doubled the error)
+            const W buu = R.c * auu - R.s * avu, buv = R.c * auv - R.s * avv;
+            const W bvu = R.s * auu + R.c * avu, bvv = R.s * auv + R.c * avv;
+            C[dst[q][0]] = S.c * buu - S.s * buv;
+            C[dst[q][1]] = S.s * buu + S.c * buv;
+            if (!diag) C[dst[q][2]] = S.c * bvu - S.s * bvv;  // a diagonal block's (v, u) is (u, v)
+            C[dst[q][3]] = S.s * bvu + S.c * bvv;
           }
         }
-        sp[tid] = p;
-        sq[tid] = q;
-        sc[tid] = c;
-        ss[tid] = sn;
-      }
-      __syncthreads();
-      // rows: A <- J^T A
-      for (int e = tid; e < nh * D; e += nth) {
-        const int r = e / D, x = e - r * D;
-        const int p = sp[r], q = sq[r];
-        if (q >= D) continue;
-        const W c = sc[r], sn = ss[r];
-        const W ap = A[(size_t)p * D + x], aq = A[(size_t)q * D + x];
-        A[(size_t)p * D + x] = c * ap - sn * aq;
-        A[(size_t)q * D + x] = sn * ap + c * aq;
-      }
-      __syncthreads();
-      // columns: A <- A J, V <- V J
-      for (int e = tid; e < nh * D; e += nth) {
-        const int r = e / D, x = e - r * D;
-        const int p = sp[r], q = sq[r];
-        if (q >= D) continue;
-        const W c = sc[r], sn = ss[r];
-        const W ap = A[(size_t)x * D + p], aq = A[(size_t)x * D + q];
-        A[(size_t)x * D + p] = c * ap - sn * aq;
-        A[(size_t)x * D + q] = sn * ap + c * aq;
-        const W vp = V[(size_t)x * D + p], vq = V[(size_t)x * D + q];
-        V[(size_t)x * D + p] = c * vp - sn * vq;
-        V[(size_t)x * D + q] = sn * vp + c * vq;
       }
       __syncthreads();
     }
   }
   if (tid == 0) s_neg = 0;
   __syncthreads();
-  for (int i = tid; i < D; i += nth) {
-    const double l = (double)A[(size_t)i * D + i];
-    s_lam[i] = l > 0.0 ? l : 0.0;
+  for (int d = tid; d < D; d += nth) {
+    // after whole sweeps the players are back where they started
+    const bool v = d >= nh;
+    const int i = v ? m - 1 - d : d;
+    const double l = (double)A[((steps & 1) * 4 + (v ? 3 : 0)) * P + fold(i, i, nh)] * up;
+    lam[d] = l;
     if (l < 0.0) atomicAdd(&s_neg, 1);
   }
   __syncthreads();
-  if (tid == 0 && clipped) *clipped = s_neg;
-  if (s_neg == 0) return;  // already positive semi-definite: Sigma unchanged
-  for (int e = tid; e < D * D; e += nth) {
-    const int i = e / D, j = e - i * D;
-    if (j < i) continue;
-    W v = 0;
-    for (int k = 0; k < D; ++k) v += V[(size_t)i * D + k] * (W)s_lam[k] * V[(size_t)j * D + k];
-    sig[(size_t)i * D + j] = v;
-    sig[(size_t)j * D + i] = v;
+  if (tid == 0) {
+    info->neg = s_neg;
+    info->steps = steps;
+    if (clipped) *clipped = s_neg;
   }
+}
+
+// Row x of V = J_1 J_2 ... J_n (block x): the unit row through the log's
+// rotations; the next kLogAhead steps' rotations are loaded while the current
+// ones are applied. Stored transposed (Vt[k][x] = V[x][k]) for k_psd_apply.
+constexpr int kLogAhead = 4;
+template <typename W, int NR>
+__global__ void __launch_bounds__(32) k_psd_vectors(const CosSin<W>* __restrict__ log,
+                                                    const PsdInfo* __restrict__ info, int D, W* __restrict__ Vt) {
+  __shared__ W u[kPsdMaxD + 2];
+  if (info->neg == 0) return;
+  const int lane = threadIdx.x;
+  const int m = (D + 1) & ~1, nh = m / 2;
+  for (int i = lane; i < m; i += 32) u[i] = i == (int)blockIdx.x ? (W)1 : (W)0;
+  __syncwarp();
+  const int steps = info->steps;
+  // players of this lane's rotations r = lane + 32 g at step 0
+  int a[NR], b[NR];
+#pragma unroll
+  for (int g = 0; g < NR; ++g) {
+    const int r = lane + 32 * g;
+    a[g] = r % (m - 1);
+    b[g] = r == 0 ? m - 1 : (2 * (m - 1) - r) % (m - 1);
+  }
+  CosSin<W> cur[kLogAhead][NR], nxt[kLogAhead][NR];
+  auto fetch = [&](CosSin<W> (&d)[kLogAhead][NR], int t0) {
+#pragma unroll
+    for (int h = 0; h < kLogAhead; ++h)
+#pragma unroll
+      for (int g = 0; g < NR; ++g) {
+        const int r = lane + 32 * g;
+        if (t0 + h < steps && r < nh) d[h][g] = log[(size_t)(t0 + h) * nh + r];
+      }
+  };
+  fetch(cur, 0);
+  for (int t0 = 0; t0 < steps; t0 += kLogAhead) {
+    fetch(nxt, t0 + kLogAhead);
+#pragma unroll
+    for (int h = 0; h < kLogAhead; ++h) {
+      if (t0 + h < steps) {
+        W up[NR], uq[NR];
+#pragma unroll
+        for (int g = 0; g < NR; ++g)
+          if (lane + 32 * g < nh) {
+            up[g] = u[a[g]];
+            uq[g] = u[b[g]];
+          }
+#pragma unroll
+        for (int g = 0; g < NR; ++g) {
+          const int r = lane + 32 * g;
+          if (r < nh) {
+            const W c = cur[h][g].c, s = cur[h][g].s;
+            u[a[g]] = c * up[g] - s * uq[g];
+            u[b[g]] = s * up[g] + c * uq[g];
+            a[g] = a[g] + 1 == m - 1 ? 0 : a[g] + 1;
+            if (r > 0) b[g] = b[g] + 1 == m - 1 ? 0 : b[g] + 1;
+          }
+        }
+        __syncwarp();
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < kLogAhead; ++h)
+#pragma unroll
+      for (int g = 0; g < NR; ++g) cur[h][g] = nxt[h][g];
+  }
+  for (int i = lane; i < D; i += 32) Vt[(size_t)i * D + blockIdx.x] = u[i];
+}
+
+// V max(Lambda, 0) V^T, one thread per entry of the upper triangle.
+template <typename W>
+__global__ void __launch_bounds__(256) k_psd_apply(double* __restrict__ sig, const W* __restrict__ Vt,
+                                                   const double* __restrict__ lam, const PsdInfo* __restrict__ info,
+                                                   int D) {
+  __shared__ W s_lam[kPsdMaxD];
+  if (info->neg == 0) return;  // already positive semi-definite: Sigma unchanged
+  for (int k = threadIdx.x; k < D; k += blockDim.x) s_lam[k] = lam[k] > 0.0 ? (W)lam[k] : (W)0;
+  __syncthreads();
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= D * D) return;
+  const int i = e / D, j = e - i * D;
+  if (j < i) return;
+  W v = 0;
+#pragma unroll 16
+  for (int k = 0; k < D; ++k) v += Vt[(size_t)k * D + i] * s_lam[k] * Vt[(size_t)k * D + j];
+  sig[(size_t)i * D + j] = v;
+  sig[(size_t)j * D + i] = v;
 }
 
 // The same cyclic Jacobi iteration over the whole GPU, for matrices larger
@@ -473,41 +724,71 @@ namespace mmgpu {
 
 int pairwise_psd_max_assets() { return kGridMaxD; }
 
+static int pairwise_splits(int D, int ld) {
+  const int nt = (D + kPT - 1) / kPT, tiles = nt * (nt + 1) / 2;
+  return std::max(1, std::min((kPairwiseCtas + tiles - 1) / tiles, (ld + kPChunk - 1) / kPChunk));
+}
+
+size_t pairwise_part_bytes(int D) {
+  const size_t nt = ((size_t)D + kPT - 1) / kPT, tiles = nt * (nt + 1) / 2;
+  return (tiles + kPairwiseCtas) * 256 * sizeof(double) + tiles * sizeof(int);
+}
+
 cudaError_t launch_pairwise(bool fp64, bool fejer, const void* coeffs, int ld, const int* Nv, int D,
-                            double* sig, cudaStream_t s) {
-  const int nt = (D + kPT - 1) / kPT;
-  const int grid = nt * (nt + 1) / 2;
+                            void* part, double* sig, cudaStream_t s) {
+  const int nt = (D + kPT - 1) / kPT, tiles = nt * (nt + 1) / 2;
+  const dim3 grid(tiles, pairwise_splits(D, ld));
+  // the tiles' arrival counters (zero between calls) after the partial sums
+  double* pt = reinterpret_cast<double*>(part);
+  int* done = reinterpret_cast<int*>(pt + ((size_t)tiles + kPairwiseCtas) * 256);
   if (fp64) {
-    if (fejer) k_pairwise<double2, double, true><<<grid, 256, 0, s>>>((const double2*)coeffs, ld, Nv, D, nt, sig);
-    else k_pairwise<double2, double, false><<<grid, 256, 0, s>>>((const double2*)coeffs, ld, Nv, D, nt, sig);
+    if (fejer) k_pairwise<double2, double, true><<<grid, 256, 0, s>>>((const double2*)coeffs, ld, Nv, D, nt, pt, done, sig);
+    else k_pairwise<double2, double, false><<<grid, 256, 0, s>>>((const double2*)coeffs, ld, Nv, D, nt, pt, done, sig);
   } else {
-    if (fejer) k_pairwise<float2, float, true><<<grid, 256, 0, s>>>((const float2*)coeffs, ld, Nv, D, nt, sig);
-    else k_pairwise<float2, float, false><<<grid, 256, 0, s>>>((const float2*)coeffs, ld, Nv, D, nt, sig);
+    if (fejer) k_pairwise<float2, float, true><<<grid, 256, 0, s>>>((const float2*)coeffs, ld, Nv, D, nt, pt, done, sig);
+    else k_pairwise<float2, float, false><<<grid, 256, 0, s>>>((const float2*)coeffs, ld, Nv, D, nt, pt, done, sig);
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_psd_repair(bool fp64, double* sig, double* A, double* V, int D, int* clipped, void* sync,
-                              int* status, cudaStream_t s) {
+static bool psd_one_cta(bool fp64, int D) { return D <= (fp64 ? kPsdMaxD64 : kPsdMaxD); }
+
+size_t psd_log_bytes(bool fp64, int D) {
+  if (D > kPsdMaxD) D = kPsdMaxD;  // larger matrices use the multi-CTA iteration, which keeps none
+  const size_t m = ((size_t)D + 1) & ~(size_t)1;
+  return ((size_t)kJacobiSweeps * (m - 1) + 1) * (m / 2) * 2 * (fp64 ? 8 : 4);
+}
+
+template <typename W>
+static cudaError_t launch_psd_one_cta(double* sig, double* A, W* V, int D, int* clipped, void* log, void* sync,
+                                      cudaStream_t s) {
+  const size_t m = ((size_t)D + 1) & ~(size_t)1;
+  const int nh = (int)(m / 2);
+  const size_t smem = 2 * (nh * sizeof(CosSin<W>) + 4 * (size_t)fold_size(nh) * sizeof(W));
+  static_assert(((kPsdMaxD / 2 + 1) / 2) * (kPsdMaxD / 2 + 1) <= kPsdRounds * (kJacobiThreads - (kPsdMaxD / 2 + 31) / 32 * 32),
+                "blocks per thread");
+  auto* lg = reinterpret_cast<CosSin<W>*>(log);
+  auto* info = reinterpret_cast<PsdInfo*>(sync);
+  cudaError_t e = cudaFuncSetAttribute(k_psd_jacobi<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_psd_jacobi<W><<<1, kJacobiThreads, smem, s>>>(sig, D, lg, A, info, clipped);
+  switch ((m / 2 + 31) / 32) {
+    case 1: k_psd_vectors<W, 1><<<D, 32, 0, s>>>(lg, info, D, V); break;
+    case 2: k_psd_vectors<W, 2><<<D, 32, 0, s>>>(lg, info, D, V); break;
+    default: k_psd_vectors<W, 3><<<D, 32, 0, s>>>(lg, info, D, V); break;
+  }
+  k_psd_apply<W><<<(D * D + 255) / 256, 256, 0, s>>>(sig, V, A, info, D);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_psd_repair(bool fp64, double* sig, double* A, double* V, int D, int* clipped, void* log,
+                              void* sync, int* status, cudaStream_t s) {
   if (D > kGridMaxD) return cudaErrorInvalidValue;
   const size_t wb = fp64 ? 8 : 4;
-  const size_t need = 2 * (size_t)D * D * wb;
-  if (need <= kPsdSmemBytes) {
-    // the working matrix and eigenvectors in one CTA's shared memory
-    auto one = [&](auto kern) -> cudaError_t {
-      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-      if (e != cudaSuccess) return e;
-      return cudaSuccess;
-    };
-    cudaError_t e;
-    if (fp64) {
-      if ((e = one(k_psd_repair<double>)) != cudaSuccess) return e;
-      k_psd_repair<double><<<1, kJacobiThreads, need, s>>>(sig, A, V, D, clipped);
-    } else {
-      if ((e = one(k_psd_repair<float>)) != cudaSuccess) return e;
-      k_psd_repair<float><<<1, kJacobiThreads, need, s>>>(sig, (float*)A, (float*)V, D, clipped);
-    }
-    return cudaGetLastError();
+  if (psd_one_cta(fp64, D)) {
+    // A holds the eigenvalues, V the eigenvectors (transposed)
+    if (fp64) return launch_psd_one_cta<double>(sig, A, V, D, clipped, log, sync, s);
+    return launch_psd_one_cta<float>(sig, A, (float*)V, D, clipped, log, sync, s);
   }
   // the whole GPU: one CTA per SM, every CTA resident (cooperative launch)
   cudaError_t e = cudaMemsetAsync(sync, 0, sizeof(GridSync), s);
