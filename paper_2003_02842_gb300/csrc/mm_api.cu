@@ -1491,6 +1491,10 @@ struct mm_batch_s {
   void* coef = nullptr;           // [reps * D][N + 1] complex64 of the last call
   int ld = 0;
   int* d_cut = nullptr;           // cutoffs of the captured sweep (device)
+  int* d_items = nullptr;         // and its work items
+  int nitems = 0;
+  void* d_part = nullptr;         // partial sums of a problem's CTAs
+  int* d_arrived = nullptr;
   std::vector<int> cut;
   cudaStream_t cap = nullptr;     // capture stream
   cudaStream_t last = nullptr;    // caller's stream of the last call
@@ -1513,6 +1517,12 @@ void batch_drop_graph(mm_batch b) {
   b->graph = nullptr;
 }
 
+void batch_free(mm_batch b) {
+  void* ptrs[] = {b->coef, b->d_cut, b->d_items, b->d_part, b->d_arrived};
+  for (void* q : ptrs)
+    if (q) cudaFree(q);
+}
+
 // Coefficients of every problem at the sweep's largest cutoff, then the
 // prefix-weighted sweep contraction, enqueued on st.
 mm_status batch_enqueue(mm_batch b, const int64_t* off, const double* t, const double* logp, int N, void* sigma,
@@ -1521,9 +1531,9 @@ mm_status batch_enqueue(mm_batch b, const int64_t* off, const double* t, const d
   mm_status r = coeffs_impl(p, off, t, logp, N, 0.0, 0.0, b->coef, nullptr, st);
   if (r != MM_OK) return r;
   StageScope sc(p, MM_STAGE_GRAM, st);
-  const int grid = std::max(1, std::min(p->G, 2 * kSMs));
-  MM_CUDA(launch_epps(b->desc.D, b->desc.basis == MM_BASIS_FEJER, p->fp64, b->coef, N + 1, b->d_cut,
-                      (int)b->cut.size(), p->G, sigma, R, p->status, grid, st));
+  EppsArgs a{b->coef, N + 1, b->d_cut, (int)b->cut.size(), b->d_items, b->nitems, p->G,
+             epps_splits(p->G, b->nitems), b->d_part, b->d_arrived, sigma, R, p->status};
+  MM_CUDA(launch_epps(b->desc.D, b->desc.basis == MM_BASIS_FEJER, p->fp64, a, st));
   return MM_OK;
 }
 
@@ -1560,10 +1570,15 @@ mm_status mm_batch_create(const mm_batch_desc* desc, mm_batch* out) {
     return r;
   }
   const size_t coef_bytes = (size_t)pd.D * ((size_t)d.N_max + 1) * (d.prec == MM_PREC_FP64 ? 16 : 8);
+  const size_t part_bytes = epps_part_bytes(d.D, d.prec == MM_PREC_FP64, d.reps);
   if (dalloc(b->p, &b->coef, coef_bytes) != MM_OK || dalloc(b->p, (void**)&b->d_cut, kMaxCutoffs * sizeof(int)) != MM_OK ||
+      dalloc(b->p, (void**)&b->d_items, epps_items_max(d.N_max) * sizeof(int)) != MM_OK ||
+      (part_bytes && (dalloc(b->p, &b->d_part, part_bytes) != MM_OK ||
+                      dalloc(b->p, (void**)&b->d_arrived, (size_t)d.reps * sizeof(int)) != MM_OK ||
+                      cudaMemset(b->d_arrived, 0, (size_t)d.reps * sizeof(int)) != cudaSuccess ||
+                      cudaDeviceSynchronize() != cudaSuccess)) ||
       cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess) {
-    if (b->coef) cudaFree(b->coef);
-    if (b->d_cut) cudaFree(b->d_cut);
+    batch_free(b);
     mm_destroy(b->p);
     delete b;
     cudaGetLastError();
@@ -1578,8 +1593,7 @@ mm_status mm_batch_destroy(mm_batch b) {
   if (check_plan(b->p) == MM_OK) cudaDeviceSynchronize();
   batch_drop_graph(b);
   if (b->cap) cudaStreamDestroy(b->cap);
-  if (b->coef) cudaFree(b->coef);
-  if (b->d_cut) cudaFree(b->d_cut);
+  batch_free(b);
   mm_destroy(b->p);
   delete b;
   return MM_OK;
@@ -1604,7 +1618,11 @@ mm_status mm_batch_epps(mm_batch b, const int64_t* d_offsets, const double* d_t,
   const bool new_cut = cut != b->cut;
   if (new_cut) {
     MM_CUDA(cudaStreamSynchronize(st));  // the previous sweep may still read the old cutoffs
+    const std::vector<int> items = epps_items(cut, p->G);
+    b->cut.clear();  // an interrupted upload is repeated by the next call
     MM_CUDA(cudaMemcpy(b->d_cut, cut.data(), cut.size() * sizeof(int), cudaMemcpyHostToDevice));
+    MM_CUDA(cudaMemcpy(b->d_items, items.data(), items.size() * sizeof(int), cudaMemcpyHostToDevice));
+    b->nitems = (int)items.size() / 2;
     b->cut = cut;
   }
   const void* key[5] = {d_offsets, d_t, d_logp, d_sigma_or_null, d_R};

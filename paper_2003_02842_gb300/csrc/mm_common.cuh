@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "../../include/mm.h"
 
 namespace mmgpu {
@@ -264,8 +266,28 @@ mm_status plan_create_no_staging(const mm_plan_desc* desc, mm_plan* out);  // no
 mm_status plan_set_active_assets(mm_plan p, int D);
 int* plan_status_word(mm_plan p);
 mm_status plan_flags_to_status(int flags);
-cudaError_t launch_epps(int Dg, bool fejer, bool fp64, const void* coef, int ld, const int* cut, int ncut, int G,
-                        void* sigma, void* R, int* status, int grid, cudaStream_t s);
+// The cutoff sweep of a batch (mm_epps.cu): G problems of Dg assets, splits
+// CTAs per problem (epps_splits) with their partial sums and zeroed arrival
+// counters, the work items of the cutoff list (epps_items).
+struct EppsArgs {
+  const void* coef;
+  int ld;
+  const int* cut;
+  int ncut;
+  const int* items;
+  int nitems;
+  int G, splits;
+  void* part;
+  int* arrived;
+  void* sigma;
+  void* R;
+  int* status;
+};
+int epps_splits(int G, int nitems);
+size_t epps_part_bytes(int Dg, bool fp64, int G);
+std::vector<int> epps_items(const std::vector<int>& cut, int G);
+size_t epps_items_max(int N_max);  // ints
+cudaError_t launch_epps(int Dg, bool fejer, bool fp64, const EppsArgs& a, cudaStream_t s);
 
 // Pairwise-cutoff covariance (float64 D x D into sig) and its repair to the
 // nearest positive semi-definite matrix (D <= pairwise_psd_max_assets(): one CTA while the
