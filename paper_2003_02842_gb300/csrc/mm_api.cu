@@ -203,6 +203,84 @@ double fit_kernel_poly(const SpreadParams& s, KernelPoly* out) {
   return worst;
 }
 
+// Even and odd polynomials of the FP64 path's float-pair spreading (PairPoly):
+// Chebyshev interpolation in y = z^2 on [0, 1/4] at kPairDeg + 1 nodes,
+// rewritten in powers of y. Returns the largest error of the taps over a sample
+// of d (float64 evaluation), or a large number when the stencil has too many.
+double fit_pair_poly(const SpreadParams& s, PairPoly* out) {
+  constexpr int n = kPairDeg + 1;
+  memset(out, 0, sizeof(*out));
+  const int last = std::max(s.khi, 1 - s.klo);  // pair k holds taps k and 1 - k
+  if (last > kPairMax) return 1e300;
+  out->npair = last;
+  out->one_sided = last > s.khi ? 1 : 0;
+  double node[n], T[n][n];
+  for (int m = 0; m < n; ++m) node[m] = cos(kPi * (m + 0.5) / n);
+  memset(T, 0, sizeof(T));
+  T[0][0] = 1.0;
+  T[1][1] = 1.0;
+  for (int i = 2; i < n; ++i)
+    for (int q = 0; q < n; ++q) T[i][q] = (q > 0 ? 2.0 * T[i - 1][q - 1] : 0.0) - T[i - 2][q];
+  double worst = 0.0;
+  for (int k = 1; k <= last; ++k) {
+    const double a = k - 0.5;
+    double v[2][n], mono[2][n];
+    for (int m = 0; m < n; ++m) {
+      const double z = sqrt((node[m] + 1.0) / 8.0);
+      const double p = kernel_at(s, a + z), q = kernel_at(s, a - z);
+      v[0][m] = 0.5 * (p + q);
+      v[1][m] = (p - q) / (2.0 * z);
+    }
+    for (int h = 0; h < 2; ++h) {
+      double in_t[n] = {};  // powers of t = 8 y - 1
+      for (int i = 0; i < n; ++i) {
+        double acc = 0.0;
+        for (int m = 0; m < n; ++m) acc += v[h][m] * cos(kPi * i * (m + 0.5) / n);
+        acc *= (i == 0 ? 1.0 : 2.0) / n;
+        for (int q = 0; q < n; ++q) in_t[q] += acc * T[i][q];
+      }
+      for (int q = 0; q < n; ++q) mono[h][q] = 0.0;
+      for (int i = n - 1; i >= 0; --i) {  // Horner in the polynomial 8 y - 1
+        for (int q = n - 1; q >= 1; --q) mono[h][q] = 8.0 * mono[h][q - 1] - mono[h][q];
+        mono[h][0] = -mono[h][0] + in_t[i];
+      }
+      float* c = out->c[k - 1][h];
+      for (int i = 0; i < n; ++i) {
+        const float hi = (float)mono[h][i];
+        if (i < kPairWide) {
+          c[i] = hi;
+          c[kPairWide + i] = (float)(mono[h][i] - (double)hi);
+        } else {
+          c[kPairWide + i] = hi;
+        }
+      }
+    }
+    for (int q = 0; q <= 32; ++q) {
+      const double z = q / 64.0, y = z * z;
+      double E = 0.0, O = 0.0;
+      for (int i = n - 1; i >= 0; --i) {
+        E = E * y + mono[0][i];
+        O = O * y + mono[1][i];
+      }
+      worst = std::max(worst, fabs(E + z * O - kernel_at(s, a + z)));
+      worst = std::max(worst, fabs(E - z * O - kernel_at(s, a - z)));
+    }
+  }
+  if (out->one_sided) {
+    // the ES kernel ends at M_sp: its tap -M_sp is zero but for a record exactly
+    // on a grid point (the kernel's edge value, counted in the error above)
+    const float(*c)[kPairCoefs] = out->c[last - 1];
+    bool zero = true;
+    for (int h = 0; h < 2; ++h)
+      for (int i = 0; i < kPairCoefs; ++i) zero = zero && c[h][i] == 0.0f;
+    if (zero) {
+      out->npair = last - 1;
+      out->one_sided = 0;
+    }
+  }
+  return worst;
+}
+
 // M_sp rules of Sec. 2.2.5 (sigma = 2).
 int msp_rule(mm_kernel k, double eps) {
   const double sigma = 2.0;
@@ -310,6 +388,8 @@ struct mm_plan_s {
   GramParams gram{};
   KernelPoly poly{};
   bool poly_ok = false;   // float32 spreading with polynomial taps and integer accumulation
+  PairPoly pair_poly{};
+  bool pair_ok = false;   // FP64 spreading in float pairs
   int tune_poly = -1;     // autotuner override: 0 off
   cudaStream_t last = nullptr;
   // replay of mm_estimate's launch sequence: one graph per accumulator in use
@@ -496,6 +576,11 @@ mm_status configure(mm_plan p, int N) {
     const double err = fit_kernel_poly(s, &p->poly);
     p->poly_ok = err <= std::max(3.0e-7, 0.1 * p->desc.tol);
   }
+  // FP64: taps in float pairs where their error (at most 1e-14) and the fit's
+  // are 50 times below the NUFFT tolerance; float64 throughout otherwise
+  p->pair_ok = false;
+  if (p->fp64 && s.algo == 0 && p->tune_poly != 0 && p->desc.tol >= 5.0e-13)
+    p->pair_ok = fit_pair_poly(s, &p->pair_poly) + 1.0e-14 <= 0.02 * p->desc.tol;
   // per-asset FFT: mixed path, the complex grid fits in shared memory and n
   // factors into at most kMaxAssetPasses compiled radices
   AssetFft af{};
@@ -718,8 +803,8 @@ mm_status coeffs_impl(mm_plan p, const int64_t* off, const double* t, const doub
     {
       StageScope sc(p, MM_STAGE_PREP, st);
       if (p->fp64)
-        MM_CUDA(launch_prep_f64(off, t, logp, p->bounds, gsc, p->gsize, D, p->Mr, p->desc.max_events, p->rec_b0,
-                                p->rec_d, p->rec_v, p->status, st));
+        MM_CUDA(launch_prep_f64(off, t, logp, p->bounds, gsc, p->gsize, D, p->Mr, p->desc.max_events, p->pair_ok,
+                                p->rec_b0, p->rec_d, p->rec_v, p->status, st));
       else
         MM_CUDA(launch_prep_f32(off, t, logp, p->bounds, gsc, p->gsize, D, p->Mr, p->desc.max_events, p->rec_b0,
                                 p->rec_d, p->rec_v, p->status, st));
@@ -734,7 +819,10 @@ mm_status coeffs_impl(mm_plan p, const int64_t* off, const double* t, const doub
     {
       StageScope sc(p, MM_STAGE_SPREAD, st);
       p->sp.order = use_order ? p->asset_order : nullptr;
-      if (p->fp64)
+      if (p->pair_ok)
+        MM_CUDA(launch_spread_pair(off, p->rec_b0, p->rec_d, p->rec_v, p->sp, p->pair_poly, (double*)p->grid,
+                                   p->status, st));
+      else if (p->fp64)
         MM_CUDA(launch_spread_f64(off, p->rec_b0, p->rec_d, p->rec_v, p->sp, (double*)p->grid, p->status, st));
       else if (p->poly_ok)
         MM_CUDA(launch_spread_poly(off, p->rec_b0, p->rec_d, p->rec_v, p->sp, p->poly, (float*)p->grid, p->status,

@@ -97,6 +97,21 @@ struct KernelPoly {
   float c[kPolyMaxTaps][kPolyDeg + 1];
 };
 
+// Averaging kernel of the FP64 path's float-pair spreading: taps k and 1 - k of a
+// record lie at phi(a - z) and phi(a + z), a = k - 1/2, z = d - 1/2, so one even
+// and one odd polynomial in y = z^2 serve both: phi(a -+ z) = E(y) -+ z O(y), each
+// of degree kPairDeg with its first kPairWide coefficients as float pairs (hi, then
+// lo) and the others as floats. one_sided: the last pair holds tap 1 - k alone.
+constexpr int kPairDeg = 6;
+constexpr int kPairWide = 5;
+constexpr int kPairCoefs = kPairDeg + 1 + kPairWide;
+constexpr int kPairMax = 16;
+struct PairPoly {
+  int npair;
+  int one_sided;
+  float c[kPairMax][2][kPairCoefs];
+};
+
 // Rescaling of Algorithm 4 in exact fixed point, written by k_bounds for the
 // current call: t_fix = trunc(t * 2^F) (int64, |t| < 2^(62-F)); the cell
 // coordinate u = (t - t0) M_r / span is u_fix = ((t_fix - t0_fix) * S) >> sh
@@ -184,9 +199,10 @@ cudaError_t launch_min_gap(const int64_t* off, const double* t, int D, const Res
 cudaError_t launch_prep_f32(const int64_t* off, const double* t, const double* logp, const Rescale* rs,
                             const GroupScale* gsc, int gsize, int D, int64_t Mr, int64_t max_events, int* rb0,
                             void* rd, void* rv, int* status, cudaStream_t s);
+// pair: the records' offsets d as float pairs z = d - 1/2 (launch_spread_pair)
 cudaError_t launch_prep_f64(const int64_t* off, const double* t, const double* logp, const Rescale* rs,
-                            const GroupScale* gsc, int gsize, int D, int64_t Mr, int64_t max_events, int* rb0,
-                            void* rd, void* rv, int* status, cudaStream_t s);
+                            const GroupScale* gsc, int gsize, int D, int64_t Mr, int64_t max_events, bool pair,
+                            int* rb0, void* rd, void* rv, int* status, cudaStream_t s);
 cudaError_t launch_spread_f32(const int64_t* off, const int* rb0, const void* rd, const void* rv,
                               const SpreadParams& p, float* grid, const int* status, cudaStream_t s);
 // float32 scatter with the polynomial taps and int32 fixed-point shared
@@ -195,6 +211,10 @@ cudaError_t launch_spread_f32(const int64_t* off, const int* rb0, const void* rd
 bool spread_poly_supported(int ntaps);
 cudaError_t launch_spread_poly(const int64_t* off, const int* rb0, const void* rd, const void* rv,
                                const SpreadParams& p, const KernelPoly& poly, float* grid, const int* status,
+                               cudaStream_t s);
+// FP64 scatter with the taps in float pairs and three-word integer accumulation
+cudaError_t launch_spread_pair(const int64_t* off, const int* rb0, const void* rd, const void* rv,
+                               const SpreadParams& p, const PairPoly& poly, double* grid, const int* status,
                                cudaStream_t s);
 cudaError_t launch_spread_f64(const int64_t* off, const int* rb0, const void* rd, const void* rv,
                               const SpreadParams& p, double* grid, const int* status, cudaStream_t s);

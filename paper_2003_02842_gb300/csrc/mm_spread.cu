@@ -287,7 +287,19 @@ template <> struct Rec4<double> {
   }
 };
 
-template <typename T>
+// z = d - 1/2 of a 40-bit offset as a float pair, exactly: 24 bits rounded into
+// hi, the rest in lo (|lo| <= 2^-24), built with 1.5 2^23 instead of conversions.
+__device__ __forceinline__ double offset_pair(unsigned long long frac) {
+  const long long s = (long long)frac - (1ll << 39);
+  const int hi = (int)((s + (1 << 16)) >> 17);
+  const int lo = (int)(s - ((long long)hi << 17));
+  const float zh = (__int_as_float(kRoundMagicBits + hi) - kRoundMagic) * 1.1920928955078125e-07f;      // 2^-23
+  const float zl = (__int_as_float(kRoundMagicBits + lo) - kRoundMagic) * 9.094947017729282e-13f;       // 2^-40
+  return __hiloint2double(__float_as_int(zh), __float_as_int(zl));
+}
+
+// PAIR (float64): the offset as the float pair of offset_pair in its 8 bytes.
+template <typename T, bool PAIR>
 __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(const int64_t* __restrict__ off, const double* __restrict__ t,
                                                        const double* __restrict__ logp,
                                                        const Rescale* __restrict__ rsp,
@@ -408,16 +420,21 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(const int64_t* __restr
     const long long dt = to_fix(tv[j], rs.F) - rs.t0_fix;
     int cb;
     T cd;
+    bool past;  // beyond the cell's start
     if (sizeof(T) == 8) {
       const unsigned long long uf = u_fix_of(tv[j], rs.t0_fix, rs.F, us);
       cb = (int)(uf >> kUFrac);
-      cd = frac_to<T>(uf & ((1ull << kUFrac) - 1));
+      const unsigned long long frac = uf & ((1ull << kUFrac) - 1);
+      if (PAIR) cd = (T)offset_pair(frac);
+      else cd = frac_to<T>(frac);
+      past = frac != 0ull;
     } else {
       float fd;
       cell_f32(dt, usf, cb, fd);
       cd = (T)fd;
+      past = fd > 0.0f;
     }
-    if (dt < 0 || cb > Mr || (cb == Mr && cd > (T)0)) {
+    if (dt < 0 || cb > Mr || (cb == Mr && past)) {
       flags |= ST_OUT_OF_WINDOW;
       continue;
     }
@@ -448,7 +465,7 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(const int64_t* __restr
   pdl_trigger();
 }
 
-template <typename T>
+template <typename T, bool PAIR>
 static cudaError_t launch_prep_t(const int64_t* off, const double* t, const double* logp, const Rescale* rs,
                                  const GroupScale* gsc, int gsize, int D, int64_t Mr, int64_t max_events, int* rb0,
                                  T* rd, T* rv, int* status, cudaStream_t s) {
@@ -456,7 +473,7 @@ static cudaError_t launch_prep_t(const int64_t* off, const double* t, const doub
   if ((((uintptr_t)rb0) | ((uintptr_t)rd) | ((uintptr_t)rv)) & 15) return cudaErrorMisalignedAddress;
   const int64_t per_block = (int64_t)kPrepThreads * kPrepE;
   const int64_t blocks = (max_events + per_block - 1) / per_block;
-  return launch_pdl(k_prep<T>, dim3((unsigned)blocks), dim3(kPrepThreads), 0, s, off, t, logp, rs, gsc, gsize,
+  return launch_pdl(k_prep<T, PAIR>, dim3((unsigned)blocks), dim3(kPrepThreads), 0, s, off, t, logp, rs, gsc, gsize,
                     status + 1, D, Mr, rb0, rd, rv, status);
 }
 
@@ -464,14 +481,17 @@ cudaError_t launch_prep_f32(const int64_t* off, const double* t, const double* l
                             const GroupScale* gsc, int gsize, int D,
                             int64_t Mr, int64_t max_events, int* rb0, void* rd, void* rv, int* status,
                             cudaStream_t s) {
-  return launch_prep_t<float>(off, t, logp, rs, gsc, gsize, D, Mr, max_events, rb0, (float*)rd, (float*)rv, status, s);
+  return launch_prep_t<float, false>(off, t, logp, rs, gsc, gsize, D, Mr, max_events, rb0, (float*)rd, (float*)rv,
+                                     status, s);
 }
 cudaError_t launch_prep_f64(const int64_t* off, const double* t, const double* logp, const Rescale* rs,
                             const GroupScale* gsc, int gsize, int D,
-                            int64_t Mr, int64_t max_events, int* rb0, void* rd, void* rv, int* status,
+                            int64_t Mr, int64_t max_events, bool pair, int* rb0, void* rd, void* rv, int* status,
                             cudaStream_t s) {
-  return launch_prep_t<double>(off, t, logp, rs, gsc, gsize, D, Mr, max_events, rb0, (double*)rd, (double*)rv, status,
-                               s);
+  auto go = [&](auto fn) {
+    return fn(off, t, logp, rs, gsc, gsize, D, Mr, max_events, rb0, (double*)rd, (double*)rv, status, s);
+  };
+  return pair ? go(launch_prep_t<double, true>) : go(launch_prep_t<double, false>);
 }
 
 // ------------------------------------------------------------------ spread
@@ -756,6 +776,214 @@ cudaError_t launch_spread_poly(const int64_t* off, const int* rb0, const void* r
   if (nt <= 24) return go(k_spread_poly<24>);
   if (nt <= 32) return go(k_spread_poly<32>);
   return cudaErrorInvalidValue;
+}
+
+// FP64 scatter in float pairs. The float64 pipe issues about two operations per
+// clock and SM, a sixty-fourth of the float32 rate, so a stencil point of some
+// sixty float64 operations (exponential and root, then a compare-and-swap loop
+// in shared memory) set this stage's time: 1095 us on the block workload (766,162 records,
+// 19 points each), 1250 us for 1024 small problems of three assets. Here a tap costs about
+// 100 float32 operations instead: the even and odd polynomials of PairPoly (two
+// taps each) by Horner's rule in float pairs h + l, the leading coefficients of
+// which need one float only; the product with the return; and an accumulation
+// that stays exact in three int32 words, as k_spread_poly's in two. Now 77 us and
+// 97 us.
+//
+// Error: against the kernel in 64 bits a tap is off by at most 7e-15 of the peak
+// (8e-16 rms; measured for the three kernels at tol 1e-12), so the path is taken
+// for tolerances from 5e-13 up, where the kernel's own truncation is at least 100
+// times that; tighter tolerances keep float64 throughout.
+//
+// Scales: V = max |v| < 2^exV over the tile's n records (from exponent fields:
+// returns of any float64 magnitude), eh = 21 - exV - max(0, bitlen(n) - 9), so
+// every |x| = |v phi 2^eh| < 2^21 and a cell's hi sum stays below 2^30. x = p + e
+// (p the rounded leading product, |e| < 0.6): hi = round(p); the residues of hi
+// and e, times 2^k, are rounded into mid (|mid| < 1.2 2^k + 2 a tap), their
+// residues times 2^k into lo (likewise). k = min(20, 30 - bitlen(m)) for the m
+// records of a staged chunk keeps a chunk's mid and lo sums below 2^31; between
+// chunks lo carries into mid and mid into hi. The quantum is 2^-(eh + 2k) (V 2^-60
+// for tiles of up to 511 records, V 2^-53 at 30,000), and no sum rounds.
+struct FloatPair {
+  float h, l;
+};
+// c + r y
+__device__ __forceinline__ FloatPair pair_step(FloatPair r, FloatPair y, float ch, float cl) {
+  const float p = __fmul_rn(r.h, y.h), e = __fmaf_rn(r.h, y.h, -p);
+  const float s = __fadd_rn(ch, p), b = __fsub_rn(s, ch);
+  const float t = __fadd_rn(__fsub_rn(ch, __fsub_rn(s, b)), __fsub_rn(p, b));
+  return {s, __fadd_rn(__fmaf_rn(r.l, y.h, __fmaf_rn(r.h, y.l, cl)), __fadd_rn(e, t))};
+}
+__device__ __forceinline__ FloatPair pair_poly(const float* __restrict__ c, FloatPair y) {
+  float top = c[2 * kPairWide + (kPairDeg - kPairWide)];
+#pragma unroll
+  for (int i = kPairDeg - 1; i >= kPairWide; --i) top = __fmaf_rn(top, y.h, c[kPairWide + i]);
+  FloatPair r{top, 0.0f};
+#pragma unroll
+  for (int i = kPairWide - 1; i >= 0; --i) r = pair_step(r, y, c[i], c[kPairWide + i]);
+  return r;
+}
+
+constexpr int kPairChunk = 1024;  // records staged per pass
+
+struct Words {
+  int hi, mid, lo;
+};
+// The three words of v w (v and w float pairs, |v w| < 2^21).
+__device__ __forceinline__ Words tap_words(FloatPair v, FloatPair w, float K) {
+  const float p = __fmul_rn(v.h, w.h);
+  const float e = __fmaf_rn(v.h, w.l, __fmaf_rn(v.l, w.h, __fmaf_rn(v.h, w.h, -p)));
+  const float th = __fadd_rn(p, kRoundMagic);
+  const float r = __fsub_rn(p, __fsub_rn(th, kRoundMagic));
+  const float tr = __fmaf_rn(r, K, kRoundMagic), te = __fmaf_rn(e, K, kRoundMagic);
+  const float r2 = __fmaf_rn(r, K, -__fsub_rn(tr, kRoundMagic)), e2 = __fmaf_rn(e, K, -__fsub_rn(te, kRoundMagic));
+  const float tl = __fmaf_rn(__fadd_rn(r2, e2), K, kRoundMagic);
+  return {__float_as_int(th) - kRoundMagicBits,
+          __float_as_int(tr) - kRoundMagicBits + (__float_as_int(te) - kRoundMagicBits),
+          __float_as_int(tl) - kRoundMagicBits};
+}
+
+__global__ void __launch_bounds__(kSpreadThreads, 4) k_spread_pair(const int64_t* __restrict__ off,
+                                                               const int* __restrict__ rb0,
+                                                               const double* __restrict__ rd,
+                                                               const double* __restrict__ rv,
+                                                               const int* __restrict__ gate, SpreadParams p,
+                                                               const __grid_constant__ PairPoly poly,
+                                                               double* __restrict__ grid) {
+  constexpr int EC = kPairChunk;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double* ev_d = reinterpret_cast<double*>(smem_raw);
+  double* ev_v = ev_d + EC;
+  int* ev_p = reinterpret_cast<int*>(ev_v + EC);
+  const int tpad = (p.tile + 3) & ~3;
+  int* tile = ev_p + EC;  // hi, mid and lo tiles
+  const uint32_t tile_s = (uint32_t)__cvta_generic_to_shared(tile);
+  __shared__ int s_max[kSpreadThreads / 32];
+  const int64_t L = (int64_t)blockIdx.x * p.tile;
+  const int Tlen = (int)min((int64_t)p.tile, p.Mr - L);
+  for (int c = threadIdx.x; c < 3 * tpad / 4; c += kSpreadThreads)
+    reinterpret_cast<int4*>(tile)[c] = make_int4(0, 0, 0, 0);
+  pdl_wait();         // the records come from the prep kernel
+  if (*gate) return;  // uniform: the whole block leaves
+  const int a = p.order ? p.order[blockIdx.y] : (int)blockIdx.y;
+  TileRanges tr;
+  tile_ranges(off, rb0, p, a, L, Tlen, tr);
+  const int64_t ntot = tr.n2 + tr.n1 + tr.n0;
+  // the largest exponent field of the tile's returns (staged with the first
+  // chunk when one chunk holds them all, else a pass over the returns)
+  int top = 0;
+  const int n_first = (int)min((int64_t)EC, ntot);
+  for (int i = threadIdx.x; i < n_first; i += kSpreadThreads) {
+    load_record<double>(rb0, rd, rv, p, tr, L, i, ev_p[i], ev_d[i], ev_v[i]);
+    top = max(top, (__double2hiint(ev_v[i]) >> 20) & 0x7FF);
+  }
+  for (int64_t i = EC + threadIdx.x; i < ntot; i += kSpreadThreads) {
+    int pp;
+    double dd, vv;
+    load_record<double>(rb0, rd, rv, p, tr, L, i, pp, dd, vv);
+    top = max(top, (__double2hiint(vv) >> 20) & 0x7FF);
+  }
+  top = __reduce_max_sync(0xffffffffu, top);
+  if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = top;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kSpreadThreads / 32; ++w) top = max(top, s_max[w]);
+  const int bitlen = 64 - __clzll((long long)ntot);
+  const int eh = 21 - (top - 1022) - max(0, bitlen - 9);
+  const int kk = min(20, 30 - (32 - __clz(n_first)));
+  const float K = __int_as_float((127 + kk) << 23);
+  const bool left = poly.one_sided != 0;
+  for (int64_t cs = 0; cs < ntot; cs += EC) {
+    const int n = (int)min((int64_t)EC, ntot - cs);
+    if (cs > 0) {
+      __syncthreads();
+      for (int c = threadIdx.x; c < Tlen; c += kSpreadThreads) {
+        const int lo = tile[c + 2 * tpad], mid = tile[c + tpad] + (lo >> kk);
+        tile[c + 2 * tpad] = lo & ((1 << kk) - 1);
+        tile[c + tpad] = mid & ((1 << kk) - 1);
+        tile[c] += mid >> kk;
+      }
+      for (int i = threadIdx.x; i < n; i += kSpreadThreads)
+        load_record<double>(rb0, rd, rv, p, tr, L, cs + i, ev_p[i], ev_d[i], ev_v[i]);
+    }
+    __syncthreads();
+    for (int e0 = threadIdx.x & ~31; e0 < n; e0 += kSpreadThreads) {
+      const int e = e0 + (threadIdx.x & 31);
+      const bool live = e < n && ev_p[e < n ? e : 0] != kNoCell;
+      const int pe = live ? ev_p[e] : kNoCell;
+      // a warp of records in one cell (dense tiles) adds its sum once
+      const bool same = __all_sync(0xffffffffu, pe == __shfl_sync(0xffffffffu, pe, 0));
+      if (same && pe == kNoCell) continue;  // uniform
+      FloatPair z{0.0f, 0.0f}, v{0.0f, 0.0f};
+      if (live) {
+        const double zz = ev_d[e];
+        z = {__int_as_float(__double2hiint(zz)), __int_as_float(__double2loint(zz))};
+        // v 2^eh from the exponent field; more than 2^1000 below V: zero
+        const long long b = __double_as_longlong(ev_v[e]);
+        const int ex = (int)((b >> 52) & 0x7FF);
+        if (ex > 0 && ex + eh > 0) split_f64(__longlong_as_double(b + ((long long)eh << 52)), v.h, v.l);
+      }
+      const float yh = __fmul_rn(z.h, z.h);
+      const FloatPair y{yh, __fmaf_rn(z.l, z.l, __fmaf_rn(__fadd_rn(z.h, z.h), z.l, __fmaf_rn(z.h, z.h, -yh)))};
+#pragma unroll 1
+      for (int q = 0; q < poly.npair; ++q) {
+        const FloatPair E = pair_poly(poly.c[q][0], y), O = pair_poly(poly.c[q][1], y);
+        const float m = __fmul_rn(z.h, O.h);
+        const float ml = __fmaf_rn(z.h, O.l, __fmaf_rn(z.l, O.h, __fmaf_rn(z.h, O.h, -m)));
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {  // tap 1 - k, then k = q + 1
+          if (side == 1 && left && q == poly.npair - 1) break;  // uniform
+          const float mh = side ? -m : m, mlo = side ? -ml : ml;
+          const float s = __fadd_rn(E.h, mh), bb = __fsub_rn(s, E.h);
+          const float t = __fadd_rn(__fsub_rn(E.h, __fsub_rn(s, bb)), __fsub_rn(mh, bb));
+          const FloatPair w{s, __fadd_rn(__fadd_rn(t, E.l), mlo)};
+          Words x = tap_words(v, w, K);
+          const unsigned c = (unsigned)(pe + (side ? q + 1 : -q));
+          bool take = live && c < (unsigned)Tlen;
+          if (same) {
+            x.hi = __reduce_add_sync(0xffffffffu, x.hi);
+            x.mid = __reduce_add_sync(0xffffffffu, x.mid);
+            x.lo = __reduce_add_sync(0xffffffffu, x.lo);
+            take = take && (threadIdx.x & 31) == 0;
+          }
+          if (take) {
+            red_shared_add(tile_s + 4u * c, x.hi);
+            red_shared_add(tile_s + 4u * (c + tpad), x.mid);
+            red_shared_add(tile_s + 4u * (c + 2 * tpad), x.lo);
+          }
+        }
+      }
+    }
+  }
+  __syncthreads();
+  // cells: (hi 2^k + mid) 2^-(eh + k) + lo 2^-(eh + 2k), each term built as a
+  // float64 with its integer in the low mantissa bits (no conversions)
+  double* g = grid + (int64_t)a * p.Mr + L;
+  const int xa = 0x433 - (eh + kk), xl = 0x433 - (eh + 2 * kk);
+  const bool plain = xl >= 1 && xa <= 0x7FE && top != 0x7FF;
+  const long long ba = ((long long)xa << 52) + (1ll << 51), bl = ((long long)xl << 52) + (1ll << 51);
+  for (int c = threadIdx.x; c < Tlen; c += kSpreadThreads) {
+    const long long A = ((long long)tile[c] << kk) + tile[c + tpad];
+    const int lo = tile[c + 2 * tpad];
+    if (plain) {
+      g[c] = (__longlong_as_double(ba + A) - __longlong_as_double(ba)) +
+             (__longlong_as_double(bl + lo) - __longlong_as_double(bl));
+    } else if (top == 0x7FF) {
+      g[c] = __longlong_as_double(0x7ff8000000000000ll);  // an infinite return
+    } else {
+      g[c] = ldexp((double)A + ldexp((double)lo, -kk), -(eh + kk));
+    }
+  }
+}
+
+cudaError_t launch_spread_pair(const int64_t* off, const int* rb0, const void* rd, const void* rv,
+                               const SpreadParams& p, const PairPoly& poly, double* grid, const int* status,
+                               cudaStream_t s) {
+  if (p.tile > spread_max_tile(true)) return cudaErrorInvalidValue;
+  const size_t smem = (size_t)kPairChunk * (2 * sizeof(double) + sizeof(int)) + 3 * (((size_t)p.tile + 3) / 4 * 16);
+  const cudaError_t e = cudaFuncSetAttribute(k_spread_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_spread_pair, dim3(p.ntiles, p.D), dim3(kSpreadThreads), smem, s, off, rb0, (const double*)rd,
+                    (const double*)rv, (const int*)(status + 1), p, poly, grid);
 }
 
 template <typename T, int K>
