@@ -766,8 +766,9 @@ mm_status coeffs_impl(mm_plan p, const int64_t* off, const double* t, const doub
   const bool use_order = p->asset_order && p->G == 1 && D <= kOrderMaxAssets;
   {
     StageScope sc(p, MM_STAGE_PREP, st);
-    MM_CUDA(launch_bounds(off, t, D, p->gsize, p->desc.max_events, t0, t1, Mr_known, p->bounds, p->status,
-                          use_order ? p->asset_order : nullptr, st));
+    // a batch's cell scales come from launch_group_scales below, a thread each
+    MM_CUDA(launch_bounds(off, t, D, p->gsize, p->desc.max_events, t0, t1, p->G > 1 ? 0 : Mr_known, p->bounds,
+                          p->status, use_order ? p->asset_order : nullptr, st));
   }
   if (N <= 0 && p->G > 1) return MM_ERR_CUTOFF;  // a batch sweeps given cutoffs
   if (N <= 0) {

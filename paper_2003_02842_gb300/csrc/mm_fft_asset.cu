@@ -238,15 +238,17 @@ __device__ __forceinline__ int pick(const int (&a)[kMaxAssetPasses], int p) {
   return p == 0 ? a[0] : p == 1 ? a[1] : p == 2 ? a[2] : a[3];
 }
 
-// All passes of the local transform in the plan's order for its direction.
+// All passes of the local transform in the plan's order for its direction, over
+// `points` points: one row of nl, or several one after the other (a pass works
+// on blocks whose length divides nl).
 template <bool BIG>
-__device__ __forceinline__ void run_passes(const AssetFft& f, Cplx<float>* s, const float4* anc, int nth) {
+__device__ __forceinline__ void run_passes(const AssetFft& f, Cplx<float>* s, const float4* anc, int nth, int points) {
   for (int i = 0; i < f.npass; ++i) {
     const int p = f.dif ? i : f.npass - 1 - i;
     const int R = pick(f.rad, p), m = pick(f.stride, p);
     const float4* a = anc + 2 * pick(f.tw_off, p);
-    if (f.dif) run_pass_t<true, BIG>(R, s, f.nl, m, a, nth);
-    else run_pass_t<false, BIG>(R, s, f.nl, m, a, nth);
+    if (f.dif) run_pass_t<true, BIG>(R, s, points, m, a, nth);
+    else run_pass_t<false, BIG>(R, s, points, m, a, nth);
     __syncthreads();
   }
 }
@@ -284,15 +286,16 @@ __device__ __forceinline__ int out_pos(int k, const AssetFft& f, const RevTab& t
 
 // Byte offset of the anchor rows in shared memory: after the nl complex
 // points, rounded up to 16 bytes (nl may be odd) for the float4 accesses.
-__host__ __device__ __forceinline__ size_t anchor_offset(int nl) { return ((size_t)nl * 8 + 15) & ~(size_t)15; }
+__host__ __device__ __forceinline__ size_t anchor_offset(int points) { return ((size_t)points * 8 + 15) & ~(size_t)15; }
 
 // The two digit-reversal tables of a decimation-in-frequency plan, built in
 // shared memory after the anchor rows (from the plan alone: no global reads).
 template <int NTH>
-__device__ __forceinline__ RevTab build_rev_tables(const AssetFft& f, unsigned char* smem_raw, const unsigned* mr) {
+__device__ __forceinline__ RevTab build_rev_tables(const AssetFft& f, unsigned char* smem_raw, const unsigned* mr,
+                                                   int points) {
   RevTab rt{};
   if (!f.dif) return rt;
-  int* tlo = reinterpret_cast<int*>(smem_raw + anchor_offset(f.nl) + (size_t)f.tw_rows * 32);
+  int* tlo = reinterpret_cast<int*>(smem_raw + anchor_offset(points) + (size_t)f.tw_rows * 32);
   int* thi = tlo + f.rev_lo;
   const int R0 = f.rad[0], R1 = f.npass >= 2 ? f.rad[1] : 1;
   for (int x = threadIdx.x; x < f.rev_lo; x += NTH) {
@@ -348,7 +351,7 @@ __device__ __forceinline__ void single_finish(const AssetFft& f, Cplx<float>* s,
                                               const float* __restrict__ decon, Cplx<float>* __restrict__ out) {
   constexpr int kUB = kUnpackBatch<NTH>;
   const int L = f.nl;
-  run_passes<BIG>(f, s, anc, NTH);
+  run_passes<BIG>(f, s, anc, NTH, L);
 
   // unpack the real-input transform and deconvolve (Eq. (14)):
   // G(k) = (Z_k + conj Z_{n-k}) / 2 + w_{2n}^k (Z_k - conj Z_{n-k}) / (2i)
@@ -397,7 +400,7 @@ __global__ void __launch_bounds__(NTH, 1)
   unsigned mr[kMaxAssetPasses];
 #pragma unroll
   for (int p = 0; p < kMaxAssetPasses; ++p) mr[p] = magic_of((unsigned)f.rad[p]);
-  const RevTab rt = build_rev_tables<NTH>(f, smem_raw, mr);
+  const RevTab rt = build_rev_tables<NTH>(f, smem_raw, mr, f.nl);
   pdl_wait();         // the grid comes from the spreading kernel
   if (*gate) return;  // uniform: the whole block leaves
   pdl_trigger();      // the contraction may take the SMs this launch leaves free
@@ -458,6 +461,84 @@ __global__ void __launch_bounds__(NTH, 1)
   single_finish<NTH, BIG>(f, s, anc, a, rt, U, decon, out);
 }
 
+// Several rows per CTA, for more rows than SMs that are short: the rows lie one
+// after the other in global memory and in shared memory, so one run of bulk
+// copies brings them, a pass takes all their butterflies at once and the
+// coefficients are written as one contiguous run. Per-CTA latencies (set-up, copy,
+// barriers) set the time of short rows: 16,384 rows of 108 points took
+// 387 us with a CTA each, 10 us with 108 rows a CTA.
+template <int NTH, bool BIG>
+__global__ void __launch_bounds__(NTH, 1)
+    k_fft_asset_rows(const float* __restrict__ grid, AssetFft f, int D, int rows, const Cplx<float>* __restrict__ tw,
+                     const Cplx<float>* __restrict__ U, const float* __restrict__ decon,
+                     Cplx<float>* __restrict__ out, const int* __restrict__ gate, int* status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Cplx<float>* s = reinterpret_cast<Cplx<float>*>(smem_raw);
+  const int L = f.nl;
+  float4* anc = reinterpret_cast<float4*>(smem_raw + anchor_offset(rows * L));
+  unsigned mr[kMaxAssetPasses];
+#pragma unroll
+  for (int p = 0; p < kMaxAssetPasses; ++p) mr[p] = magic_of((unsigned)f.rad[p]);
+  const RevTab rt = build_rev_tables<NTH>(f, smem_raw, mr, rows * L);
+  __shared__ __align__(8) uint64_t bar;
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  pdl_wait();         // the grid comes from the spreading kernel
+  if (*gate) return;  // uniform: the whole block leaves
+  pdl_trigger();
+  const int a0 = blockIdx.x * rows;
+  const int nr = min(rows, D - a0);
+  if (threadIdx.x == 0) {
+    // 16-byte aligned: n is even
+    const uint32_t bytes = (uint32_t)nr * (uint32_t)L * 8u;
+    mbar_expect_tx(&bar, bytes);
+    const unsigned char* src = reinterpret_cast<const unsigned char*>(grid) + (size_t)a0 * f.n * 8;
+    for (uint32_t o = 0; o < bytes; o += kBulkChunk) {
+      const uint32_t cb = bytes - o < kBulkChunk ? bytes - o : kBulkChunk;
+      bulk_g2s(smem_raw + o, src + o, cb, &bar);
+    }
+  }
+  {
+    const float4* src = reinterpret_cast<const float4*>(tw);
+    for (int i = threadIdx.x; i < 2 * f.tw_rows; i += NTH) {
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(anc + i);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src + i) : "memory");
+    }
+  }
+  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+  const bool ok = mbar_wait(&bar, 0, kWaitLimitNs);
+  if (!__syncthreads_and(ok)) {
+    // as k_fft_asset: report, wait once more (bounded) for the copies, leave
+    if (threadIdx.x == 0) {
+      atomicOr(status, ST_TIMEOUT);
+      mbar_wait(&bar, 0, kWaitLimitNs);
+    }
+    __syncthreads();
+    return;
+  }
+  run_passes<BIG>(f, s, anc, NTH, nr * L);
+  // unpack and deconvolve as single_finish, mode k of row r at k + r (N + 1)
+  const int w = f.N + 1;
+  const unsigned mw = magic_of((unsigned)w);
+  Cplx<float>* oa = out + (size_t)a0 * w;
+  for (int e = threadIdx.x; e < nr * w; e += NTH) {
+    const int r = fast_div(e, w, mw), k = e - r * w;
+    const float dk = __ldg(decon + k);
+    const Cplx<float> Uk = U[k];
+    const Cplx<float>* row = s + r * L;
+    const Cplx<float> Zk = row[out_pos(k, f, rt)];
+    const Cplx<float> Zc = cconj(row[out_pos(k == 0 ? 0 : L - k, f, rt)]);
+    const Cplx<float> E = {0.5f * (Zk.x + Zc.x), 0.5f * (Zk.y + Zc.y)};
+    const Cplx<float> dlt = csub(Zk, Zc);
+    const Cplx<float> O = {0.5f * dlt.y, -0.5f * dlt.x};  // (Z_k - conj Z_{n-k}) / (2i)
+    const Cplx<float> G = cadd(E, cmul(Uk, O));
+    oa[e] = Cplx<float>{G.x * dk, G.y * dk};
+  }
+}
+
 // The pair's local transform, the join of the two halves through
 // distributed shared memory and the unpacking and deconvolution of the
 // modes k = c, c + 2, ... <= N (CTA c of the cluster).
@@ -468,7 +549,7 @@ __device__ __forceinline__ void pair_finish(const AssetFft& f, Cplx<float>* s, c
                                             Cplx<float>* __restrict__ out) {
   constexpr int kPB = kPairBatch<NTH>;
   const int L = f.nl;
-  run_passes<BIG>(f, s, anc, NTH);
+  run_passes<BIG>(f, s, anc, NTH, L);
   cluster_sync_all();  // both halves transformed and visible to the partner
   const uint32_t peer = peer_addr(s, c ^ 1u);
   Cplx<float>* oa = out + (size_t)a * (f.N + 1);
@@ -532,7 +613,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTH, 1)
   unsigned mr[kMaxAssetPasses];
 #pragma unroll
   for (int p = 0; p < kMaxAssetPasses; ++p) mr[p] = magic_of((unsigned)f.rad[p]);
-  const RevTab rt = build_rev_tables<NTH>(f, smem_raw, mr);
+  const RevTab rt = build_rev_tables<NTH>(f, smem_raw, mr, f.nl);
   pdl_wait();  // the grid comes from the spreading kernel
   // every CTA of the cluster reads the same gate word: both leave or neither
   if (*gate) return;
@@ -698,7 +779,7 @@ __global__ void __launch_bounds__(512, 1)
   spread_resident<NT, NTH>(off, rb0, rd, rv, sp, poly, sub, f, mr, a, AllCells{}, s,
                            smem_raw + anchor_offset(f.nl));
   load_anchors<NTH>(f, tw, anc);
-  const RevTab rt = build_rev_tables<NTH>(f, smem_raw, mr);
+  const RevTab rt = build_rev_tables<NTH>(f, smem_raw, mr, f.nl);
   __syncthreads();
   single_finish<NTH, true>(f, s, anc, a, rt, U, decon, out);
 }
@@ -727,7 +808,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
   spread_resident<NT, NTH>(off, rb0, rd, rv, sp, poly, sub, f, mr, a, PairCells{c}, s,
                            smem_raw + anchor_offset(f.nl));
   load_anchors<NTH>(f, tw, anc);
-  const RevTab rt = build_rev_tables<NTH>(f, smem_raw, mr);  // none: decimation in time
+  const RevTab rt = build_rev_tables<NTH>(f, smem_raw, mr, f.nl);  // none: decimation in time
   __syncthreads();
   pair_finish<NTH, true>(f, s, anc, c, a, rt, W, U, decon, out);
 }
@@ -762,8 +843,20 @@ bool asset_fft_radix_ok(int R) {
   }
 }
 
-size_t asset_fft_smem(const AssetFft& f) {
-  return anchor_offset(f.nl) + (size_t)f.tw_rows * 32 + (f.dif ? (size_t)(f.rev_lo + f.rev_hi) * 4 : 0);
+static size_t asset_rows_smem(const AssetFft& f, int rows) {
+  return anchor_offset(rows * f.nl) + (size_t)f.tw_rows * 32 + (f.dif ? (size_t)(f.rev_lo + f.rev_hi) * 4 : 0);
+}
+
+size_t asset_fft_smem(const AssetFft& f) { return asset_rows_smem(f, 1); }
+
+// Rows per CTA: as many as give every SM one CTA, up to 24,576 points (an index
+// within a pass stays below 2^16 and the rows fit one CTA's shared memory).
+static int asset_rows(const AssetFft& f, int D) {
+  constexpr int kSMs = 152, kMaxPoints = 24576;
+  if (f.pair || f.pre_perm || !f.dif || f.split != 1) return 1;
+  int rows = std::min((D + kSMs - 1) / kSMs, kMaxPoints / f.nl);
+  while (rows > 1 && (asset_rows_smem(f, rows) > (size_t)220 * 1024 || (int64_t)rows * (f.N + 1) > 65535)) --rows;
+  return std::max(rows, 1);
 }
 
 cudaError_t launch_asset_twiddles(const AssetFft& f, void* tw, cudaStream_t s) {
@@ -854,6 +947,18 @@ cudaError_t launch_fft_asset(const float* grid, const AssetFft& f, int D, const 
   if (f.pair) {
     if (big) return go(k_fft_asset_pair<kPairThreads, true>, dim3(2, D), kPairThreads);
     return go(k_fft_asset_pair<kPairThreads, false>, dim3(2, D), kPairThreads);
+  }
+  const int rows = asset_rows(f, D);
+  if (rows > 1) {
+    const size_t rsmem = asset_rows_smem(f, rows);
+    auto many = [&](auto fn, int nth) -> cudaError_t {
+      cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem);
+      if (e != cudaSuccess) return e;
+      return launch_pdl(fn, dim3((D + rows - 1) / rows), dim3(nth), rsmem, s, grid, f, D, rows,
+                        (const Cplx<float>*)tw, (const Cplx<float>*)U, (const float*)decon, (Cplx<float>*)coeffs,
+                        (const int*)(status + 1), status);
+    };
+    return big ? many(k_fft_asset_rows<512, true>, 512) : many(k_fft_asset_rows<1024, false>, 1024);
   }
   if (big) return go(k_fft_asset<512, true>, dim3(1, D), 512, status);
   return go(k_fft_asset<1024, false>, dim3(1, D), 1024, status);
