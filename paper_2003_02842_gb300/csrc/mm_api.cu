@@ -18,7 +18,6 @@ using namespace mmgpu;
 namespace {
 
 constexpr int kSMs = 152;           // GB300: 2 dies x 76 SMs
-constexpr int kGlNodes = 128;       // Gauss-Legendre nodes for the ES transform
 constexpr int kMaxGramCtas = 2 * kSMs;
 constexpr int kMaxGramF64Splits = 256;
 constexpr int kGramTmaMinAssets = 192;  // default switch to the pre-split contraction
@@ -330,9 +329,7 @@ struct mm_plan_s {
   int atw_rad[kMaxAssetPasses] = {};
   void* U = nullptr;
   void* decon = nullptr;
-  double* esy = nullptr;          // ES transform: quadrature nodes and weights,
-  double* esf = nullptr;
-  double* es_cheb = nullptr;      // and its Chebyshev series (mixed precision)
+  double* es = nullptr;           // ES transform: quadrature nodes, weights and Chebyshev series
   Rescale* bounds = nullptr;       // one per problem
   void* gscale = nullptr;          // per-problem cell scales (batched form)
   int* status = nullptr;  // [0] sticky flags, [1] gate, [2] Nyquist N
@@ -435,7 +432,7 @@ mm_status dalloc(mm_plan p, void** ptr, size_t bytes) {
 }
 
 void free_all(mm_plan p) {
-  void* ptrs[] = {p->grid, p->rec_b0, p->rec_d, p->rec_v, p->W, p->atw, p->U, p->decon, p->esy, p->esf, p->es_cheb, p->bounds, p->gscale, p->status, p->gapbits, p->wsq,
+  void* ptrs[] = {p->grid, p->rec_b0, p->rec_d, p->rec_v, p->W, p->atw, p->U, p->decon, p->es, p->bounds, p->gscale, p->status, p->gapbits, p->wsq,
                   p->partial, p->acc[0], p->acc[1], p->gram_done, p->pw_N, p->pw_sig, p->pw_A,
                   p->pw_V, p->pw_clip, p->s_off, p->s_t, p->s_p, p->s_coef,
                   p->s_sigma, p->s_R, p->asset_order, p->tma_hi, p->tma_lo, p->pw_sync, p->pw_part, p->pw_log};
@@ -680,8 +677,8 @@ mm_status configure(mm_plan p, int N) {
 mm_status ensure_tables(mm_plan p, int N, cudaStream_t st) {
   if (p->tab_N == N) return MM_OK;
   StageScope sc(p, MM_STAGE_SETUP, st);
-  MM_CUDA(launch_setup_tables(p->desc.kernel, p->msp, p->Mr, N, p->fft.n, p->sp, p->tau, p->esy, p->esf, kGlNodes,
-                              p->es_cheb, p->W, p->U, p->decon, p->fp64, st));
+  MM_CUDA(launch_setup_tables(p->desc.kernel, p->msp, p->Mr, N, p->fft.n, p->sp, p->tau, p->es,
+                              p->es + kEsNodes, p->es + 2 * kEsNodes, p->W, p->U, p->decon, p->fp64, st));
   p->tab_N = N;
   return MM_OK;
 }
@@ -1086,9 +1083,7 @@ mm_status plan_create_impl(const mm_plan_desc* desc, int gsize, bool batch, mm_p
   }
   A(&p->U, Np1 * p->cs);
   A(&p->decon, Np1 * p->rs);
-  A((void**)&p->esy, kGlNodes * sizeof(double));
-  A((void**)&p->esf, kGlNodes * sizeof(double));
-  A((void**)&p->es_cheb, kEsChebMax * sizeof(double));
+  A((void**)&p->es, (2 * kEsNodes + kEsChebMax) * sizeof(double));
   A((void**)&p->bounds, (size_t)p->G * sizeof(Rescale));
   if (!batch && D <= (size_t)kOrderMaxAssets) A((void**)&p->asset_order, std::max<size_t>(D, 1) * sizeof(int));
   if (p->G > 1) A(&p->gscale, (size_t)p->G * group_scale_bytes());
@@ -1125,12 +1120,15 @@ mm_status plan_create_impl(const mm_plan_desc* desc, int gsize, bool batch, mm_p
     if (cudaMemset(p->status, 0, 4 * sizeof(int)) != cudaSuccess) r = MM_ERR_CUDA;
     if (p->gram_done && cudaMemset(p->gram_done, 0, sizeof(int)) != cudaSuccess) r = MM_ERR_CUDA;
   }
-  if (r == MM_OK) {
-    if (launch_es_nodes(kGlNodes, 2.3 * 2.0 * p->msp, p->esy, p->esf, 0) != cudaSuccess ||
-        launch_es_fit(kGlNodes, p->msp, p->esy, p->esf, p->es_cheb, 0) != cudaSuccess)
-      r = MM_ERR_CUDA;
-    p->launches += 2;
-    p->nl[MM_STAGE_SETUP] += 2;
+  if (r == MM_OK && d.kernel == MM_KERNEL_ES) {
+    double q[2 * kEsNodes];
+    es_quadrature(2.3 * 2.0 * p->msp, q, q + kEsNodes);
+    if (cudaMemcpy(p->es, q, sizeof(q), cudaMemcpyHostToDevice) != cudaSuccess) r = MM_ERR_CUDA;
+    if (r == MM_OK && !p->fp64) {
+      if (launch_es_fit(p->msp, p->es, p->es + kEsNodes, p->es + 2 * kEsNodes, 0) != cudaSuccess) r = MM_ERR_CUDA;
+      p->launches += 1;
+      p->nl[MM_STAGE_SETUP] += 1;
+    }
   }
   if (r == MM_OK && cudaDeviceSynchronize() != cudaSuccess) r = MM_ERR_CUDA;
   if (r != MM_OK) {

@@ -221,12 +221,13 @@ cudaError_t launch_spread_f64(const int64_t* off, const int* rb0, const void* rd
 
 // Quadrature nodes y and weights f of the ES transform, its Chebyshev series
 // (mixed precision) and the per-cutoff tables (mm_fft.cu).
+constexpr int kEsNodes = 128;
 constexpr int kEsChebMax = 64;
-cudaError_t launch_es_nodes(int nq, double beta, double* y, double* f, cudaStream_t s);
-cudaError_t launch_es_fit(int nq, int msp, const double* y, const double* f, double* cheb, cudaStream_t s);
+void es_quadrature(double beta, double* y, double* f);  // kEsNodes each, on the host
+cudaError_t launch_es_fit(int msp, const double* y, const double* f, double* cheb, cudaStream_t s);
 cudaError_t launch_setup_tables(int kernel, int msp, int64_t Mr, int N, int64_t n,
                                 const SpreadParams& sp, double tau, const double* esy,
-                                const double* esf, int nq, const double* cheb, void* W, void* U, void* decon,
+                                const double* esf, const double* cheb, void* W, void* U, void* decon,
                                 bool fp64, cudaStream_t s);
 cudaError_t launch_fft_cols_f32(float* grid, const FftParams& f, int D, const void* W, const int* status, cudaStream_t s);
 cudaError_t launch_fft_cols_f64(double* grid, const FftParams& f, int D, const void* W, const int* status, cudaStream_t s);

@@ -182,42 +182,38 @@ __global__ void __launch_bounds__(kFftThreads) k_fft_rows(const Cplx<T>* __restr
 // Quadrature of the ES kernel's transform (steps D.1-D.2 of Algorithm 10):
 //   phihat(k) = 2 alpha I(alpha k), I(theta) = int_0^1 e(y) cos(theta y) dy,
 //   e(y) = exp(beta (sqrt(1 - y^2) - 1)), alpha = 2 pi M_sp / M_r,
-// by nq-point Gauss-Legendre in y: nodes y_q and weights f_q = w_q e(y_q),
-// which depend on the plan's M_sp alone. Legendre roots by Newton's method on
-// P_nq (one thread per node).
-__global__ void k_es_nodes(int nq, double beta, double* y, double* f) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nq) return;
-  double zz = cos(kPi * (i + 0.75) / (nq + 0.5));
-  double dp = 1.0;
-  for (int it = 0; it < 100; ++it) {
-    double p0 = 1.0, p1 = zz;
-    for (int k = 2; k <= nq; ++k) {
-      const double p2 = ((2.0 * k - 1.0) * zz * p1 - (k - 1.0) * p0) / k;
-      p0 = p1;
-      p1 = p2;
+// by Gauss-Legendre in y: nodes y_q and weights f_q = w_q e(y_q), which depend on
+// the plan's M_sp alone. The Legendre roots, by Newton's method on P_nq, are found
+// on the host once per process (float64 recurrences, a long chain of divisions
+// for the GPU).
+void es_quadrature(double beta, double* y, double* f) {
+  struct Rule {
+    double y[kEsNodes], w[kEsNodes];
+    Rule() {
+      for (int i = 0; i < kEsNodes; ++i) {
+        double z = cos(kPi * (i + 0.75) / (kEsNodes + 0.5)), dp = 1.0;
+        for (int it = 0; it < 100; ++it) {
+          double p0 = 1.0, p1 = z;
+          for (int k = 2; k <= kEsNodes; ++k) {
+            const double p2 = ((2.0 * k - 1.0) * z * p1 - (k - 1.0) * p0) / k;
+            p0 = p1;
+            p1 = p2;
+          }
+          dp = kEsNodes * (z * p1 - p0) / (z * z - 1.0);
+          const double dz = p1 / dp;
+          z -= dz;
+          if (fabs(dz) < 1e-16) break;
+        }
+        y[i] = 0.5 * (z + 1.0);
+        w[i] = 1.0 / ((1.0 - z * z) * dp * dp);  // half of 2 / ((1 - z^2) P'^2): y in [0, 1]
+      }
     }
-    dp = nq * (zz * p1 - p0) / (zz * zz - 1.0);
-    const double dz = p1 / dp;
-    zz -= dz;
-    if (fabs(dz) < 1e-16) break;
+  };
+  static const Rule rule;
+  for (int i = 0; i < kEsNodes; ++i) {
+    y[i] = rule.y[i];
+    f[i] = rule.w[i] * exp(beta * (sqrt(fmax(1.0 - y[i] * y[i], 0.0)) - 1.0));
   }
-  double p0 = 1.0, p1 = zz;
-  for (int k = 2; k <= nq; ++k) {
-    const double p2 = ((2.0 * k - 1.0) * zz * p1 - (k - 1.0) * p0) / k;
-    p0 = p1;
-    p1 = p2;
-  }
-  dp = nq * (zz * p1 - p0) / (zz * zz - 1.0);
-  const double w = 2.0 / ((1.0 - zz * zz) * dp * dp);
-  const double yy = 0.5 * (zz + 1.0);
-  y[i] = yy;
-  f[i] = 0.5 * w * exp(beta * (sqrt(fmax(1.0 - yy * yy, 0.0)) - 1.0));
-}
-
-cudaError_t launch_es_nodes(int nq, double beta, double* y, double* f, cudaStream_t s) {
-  k_es_nodes<<<(nq + 31) / 32, 32, 0, s>>>(nq, beta, y, f);
-  return cudaGetLastError();
 }
 
 // Chebyshev coefficients of I(theta) in x = 2 (theta / theta_max)^2 - 1 (I is
@@ -228,14 +224,14 @@ cudaError_t launch_es_nodes(int nq, double beta, double* y, double* f, cudaStrea
 // M_sp = 1..30), far below float32 rounding. So a mixed-precision plan fits
 // once and its per-cutoff tables need some 25 float64 multiply-adds a mode
 // instead of 128 exponentials and cosines (k_setup_tables).
-__global__ void __launch_bounds__(1024) k_es_fit(int nq, const double* __restrict__ y, const double* __restrict__ f,
+__global__ void __launch_bounds__(1024) k_es_fit(const double* __restrict__ y, const double* __restrict__ f,
                                                  double theta_max, int nt, double* cheb) {
   __shared__ double val[kEsChebMax];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int m = warp; m < nt; m += 32) {
     const double theta = theta_max * sqrt(0.5 * (cospi((m + 0.5) / nt) + 1.0));
     double acc = 0.0;
-    for (int q = lane; q < nq; q += 32) acc = fma(f[q], cos(theta * y[q]), acc);
+    for (int q = lane; q < kEsNodes; q += 32) acc = fma(f[q], cos(theta * y[q]), acc);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) val[m] = acc;
@@ -252,10 +248,10 @@ __global__ void __launch_bounds__(1024) k_es_fit(int nq, const double* __restric
 
 int es_cheb_terms(int msp) { return 12 + (9 * msp + 9) / 10; }  // 18 at M_sp = 6, 39 at 30
 
-cudaError_t launch_es_fit(int nq, int msp, const double* y, const double* f, double* cheb, cudaStream_t s) {
+cudaError_t launch_es_fit(int msp, const double* y, const double* f, double* cheb, cudaStream_t s) {
   const int nt = es_cheb_terms(msp);
   if (nt > kEsChebMax) return cudaErrorInvalidValue;
-  k_es_fit<<<1, 1024, 0, s>>>(nq, y, f, 0.5 * kPi * msp, nt, cheb);
+  k_es_fit<<<1, 1024, 0, s>>>(y, f, 0.5 * kPi * msp, nt, cheb);
   return cudaGetLastError();
 }
 
@@ -269,7 +265,7 @@ cudaError_t launch_es_fit(int nq, int msp, const double* y, const double* f, dou
 // workload (eight requests in flight), now 9.4 us.
 template <typename T>
 __global__ void k_setup_tables(int kernel, int msp, int64_t Mr, int N, int64_t n, double kb_b, double kb_inv_phi0,
-                               double tau, const double* __restrict__ esy, const double* __restrict__ esf, int nq,
+                               double tau, const double* __restrict__ esy, const double* __restrict__ esf,
                                const double* __restrict__ cheb, int nt, Cplx<T>* W, Cplx<T>* U, T* decon) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) {
@@ -306,7 +302,7 @@ __global__ void k_setup_tables(int kernel, int msp, int64_t Mr, int N, int64_t n
         }
         acc = fma(0.5 * x2, b1, cheb[0] - b2);
       } else {
-        for (int q = 0; q < nq; ++q) acc = fma(esf[q], cos(alpha * k * esy[q]), acc);
+        for (int q = 0; q < kEsNodes; ++q) acc = fma(esf[q], cos(alpha * k * esy[q]), acc);
       }
       const double ph = 2.0 * alpha * acc;
       v = 1.0 / ((double)Mr * ph);
@@ -316,17 +312,17 @@ __global__ void k_setup_tables(int kernel, int msp, int64_t Mr, int N, int64_t n
 }
 
 cudaError_t launch_setup_tables(int kernel, int msp, int64_t Mr, int N, int64_t n, const SpreadParams& sp,
-                                double tau, const double* esy, const double* esf, int nq, const double* cheb,
+                                double tau, const double* esy, const double* esf, const double* cheb,
                                 void* W, void* U, void* decon, bool fp64, cudaStream_t s) {
   const int64_t m = n > (int64_t)N + 1 ? n : (int64_t)N + 1;
   const int nth = 128;
   const int blocks = (int)((m + nth - 1) / nth);
   const int nt = es_cheb_terms(msp);
   if (fp64)
-    k_setup_tables<double><<<blocks, nth, 0, s>>>(kernel, msp, Mr, N, n, sp.kb_b, sp.kb_inv_phi0, tau, esy, esf, nq,
+    k_setup_tables<double><<<blocks, nth, 0, s>>>(kernel, msp, Mr, N, n, sp.kb_b, sp.kb_inv_phi0, tau, esy, esf,
                                                   cheb, nt, (Cplx<double>*)W, (Cplx<double>*)U, (double*)decon);
   else
-    k_setup_tables<float><<<blocks, nth, 0, s>>>(kernel, msp, Mr, N, n, sp.kb_b, sp.kb_inv_phi0, tau, esy, esf, nq,
+    k_setup_tables<float><<<blocks, nth, 0, s>>>(kernel, msp, Mr, N, n, sp.kb_b, sp.kb_inv_phi0, tau, esy, esf,
                                                  cheb, nt, (Cplx<float>*)W, (Cplx<float>*)U, (float*)decon);
   return cudaGetLastError();
 }
