@@ -538,10 +538,14 @@ mm_status configure(mm_plan p, int N) {
   s.khi = p->khi;
   s.kernel = p->desc.kernel;
   s.max_events = p->desc.max_events;
+  s.asset_events = p->desc.max_events / p->desc.D;
   const int tmax = spread_max_tile(p->fp64);
   // default tile: the largest (measured on GB300 with the polynomial scatter:
-  // 4096 cells beat 2048 on both the block and the batched workloads)
-  int tile = p->desc.spread_tile > 0 ? std::min(p->desc.spread_tile, tmax) : tmax;
+  // 4096 cells beat 2048 on both the block and the batched workloads), or half
+  // of it where the assets' mean density says that tiles will be dense (a cell
+  // then takes two words, and one tile fills the shared memory of 4096 words)
+  const bool dense = !p->fp64 && 2.0 * (double)p->desc.max_events > (double)Mr * p->desc.D;
+  int tile = p->desc.spread_tile > 0 ? std::min(p->desc.spread_tile, tmax) : (dense ? tmax / 2 : tmax);
   if (p->tune_tile > 0) tile = std::min(p->tune_tile, tmax);
   if (Mr <= (int64_t)tile) {
     tile = (int)Mr;

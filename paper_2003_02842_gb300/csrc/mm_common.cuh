@@ -79,6 +79,7 @@ struct SpreadParams {
   double kb_b;       // KB: b = pi (2 - 1/sigma)
   double kb_inv_phi0;// KB: 1 / phi(0) (kernel normalised to peak 1)
   int64_t max_events;
+  int64_t asset_events;  // capacity per asset of the plan (max_events over its assets)
   // spreading tiles are dispatched asset by asset in this order (the assets
   // ranked by event count, heaviest first, written by k_bounds), or in index
   // order when null

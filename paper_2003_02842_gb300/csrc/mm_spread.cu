@@ -26,6 +26,9 @@
 // malformed input cannot write out of bounds.
 #include <math.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "mm_common.cuh"
 #include "mm_spread_dev.cuh"
 
@@ -643,80 +646,95 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread_scatter(const int64_t
 // round(y) for |y| < 2^22 is taken as y + 1.5 2^23, whose float spacing is 1
 // (one FMA, no conversion instruction; kRoundMagic).
 
-// Records staged per pass of the polynomial scatter: with two 4096-cell
-// tiles, 44 KB of shared memory per block and five blocks per SM. On the
-// block workload 512 to 1536 records and 2048- or 4096-cell tiles all ran
-// the stage within 2 us of one another: its time is the reductions.
-constexpr int kPolyChunk = 1024;
+// Threads of a polynomial-scatter block and records it stages at a time. A block is
+// a chain of dependent latencies (offsets, search, records, barriers), which other
+// blocks hide when there are many: 128 threads and eight blocks an SM from
+// kPolyBlocksMany tiles up (512 replications of ten assets: 463 us against 609 us
+// with 256 threads), 256 threads and six blocks down to kPolyBlocksSome (the block
+// workload's 1000 tiles: 17.6 us against 20.7 us with 128), else 512 threads. 512 also where the assets' capacity gives a tile more than
+// kPolyManyRecords (a busy day in the one tile of a low cutoff's grid): a thread
+// then sums runs of several records of a cell before it reduces.
+template <int NTH> struct PolyBlock;
+template <> struct PolyBlock<128> { static constexpr int chunk = 896, per_sm = 8; };
+template <> struct PolyBlock<256> { static constexpr int chunk = 1536, per_sm = 6; };
+template <> struct PolyBlock<512> { static constexpr int chunk = 4096, per_sm = 2; };
+constexpr int64_t kPolyBlocksMany = 8 * 152 * 2;
+constexpr int64_t kPolyBlocksSome = 2 * 152;
+constexpr int kPolyManyRecords = 4096;
 
-template <int NT>
-__global__ void __launch_bounds__(kSpreadThreads, 5) k_spread_poly(const int64_t* __restrict__ off,
-                                                               const int* __restrict__ rb0,
-                                                               const float* __restrict__ rd,
-                                                               const float* __restrict__ rv,
-                                                               const int* __restrict__ gate, SpreadParams p,
-                                                               KernelPoly poly, float* __restrict__ grid) {
-  constexpr int EC = kPolyChunk;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  int* ev_p = reinterpret_cast<int*>(smem_raw);
-  float* ev_d = reinterpret_cast<float*>(smem_raw + EC * sizeof(int));
-  float* ev_v = ev_d + EC;
-  const int tpad = (p.tile + 3) & ~3;  // tile cells rounded up to whole int4
-  int* tile_hi = reinterpret_cast<int*>(ev_v + EC);
-  int* tile_lo = tile_hi + tpad;
-  const uint32_t hi_s = (uint32_t)__cvta_generic_to_shared(tile_hi);
-  const uint32_t lo_s = (uint32_t)__cvta_generic_to_shared(tile_lo);
-  __shared__ float s_sum[kSpreadThreads / 32], s_max[kSpreadThreads / 32];
-  const int64_t L = (int64_t)blockIdx.x * p.tile;
-  const int Tlen = (int)min((int64_t)p.tile, p.Mr - L);
-  {
-    int4* t4 = reinterpret_cast<int4*>(tile_hi);
-    const int n4 = tpad / 2;  // both tiles
-    for (int c = threadIdx.x; c < n4; c += kSpreadThreads) t4[c] = make_int4(0, 0, 0, 0);
-  }
-  pdl_wait();         // the records come from the prep kernel
-  if (*gate) return;  // uniform: the whole block leaves
-  const int a = p.order ? p.order[blockIdx.y] : (int)blockIdx.y;
-  TileRanges tr;
-  tile_ranges(off, rb0, p, a, L, Tlen, tr);
-  const int64_t ntot = tr.n2 + tr.n1 + tr.n0;
-  // the tile's scales: sum and maximum of |v| over its records (staged with
-  // the first chunk when one chunk holds them all, else a pass over the returns)
-  float part = 0.f, pmax = 0.f;
-  const int n_first = (int)min((int64_t)EC, ntot);
-  for (int i = threadIdx.x; i < n_first; i += kSpreadThreads) {
-    load_record<float>(rb0, rd, rv, p, tr, L, i, ev_p[i], ev_d[i], ev_v[i]);
-    part += fabsf(ev_v[i]);
-    pmax = fmaxf(pmax, fabsf(ev_v[i]));
-  }
-  for (int64_t i = EC + threadIdx.x; i < ntot; i += kSpreadThreads) {
-    int pp;
-    float dd, vv;
-    load_record<float>(rb0, rd, rv, p, tr, L, i, pp, dd, vv);
-    part += fabsf(vv);
-    pmax = fmaxf(pmax, fabsf(vv));
-  }
-  const TileScales ts = tile_scales<kSpreadThreads>(part, pmax, ntot, s_sum, s_max);
-  const float inv_h = ts.inv_h, inv_l = ts.inv_l;
-  for (int64_t cs = 0; cs < ntot; cs += EC) {
-    const int n = (int)min((int64_t)EC, ntot - cs);
-    if (cs > 0) {
-      __syncthreads();
-      for (int i = threadIdx.x; i < n; i += kSpreadThreads)
-        load_record<float>(rb0, rd, rv, p, tr, L, cs + i, ev_p[i], ev_d[i], ev_v[i]);
+// Sparse tiles, one word per cell. When no stretch of 2 NP cells (a stencil)
+// holds more than kOneRun records, a cell's sum is at most the largest sum W of
+// |v| over kOneRun records in a row, not that of the tile: with x = v phi 2^e,
+// e = 30 - ex(W), every cell's sum of the rounded x stays below 2^30 (1 + 1e-6)
+// + kOneRun / 2 < 2^31 in one int32, with a quantum of at most W 2^-29. A run's W
+// is some 16 times the typical return at 20 records, so a tap is off by 2^-25 of
+// that at most and 2^-27 rms, as its float32 product's own rounding. That halves
+// the shared-memory reductions, which bound the taps, and the tile. With the shorter
+// taps below, the guessed search and the block sizes above the block workload's
+// spreading took 17.6 us (20.2 us with two words a cell in every tile), 500 stocks'
+// day 127 us (143 us), 512 replications of ten assets 463 us (715 us).
+constexpr int kOneRun = 20;
+
+// Taps k and 1 - k of a record are phi(a - z) and phi(a + z), a = k - 1/2,
+// z = d - 1/2: with tap k's polynomial E(z^2) + z O(z^2), tap 1 - k is
+// E - z O, nine multiply-adds for two taps instead of sixteen. The ES and
+// Kaiser-Bessel stencils have one tap more, -M_sp (zero for ES inside a cell).
+struct PairTaps {
+  float e[kPolyMaxTaps / 2][kPolyDeg / 2 + 1];
+  float o[kPolyMaxTaps / 2][kPolyDeg / 2];
+  float left[kPolyDeg + 1];
+  int npair;
+  int has_left;
+};
+
+template <int NP, int NTH>
+__device__ __forceinline__ void spread_one_word(const int* ev_p, const float* ev_d, const float* ev_v, int n, int Tlen,
+                                                const PairTaps& t, float scale, uint32_t tile_s) {
+  constexpr int H = kPolyDeg / 2;
+  for (int ei = threadIdx.x; ei < n; ei += NTH) {
+    const int pe = ev_p[ei];
+    if (pe == kNoCell) continue;
+    const float z = ev_d[ei] - 0.5f, y = z * z;
+    const float vs = ev_v[ei] * scale;
+    const bool inside = pe >= NP && pe + NP < Tlen;  // every tap, -M_sp included
+    const uint32_t at = tile_s + 4u * (uint32_t)pe;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+      if (q >= t.npair) break;  // uniform; NP taps pairs in the exact instantiations
+      float E = t.e[q][H], O = t.o[q][H - 1];
+#pragma unroll
+      for (int i = H - 1; i >= 0; --i) E = fmaf(E, y, t.e[q][i]);
+#pragma unroll
+      for (int i = H - 2; i >= 0; --i) O = fmaf(O, y, t.o[q][i]);
+      const int xk = __float2int_rn(vs * fmaf(z, O, E));
+      const int xm = __float2int_rn(vs * fmaf(-z, O, E));
+      if (inside) {
+        red_shared_add(at + 4 * (q + 1), xk);
+        red_shared_add(at - 4 * q, xm);
+      } else {
+        if ((unsigned)(pe + q + 1) < (unsigned)Tlen) red_shared_add(at + 4 * (q + 1), xk);
+        if ((unsigned)(pe - q) < (unsigned)Tlen) red_shared_add(at - 4 * q, xm);
+      }
     }
-    __syncthreads();
-    spread_chunk<NT, kSpreadThreads>(ev_p, ev_d, ev_v, n, Tlen, p.klo, poly, ts, hi_s, lo_s, AllCells{});
+    if (t.has_left && (unsigned)(pe - t.npair) < (unsigned)Tlen) {
+      float w = t.left[kPolyDeg];
+#pragma unroll
+      for (int i = kPolyDeg - 1; i >= 0; --i) w = fmaf(w, z, t.left[i]);
+      red_shared_add(at - 4 * t.npair, __float2int_rn(vs * w));
+    }
   }
-  __syncthreads();
+}
+
+// Cells [s0, s0 + len) of a tile to the grid, cell c's value from get(c).
+template <int NTH, class Get>
+__device__ __forceinline__ void write_cells(const SpreadParams& p, float* __restrict__ grid, int a, int64_t L, int s0,
+                                            int len, Get get) {
   if (p.perm_np > 0) {
     // the per-asset FFT's input order: complex point m = (L + c) / 2 goes to
     // its digit reversal (tiles and M_r are even, so cells pair up)
     float2* gz = reinterpret_cast<float2*>(grid + (int64_t)a * p.Mr);
-    const int2* h2 = reinterpret_cast<const int2*>(tile_hi);
-    const int2* l2 = reinterpret_cast<const int2*>(tile_lo);
-    const int m0 = (int)(L >> 1);
-    for (int c2 = threadIdx.x; c2 < (Tlen >> 1); c2 += kSpreadThreads) {
+    const int m0 = (int)((L + s0) >> 1);
+    for (int c2 = threadIdx.x; c2 < (len >> 1); c2 += NTH) {
       int m = m0 + c2, pos = 0;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -727,26 +745,134 @@ __global__ void __launch_bounds__(kSpreadThreads, 5) k_spread_poly(const int64_t
           m = h;
         }
       }
-      const int2 hv = h2[c2], lv = l2[c2];
-      gz[pos] = make_float2(fmaf((float)lv.x, inv_l, (float)hv.x * inv_h),
-                            fmaf((float)lv.y, inv_l, (float)hv.y * inv_h));
+      gz[pos] = make_float2(get(2 * c2), get(2 * c2 + 1));
     }
+    return;
+  }
+  float* g = grid + (int64_t)a * p.Mr + L + s0;
+  if (((reinterpret_cast<uintptr_t>(g) & 15) == 0) && (len & 3) == 0) {
+    float4* g4 = reinterpret_cast<float4*>(g);
+    for (int c = threadIdx.x; c < len / 4; c += NTH)
+      g4[c] = make_float4(get(4 * c), get(4 * c + 1), get(4 * c + 2), get(4 * c + 3));
+  } else {
+    for (int c = threadIdx.x; c < len; c += NTH) g[c] = get(c);
+  }
+}
+
+// One block per tile. `cells` int32 of shared memory: a sparse tile has one word
+// per cell, a dense one (by the records themselves) is taken in parts of cells / 2
+// with a hi and a lo word each.
+template <int NT, int NP, int NTH>
+__global__ void __launch_bounds__(NTH, PolyBlock<NTH>::per_sm) k_spread_poly(const int64_t* __restrict__ off,
+                                                               const int* __restrict__ rb0,
+                                                               const float* __restrict__ rd,
+                                                               const float* __restrict__ rv,
+                                                               const int* __restrict__ gate, SpreadParams p,
+                                                               const __grid_constant__ KernelPoly poly,
+                                                               const __grid_constant__ PairTaps taps, int cells,
+                                                               float* __restrict__ grid) {
+  constexpr int EC = PolyBlock<NTH>::chunk;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  int* ev_p = reinterpret_cast<int*>(smem_raw);
+  float* ev_d = reinterpret_cast<float*>(smem_raw + EC * sizeof(int));
+  float* ev_v = ev_d + EC;
+  int* tile = reinterpret_cast<int*>(ev_v + EC);
+  const uint32_t tile_s = (uint32_t)__cvta_generic_to_shared(tile);
+  __shared__ float s_sum[NTH / 32], s_max[NTH / 32], s_run[NTH / 32];
+  const int64_t L = (int64_t)blockIdx.x * p.tile;
+  const int Tlen = (int)min((int64_t)p.tile, p.Mr - L);
+  auto clear = [&] {
+    for (int c = threadIdx.x; c < cells / 4; c += NTH) reinterpret_cast<int4*>(tile)[c] = make_int4(0, 0, 0, 0);
+  };
+  clear();
+  pdl_wait();         // the records come from the prep kernel
+  if (*gate) return;  // uniform: the whole block leaves
+  const int a = p.order ? p.order[blockIdx.y] : (int)blockIdx.y;
+  TileRanges tr;
+  tile_ranges(off, rb0, p, a, L, Tlen, tr);
+  const int64_t ntot = tr.n2 + tr.n1 + tr.n0;
+  auto stage = [&](int64_t c0, int n) {
+    for (int i = threadIdx.x; i < n; i += NTH)
+      load_record<float>(rb0, rd, rv, p, tr, L, c0 + i, ev_p[i], ev_d[i], ev_v[i]);
+  };
+  // at most kOneRun records in any stencil's width, and their sums of |v|;
+  // chunks overlap by a run, and the last one stays staged
+  bool sparse = Tlen <= cells;
+  float run = 0.f;
+  int64_t cs = 0;
+  int n = 0;
+  while (true) {
+    n = (int)min((int64_t)EC, ntot - cs);
+    stage(cs, n);
+    __syncthreads();
+    const bool last = cs + n == ntot;
+    const int lim = last ? n : n - kOneRun;
+    for (int i = threadIdx.x; i < lim; i += NTH) {
+      if (i + kOneRun < n) sparse = sparse && ev_p[i + kOneRun] - ev_p[i] > 2 * NP;
+      float w = 0.f;
+#pragma unroll
+      for (int j = 0; j < kOneRun; ++j) w += i + j < n ? fabsf(ev_v[i + j]) : 0.f;
+      run = fmaxf(run, w);
+    }
+    if (last) break;
+    cs += EC - kOneRun;
+    if (!__syncthreads_and(sparse)) {  // dense already: the rest does not matter
+      sparse = false;
+      break;
+    }
+  }
+  run = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(run)));  // not negative
+  if ((threadIdx.x & 31) == 0) s_run[threadIdx.x >> 5] = run;
+  sparse = __syncthreads_and(sparse);
+#pragma unroll
+  for (int w = 0; w < NTH / 32; ++w) run = fmaxf(run, s_run[w]);
+  // 2^e and 2^-e have to be normal floats
+  if (sparse && run < 1.0e30f && (run > 1.0e-27f || run == 0.f)) {
+    int ex = 0;
+    if (run > 0.f) frexpf(run, &ex);  // run < 2^ex
+    const int e = 30 - ex;
+    const float scale = __int_as_float((127 + e) << 23), inv = __int_as_float((127 - e) << 23);
+    spread_one_word<NP, NTH>(ev_p, ev_d, ev_v, n, Tlen, taps, scale, tile_s);
+    for (int64_t c0 = 0; c0 < cs; c0 += EC) {  // the records before the staged chunk
+      __syncthreads();
+      const int m = (int)min((int64_t)EC, cs - c0);
+      stage(c0, m);
+      __syncthreads();
+      spread_one_word<NP, NTH>(ev_p, ev_d, ev_v, m, Tlen, taps, scale, tile_s);
+    }
+    __syncthreads();
+    write_cells<NTH>(p, grid, a, L, 0, Tlen, [&](int c) { return (float)tile[c] * inv; });
     pdl_trigger();
     return;
   }
-  float* g = grid + (int64_t)a * p.Mr + L;
-  if (((reinterpret_cast<uintptr_t>(g) & 15) == 0) && (Tlen & 3) == 0) {
-    const int4* h4 = reinterpret_cast<const int4*>(tile_hi);
-    const int4* l4 = reinterpret_cast<const int4*>(tile_lo);
-    float4* g4 = reinterpret_cast<float4*>(g);
-    for (int c = threadIdx.x; c < Tlen / 4; c += kSpreadThreads) {
-      const int4 hq = h4[c], lq = l4[c];
-      g4[c] = make_float4(fmaf((float)lq.x, inv_l, (float)hq.x * inv_h), fmaf((float)lq.y, inv_l, (float)hq.y * inv_h),
-                          fmaf((float)lq.z, inv_l, (float)hq.z * inv_h), fmaf((float)lq.w, inv_l, (float)hq.w * inv_h));
+  // the tile's scales: sum and maximum of |v| over its records
+  float part = 0.f, pmax = 0.f;
+  for (int64_t i = threadIdx.x; i < ntot; i += NTH) {
+    int pp;
+    float dd, vv;
+    load_record<float>(rb0, rd, rv, p, tr, L, i, pp, dd, vv);
+    part += fabsf(vv);
+    pmax = fmaxf(pmax, fabsf(vv));
+  }
+  const TileScales ts = tile_scales<NTH>(part, pmax, ntot, s_sum, s_max);
+  const float inv_h = ts.inv_h, inv_l = ts.inv_l;
+  const int half = cells / 2 & ~3;
+  for (int s0 = 0; s0 < Tlen; s0 += half) {
+    const int len = min(half, Tlen - s0);
+    if (s0 > 0) {
+      __syncthreads();
+      clear();
     }
-  } else {
-    for (int c = threadIdx.x; c < Tlen; c += kSpreadThreads)
-      g[c] = fmaf((float)tile_lo[c], inv_l, (float)tile_hi[c] * inv_h);
+    for (int64_t c0 = 0; c0 < ntot; c0 += EC) {
+      const int m = (int)min((int64_t)EC, ntot - c0);
+      __syncthreads();
+      stage(c0, m);
+      __syncthreads();
+      spread_chunk<NT, NTH>(ev_p, ev_d, ev_v, m, len, p.klo - s0, poly, ts, tile_s, tile_s + 4u * half, AllCells{});
+    }
+    __syncthreads();
+    write_cells<NTH>(p, grid, a, L, s0, len,
+                     [&](int c) { return fmaf((float)tile[half + c], inv_l, (float)tile[c] * inv_h); });
   }
   pdl_trigger();
 }
@@ -760,27 +886,46 @@ cudaError_t launch_spread_poly(const int64_t* off, const int* rb0, const void* r
                                cudaStream_t s) {
   if (p.tile > spread_max_tile(false)) return cudaErrorInvalidValue;
   const int nt = p.khi - p.klo + 1;
-  // staged records, then the hi and lo tiles (each rounded up to whole int4)
-  const size_t smem = (size_t)kPolyChunk * (sizeof(int) + 2 * sizeof(float)) + 2 * (((size_t)p.tile + 3) / 4 * 16);
+  PairTaps taps{};
+  taps.npair = p.khi;  // tap k = 1 .. M_sp pairs with 1 - k
+  for (int k = 1; k <= p.khi; ++k) {
+    const float* c = poly.c[k - p.klo];
+    for (int i = 0; i <= kPolyDeg / 2; ++i) taps.e[k - 1][i] = c[2 * i];
+    for (int i = 0; i < kPolyDeg / 2; ++i) taps.o[k - 1][i] = c[2 * i + 1];
+  }
+  if (p.klo == -p.khi) {
+    for (int i = 0; i <= kPolyDeg; ++i) {
+      taps.left[i] = poly.c[0][i];
+      if (poly.c[0][i] != 0.0f) taps.has_left = 1;
+    }
+  }
+  // staged records, then the tile: a word per cell, two while 4096 words hold
+  // them (a small grid's only tile may be dense)
+  const int tpad = (p.tile + 3) & ~3;
+  const int cells = std::max({tpad, std::min(2 * tpad, 4096), 8});
   dim3 grd(p.ntiles, p.D);
-  auto go = [&](auto fn) -> cudaError_t {
+  auto go = [&](auto fn, int nth, int chunk) -> cudaError_t {
+    const size_t smem = (size_t)chunk * (sizeof(int) + 2 * sizeof(float)) + (size_t)cells * sizeof(int);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(fn, grd, dim3(kSpreadThreads), smem, s, off, rb0, (const float*)rd, (const float*)rv,
-                      (const int*)(status + 1), p, poly, grid);
+    return launch_pdl(fn, grd, dim3(nth), smem, s, off, rb0, (const float*)rd, (const float*)rv,
+                      (const int*)(status + 1), p, poly, taps, cells, grid);
   };
-  switch (nt) {
-    case 9: return go(k_spread_poly<9>);
-    case 13: return go(k_spread_poly<13>);
-    case 14: return go(k_spread_poly<14>);
-    default: break;
-  }
-  // other tap counts: the next instantiation up, padded with zero taps
-  if (nt <= 8) return go(k_spread_poly<8>);
-  if (nt <= 16) return go(k_spread_poly<16>);
-  if (nt <= 24) return go(k_spread_poly<24>);
-  if (nt <= 32) return go(k_spread_poly<32>);
-  return cudaErrorInvalidValue;
+  // tap counts without an instantiation: the next one up, padded with zero taps
+  auto pick = [&](auto w) -> cudaError_t {
+    constexpr int NTH = decltype(w)::value, EC = PolyBlock<NTH>::chunk;
+    if (nt <= 9) return go(k_spread_poly<9, 4, NTH>, NTH, EC);
+    if (nt <= 13) return go(k_spread_poly<13, 6, NTH>, NTH, EC);
+    if (nt <= 14) return go(k_spread_poly<14, 7, NTH>, NTH, EC);
+    if (nt <= 16) return go(k_spread_poly<16, 8, NTH>, NTH, EC);
+    if (nt <= 32) return go(k_spread_poly<32, 16, NTH>, NTH, EC);
+    return cudaErrorInvalidValue;
+  };
+  const int64_t blocks = (int64_t)p.ntiles * p.D;
+  if (p.asset_events > (int64_t)kPolyManyRecords * p.ntiles || blocks < kPolyBlocksSome)
+    return pick(std::integral_constant<int, 512>{});
+  if (blocks < kPolyBlocksMany) return pick(std::integral_constant<int, 256>{});
+  return pick(std::integral_constant<int, 128>{});
 }
 
 // FP64 scatter in float pairs. The float64 pipe issues about two operations per

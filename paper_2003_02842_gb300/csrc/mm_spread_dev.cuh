@@ -240,9 +240,24 @@ struct TileRanges {
 // First index h in [e0, e1) with key[h] >= x (e1 if none), by one warp: each
 // step the 32 lanes sample the bracket at 32 evenly spaced points and a
 // ballot keeps the segment where the predicate turns true (32-ary search).
-__device__ __forceinline__ int64_t warp_first_ge(const int* __restrict__ key, int64_t e0, int64_t e1, long long x) {
+// A first step around `guess` (>= 0) with a stride of about the square root of the
+// length narrows the bracket to that stride when the keys are nearly uniform:
+// two dependent loads instead of three for 1,024 to 32,768 records.
+__device__ __forceinline__ int64_t warp_first_ge(const int* __restrict__ key, int64_t e0, int64_t e1, long long x,
+                                                 int64_t guess = -1) {
   const int lane = threadIdx.x & 31;
   int64_t lo = e0, hi = e1;  // answer in [lo, hi]
+  if (guess >= 0 && e1 - e0 > 1024) {
+    const int64_t stride = max((int64_t)8, (int64_t)sqrtf((float)(e1 - e0)) / 4);
+    const int64_t g = e0 + guess - 16 * stride + lane * stride;
+    const bool in = g >= e0 && g < e1;
+    const bool below = in ? (long long)key[in ? g : e0] < x : g < e0;
+    const int c = __popc(__ballot_sync(0xffffffffu, below));
+    const int64_t first = e0 + guess - 16 * stride;
+    if (c > 0) lo = max(e0, first + (c - 1) * stride + 1);
+    if (c < 32) hi = min(e1, first + c * stride);
+    lo = min(lo, hi);
+  }
   for (int it = 0; it < 16 && hi > lo; ++it) {
     const int64_t len = hi - lo;
     const int64_t stride = (len + 31) / 32;
@@ -267,18 +282,26 @@ __device__ __forceinline__ void tile_ranges(const int64_t* __restrict__ off, con
   __shared__ int64_t s_res[6];
   const int64_t e0 = off[a], eend = off[a + 1];
   const int64_t e1 = eend > e0 ? eend - 1 : e0;  // returns live at h in [e0, e1)
+  // bounds q = 2 r (lower) and 2 r + 1 of image m = r - 1: warps 0 and 1 take
+  // those of the tile itself, warps 2 and 3 the two of an image each (mostly empty)
   const int w = threadIdx.x >> 5;
-  if (w < 6) {
-    // warp w: threshold w of image m = w/2 - 1 (lower bound for even w)
-    const int m = w / 2 - 1;
-    long long A = L - p.khi + (long long)m * p.Mr;
-    long long B = L + Tlen - p.klo + (long long)m * p.Mr;
-    if (A < 0) A = 0;
-    if (B > p.Mr + 1) B = p.Mr + 1;
-    int64_t r = 0;
-    if (A < B) r = warp_first_ge(rb0, e0, e1, (w & 1) ? B : A);
-    else r = -1;  // empty image
-    if ((threadIdx.x & 31) == 0) s_res[w] = r;
+  if (w < 4) {
+    const int q0 = w < 2 ? 2 + w : (w == 2 ? 0 : 4), nq = w < 2 ? 1 : 2;
+    for (int q = q0; q < q0 + nq; ++q) {
+      const int m = q / 2 - 1;
+      long long A = L - p.khi + (long long)m * p.Mr;
+      long long B = L + Tlen - p.klo + (long long)m * p.Mr;
+      if (A < 0) A = 0;
+      if (B > p.Mr + 1) B = p.Mr + 1;
+      int64_t r = -1;  // empty image
+      if (A < B) {
+        const long long x = (q & 1) ? B : A;
+        // where it would lie were the records spread evenly
+        const int64_t guess = (int64_t)((float)(e1 - e0) * ((float)x / (float)p.Mr));
+        r = warp_first_ge(rb0, e0, e1, x, guess);
+      }
+      if ((threadIdx.x & 31) == 0) s_res[q] = r;
+    }
   }
   __syncthreads();
   for (int r = 0; r < 3; ++r) {

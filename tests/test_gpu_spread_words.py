@@ -1,0 +1,83 @@
+"""The float32 scatter's choice between one word per cell (sparse tiles) and two
+(dense ones), at its edges: stencils' widths holding 20 and 21 records, 1024
+and 1025 records in a tile, dense tiles larger than half the shared words, odd
+tile sizes, one return dwarfing the others, returns near the ends of the float
+range. Against an FP64 plan of the same tolerance, which shares the kernel's
+truncation: the float32 path's own rounding is at most 1e-6 relative (its parity
+tests bound it by the same figure); and the oracle's direct sum (Eq. (15) <=
+1e-5)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2003_02842_gb300 import synth
+
+from gpu_helpers import rel_l2_rows, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__ as g
+    g.build()
+
+
+def _coeffs(ev, N, kernel, prec, tile=0, tol=1e-6):
+    import paper_2003_02842_gb300 as mm
+    plan = mm.mm_plan_create(D=ev.D, N_max=N, max_events=ev.n_events, tol=tol, kernel=kernel, prec=prec,
+                             spread_tile=tile)
+    F, _ = mm.mm_coeffs(plan, *to_dev(ev), N)
+    assert mm.mm_plan_sync(plan) == 0
+    F = F.cpu().numpy()
+    mm.mm_destroy(plan)
+    return F.astype(np.complex128)
+
+
+def _check(ev, N, kernel="es", tile=0, scale=1.0):
+    F, G = _coeffs(ev, N, kernel, "bf16x3", tile) / scale, _coeffs(ev, N, kernel, "fp64") / scale
+    assert rel_l2_rows(F, G).max() <= 1e-6
+    assert rel_l2_rows(F, oracle.coeffs_F(ev.offsets, ev.t, ev.logp, N) / scale).max() <= 1e-5
+
+
+def _clusters(per, N, seed=0):
+    # clusters of `per` records inside a few cells, between empty stretches
+    rng = np.random.default_rng([per, N, seed])
+    T, cell = 10000.0, 10000.0 / (4 * N + 2)
+    t = np.sort(np.concatenate([[0.0, T], (np.arange(20)[:, None] * 500 + 7.3 +
+                                           rng.uniform(0, 8 * cell, (20, per))).ravel()]))
+    p = 4.6 + np.cumsum(0.01 * rng.standard_normal(len(t)))
+    return synth.from_lists([t, t[::2]], [p, p[::2]])
+
+
+@pytest.mark.parametrize("kernel", ["es", "kb", "gauss"])
+@pytest.mark.parametrize("per", [19, 20, 21, 40])
+def test_records_per_stencil_width(kernel, per):
+    _check(_clusters(per, 900), 900, kernel)
+
+
+@pytest.mark.parametrize("n", [1024, 1025, 1026, 3000])
+@pytest.mark.parametrize("tile", [0, 37, 2047, 4095])
+def test_chunk_and_tile_edges(n, tile):
+    ev = synth.random_events(n + tile, D=2, n_range=(n, n), T=5000.0)
+    _check(ev, 1000, tile=tile)
+
+
+@pytest.mark.parametrize("N,n", [(1000, 20000), (2100, 60000), (500, 4000)])
+def test_dense_tiles_in_parts(N, n):
+    ev = synth.random_events(n, D=2, n_range=(n, n), T=28800.0)
+    _check(ev, N, tile=4096)
+    _check(ev, N)
+
+
+@pytest.mark.parametrize("scale", [2.0**-100, 2.0**-92, 2.0**-80, 2.0**80])
+def test_returns_near_the_float_range(scale):
+    ev = synth.random_events(5, D=2, n_range=(300, 600), T=2000.0)
+    _check(synth.Events(ev.offsets, ev.t, (ev.logp - 4.6) * scale), 700, scale=scale)
+
+
+def test_one_return_dwarfs_the_others():
+    ev = synth.random_events(6, D=2, n_range=(500, 600), T=2000.0)
+    lp = ev.logp.copy()
+    lp[100:] += 1.0e4
+    _check(synth.Events(ev.offsets, ev.t, lp), 700)
