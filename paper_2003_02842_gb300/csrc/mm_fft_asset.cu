@@ -231,6 +231,85 @@ __device__ __forceinline__ void run_pass_t(int R, Cplx<float>* s, int L, int m, 
   }
 }
 
+// Decimation-in-time passes of a pair's half row. Its positions are padded by
+// one point after every m_1 (the largest stride): consecutive natural inputs lie
+// m_1 apart, which is a multiple of the 32 banks for many lengths (600 at 14,400
+// points), and the first pass stores them so. nb = blocks of the pass per m_1
+// (1 for the last one, p = 0, whose elements lie m_1 + 1 apart).
+template <int R>
+__device__ __forceinline__ void fft_pass_pad(Cplx<float>* __restrict__ s, int L, int m, int nb,
+                                             const float4* __restrict__ anc, int nth) {
+  const int nbf = L / R;
+  const unsigned mm = magic_of((unsigned)m), mb = magic_of((unsigned)nb);
+  const int step = nb == 0 ? m + 1 : m;
+  for (int i = threadIdx.x; i < nbf; i += nth) {
+    const int b = fast_div(i, m, mm);
+    const int j = i - b * m;
+    const int base = nb == 0 ? j : b * (R * m) + j + fast_div(b, nb, mb);
+    Cplx<float> v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = s[base + r * step];
+    apply_twiddles<R>(v, anc, j);
+    Codelet<R>::run(v);
+#pragma unroll
+    for (int q = 0; q < R; ++q) s[base + q * step] = v[q];
+  }
+}
+// The first pass (unit stride, no twiddles) on points fetched from global memory:
+// butterfly u takes the natural inputs u + r L / R, r < R, of which z holds every
+// second point, and stores its block of R at the digit reversal of u. Lanes
+// fetch neighbouring points and all of a CTA's fetches are in flight at once.
+template <int R, class Pos>
+__device__ __forceinline__ void fft_first_pass(Cplx<float>* __restrict__ s, const Cplx<float>* __restrict__ z, int L,
+                                               int nth, Pos pos) {
+  const int nbf = L / R;
+  for (int u = threadIdx.x; u < nbf; u += nth) {
+    Cplx<float> v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = z[2 * (size_t)(u + r * nbf)];
+    Codelet<R>::run(v);
+    Cplx<float>* d = s + pos(u);
+#pragma unroll
+    for (int q = 0; q < R; ++q) d[q] = v[q];
+  }
+}
+
+// f(radix as a compile-time constant); MAXR bounds the codelets compiled in.
+template <int MAXR, class F>
+__device__ __forceinline__ void with_radix(int R, F&& f) {
+  switch (R) {
+    case 2: f(std::integral_constant<int, 2>{}); return;
+    case 3: f(std::integral_constant<int, 3>{}); return;
+    case 4: f(std::integral_constant<int, 4>{}); return;
+    case 5: f(std::integral_constant<int, 5>{}); return;
+    case 6: f(std::integral_constant<int, 6>{}); return;
+    case 8: f(std::integral_constant<int, 8>{}); return;
+    case 9: f(std::integral_constant<int, 9>{}); return;
+    case 10: f(std::integral_constant<int, 10>{}); return;
+    case 12: f(std::integral_constant<int, 12>{}); return;
+    case 15: f(std::integral_constant<int, 15>{}); return;
+    case 16: f(std::integral_constant<int, 16>{}); return;
+    default: break;
+  }
+  if constexpr (MAXR >= 25) {
+    switch (R) {
+      case 18: f(std::integral_constant<int, 18>{}); return;
+      case 20: f(std::integral_constant<int, 20>{}); return;
+      case 24: f(std::integral_constant<int, 24>{}); return;
+      case 25: f(std::integral_constant<int, 25>{}); return;
+      default: break;
+    }
+  }
+  if constexpr (MAXR >= 32) {
+    switch (R) {
+      case 27: f(std::integral_constant<int, 27>{}); return;
+      case 30: f(std::integral_constant<int, 30>{}); return;
+      case 32: f(std::integral_constant<int, 32>{}); return;
+      default: break;
+    }
+  }
+}
+
 // Entry p of a per-pass array, selected without indexing it at run time (a
 // run-time index would move the kernel parameter into local memory).
 __device__ __forceinline__ int pick(const int (&a)[kMaxAssetPasses], int p) {
@@ -287,6 +366,9 @@ __device__ __forceinline__ int out_pos(int k, const AssetFft& f, const RevTab& t
 // Byte offset of the anchor rows in shared memory: after the nl complex
 // points, rounded up to 16 bytes (nl may be odd) for the float4 accesses.
 __host__ __device__ __forceinline__ size_t anchor_offset(int points) { return ((size_t)points * 8 + 15) & ~(size_t)15; }
+
+// Shared-memory points of a pair's half row, padding included.
+__host__ __device__ __forceinline__ int pair_points(const AssetFft& f) { return f.nl + f.rad[0]; }
 
 // The two digit-reversal tables of a decimation-in-frequency plan, built in
 // shared memory after the anchor rows (from the plan alone: no global reads).
@@ -539,33 +621,47 @@ __global__ void __launch_bounds__(NTH, 1)
   }
 }
 
-// The pair's local transform, the join of the two halves through
-// distributed shared memory and the unpacking and deconvolution of the
-// modes k = c, c + 2, ... <= N (CTA c of the cluster).
-template <int NTH, bool BIG>
-__device__ __forceinline__ void pair_finish(const AssetFft& f, Cplx<float>* s, const float4* anc, unsigned c, int a,
-                                            const RevTab& rt, const Cplx<float>* __restrict__ W,
-                                            const Cplx<float>* __restrict__ U, const float* __restrict__ decon,
-                                            Cplx<float>* __restrict__ out) {
+// The join of a pair's two halves (X_c in the shared memory of CTA c, natural
+// order, padded by one point after every `m1`; 0: not padded) through
+// distributed shared memory, and the unpacking and deconvolution of the modes
+// k <= N. With L = n / 2, Z_k = X_0[k] + w_n^k X_1[k] for k < L and Z_{k+L} =
+// X_0[k] - w_n^k X_1[k]; the modes k and L - k need the same four values (X_0,
+// X_1 at k and L - k) and their tables mirror (w_n^{L-k} = -conj w_n^k,
+// U[L-k] = -i conj U[k]), so a thread takes both: half the reads of a mode each.
+// CTA c takes the pairs k = c, c + 2, ... <= L / 2.
+template <int NTH>
+__device__ __forceinline__ void pair_unpack(const AssetFft& f, const Cplx<float>* s, unsigned c, int a, int m1,
+                                            const Cplx<float>* __restrict__ W, const Cplx<float>* __restrict__ U,
+                                            const float* __restrict__ decon, Cplx<float>* __restrict__ out) {
   constexpr int kPB = kPairBatch<NTH>;
   const int L = f.nl;
-  run_passes<BIG>(f, s, anc, NTH, L);
-  cluster_sync_all();  // both halves transformed and visible to the partner
+  const unsigned mm1 = magic_of((unsigned)(m1 > 0 ? m1 : 1));
+  auto at = [&](int k) { return m1 > 0 ? k + fast_div(k, m1, mm1) : k; };
   const uint32_t peer = peer_addr(s, c ^ 1u);
   Cplx<float>* oa = out + (size_t)a * (f.N + 1);
-  for (int k0 = (int)c + 2 * (int)threadIdx.x; k0 <= f.N; k0 += 2 * NTH * kPB) {
-    float dk[kPB];
-    Cplx<float> Uk[kPB], Wk[kPB], A0[kPB], A1[kPB], B0[kPB],
-        B1[kPB];
+  // G(k) from Z_k and Z_{n-k}
+  auto emit = [&](int k, Cplx<float> Zk, Cplx<float> Znk, Cplx<float> Uk, float dk) {
+    const Cplx<float> Zc = cconj(Znk);
+    const Cplx<float> E = {0.5f * (Zk.x + Zc.x), 0.5f * (Zk.y + Zc.y)};
+    const Cplx<float> dlt = csub(Zk, Zc);
+    const Cplx<float> O = {0.5f * dlt.y, -0.5f * dlt.x};  // (Z_k - conj Z_{n-k}) / (2i)
+    const Cplx<float> G = cadd(E, cmul(Uk, O));
+    oa[k] = Cplx<float>{G.x * dk, G.y * dk};
+  };
+  const int last = min(L / 2, f.N);
+  for (int k0 = (int)c + 2 * (int)threadIdx.x; k0 <= last; k0 += 2 * NTH * kPB) {
+    float dk[kPB], dj[kPB];
+    Cplx<float> Uk[kPB], Wk[kPB], A0[kPB], A1[kPB], B0[kPB], B1[kPB];
 #pragma unroll
     for (int u = 0; u < kPB; ++u) {
       const int k = k0 + u * 2 * NTH;
-      if (k <= f.N) {
+      if (k <= last) {
         const int j = k == 0 ? 0 : L - k;  // (n - k) mod L
         dk[u] = __ldg(decon + k);
+        dj[u] = k > 0 && j <= f.N ? __ldg(decon + j) : 0.0f;
         Uk[u] = U[k];
         Wk[u] = W[k];
-        const int pk = out_pos(k, f, rt), pj = out_pos(j, f, rt);  // the same layout in both CTAs
+        const int pk = at(k), pj = at(j);  // the same layout in both CTAs
         const Cplx<float> lk = s[pk], lj = s[pj];
         const Cplx<float> rk = ld_cluster(peer + 8u * (uint32_t)pk), rj = ld_cluster(peer + 8u * (uint32_t)pj);
         A0[u] = c == 0 ? lk : rk;  // X_0[k]
@@ -577,43 +673,57 @@ __device__ __forceinline__ void pair_finish(const AssetFft& f, Cplx<float>* s, c
 #pragma unroll
     for (int u = 0; u < kPB; ++u) {
       const int k = k0 + u * 2 * NTH;
-      if (k <= f.N) {
-        const Cplx<float> Zk = cadd(A0[u], cmul(Wk[u], A1[u]));
-        const Cplx<float> Znk = cadd(B0[u], cmul(cconj(Wk[u]), B1[u]));  // w_n^{n-k} = conj(w_n^k)
-        const Cplx<float> Zc = cconj(Znk);
-        const Cplx<float> E = {0.5f * (Zk.x + Zc.x), 0.5f * (Zk.y + Zc.y)};
-        const Cplx<float> dlt = csub(Zk, Zc);
-        const Cplx<float> O = {0.5f * dlt.y, -0.5f * dlt.x};  // (Z_k - conj Z_{n-k}) / (2i)
-        const Cplx<float> G = cadd(E, cmul(Uk[u], O));
-        oa[k] = Cplx<float>{G.x * dk[u], G.y * dk[u]};
+      if (k <= last) {
+        const Cplx<float> ta = cmul(Wk[u], A1[u]), tb = cmul(cconj(Wk[u]), B1[u]);
+        // Z_k and Z_{n-k}: w_n^{n-k} = conj(w_n^k)
+        emit(k, cadd(A0[u], ta), cadd(B0[u], tb), Uk[u], dk[u]);
+        const int j = L - k;
+        // Z_{L-k} = X_0[j] - conj(w_n^k) X_1[j] and Z_{n-(L-k)} = Z_{L+k}
+        if (k > 0 && j != k && j <= f.N)
+          emit(j, csub(B0[u], tb), csub(A0[u], ta), Cplx<float>{-Uk[u].y, -Uk[u].x}, dj[u]);
       }
     }
+  }
+  // k = L alone when N reaches it: Z_L = X_0[0] - X_1[0], its own mirror
+  if (f.N >= L && c == 0 && threadIdx.x == 0) {
+    const Cplx<float> Z = csub(s[0], ld_cluster(peer));
+    emit(L, Z, Z, U[L], decon[L]);
   }
   cluster_sync_all();  // the partner has finished reading this CTA's shared memory
 }
 
-// Two CTAs per asset as a thread-block cluster (decimation in time by 2):
-// CTA c transforms x_c[m] = z[2m + c], m < L = n/2, loaded straight into
-// its shared memory by asynchronous copies; then
-//   Z_k = X_0[k mod L] + w_n^k X_1[k mod L]
-// joins the halves, each CTA reading its partner's X through distributed
-// shared memory while it unpacks and deconvolves every other mode.
+// The resident form's finish: every pass from shared memory, then the join.
 template <int NTH, bool BIG>
+__device__ __forceinline__ void pair_finish(const AssetFft& f, Cplx<float>* s, const float4* anc, unsigned c, int a,
+                                            const Cplx<float>* __restrict__ W, const Cplx<float>* __restrict__ U,
+                                            const float* __restrict__ decon, Cplx<float>* __restrict__ out) {
+  run_passes<BIG>(f, s, anc, NTH, f.nl);
+  cluster_sync_all();  // both halves transformed and visible to the partner
+  pair_unpack<NTH>(f, s, c, a, 0, W, U, decon, out);
+}
+
+// Two CTAs per asset as a thread-block cluster (decimation in time by 2):
+// CTA c transforms x_c[m] = z[2m + c], m < L = n/2, then the halves join (above).
+// One CTA per SM runs (its half row fills the shared memory), so each phase's
+// latency counts: the row is fetched straight into the first pass's registers
+// (a copy into digit-reversed slots first cost 5 of 22.6 us), the slots are padded
+// against bank conflicts, and a thread unpacks two modes from the same values.
+// 5120 rows of 28,800 points: 1595 us before, 1059 us with these.
+template <int NTH, int MAXR>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTH, 1)
     k_fft_asset_pair(const float* __restrict__ grid, AssetFft f, const Cplx<float>* __restrict__ W,
                      const Cplx<float>* __restrict__ tw, const Cplx<float>* __restrict__ U,
                      const float* __restrict__ decon, Cplx<float>* __restrict__ out, const int* __restrict__ gate) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Cplx<float>* s = reinterpret_cast<Cplx<float>*>(smem_raw);
-  float4* anc = reinterpret_cast<float4*>(smem_raw + anchor_offset(f.nl));
+  const int L = f.nl, m1 = f.stride[0];
+  float4* anc = reinterpret_cast<float4*>(smem_raw + anchor_offset(pair_points(f)));
   unsigned c;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(c));
   const int a = blockIdx.y;
-  const int L = f.nl;
   unsigned mr[kMaxAssetPasses];
 #pragma unroll
   for (int p = 0; p < kMaxAssetPasses; ++p) mr[p] = magic_of((unsigned)f.rad[p]);
-  const RevTab rt = build_rev_tables<NTH>(f, smem_raw, mr, f.nl);
   pdl_wait();  // the grid comes from the spreading kernel
   // every CTA of the cluster reads the same gate word: both leave or neither
   if (*gate) return;
@@ -624,15 +734,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTH, 1)
       const uint32_t dst = (uint32_t)__cvta_generic_to_shared(anc + i);
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src + i) : "memory");
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   }
   const Cplx<float>* z = reinterpret_cast<const Cplx<float>*>(grid) + (size_t)a * f.n + c;
-  for (int m = threadIdx.x; m < L; m += NTH) {
-    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s + (f.dif ? m : digit_rev(m, f, mr)));
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(z + 2 * (size_t)m) : "memory");
-  }
-  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+  // a position below m_1 times q_0 is padded by q_0, the first digit of u
+  with_radix<MAXR>(pick(f.rad, f.npass - 1), [&](auto r) {
+    fft_first_pass<decltype(r)::value>(s, z, L, NTH, [&](int u) {
+      const int q0 = u - fast_div(u, f.rad[0], mr[0]) * f.rad[0];
+      return digit_rev(u, f, mr) + (f.npass > 1 ? q0 : 0);
+    });
+  });
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  pair_finish<NTH, BIG>(f, s, anc, c, a, rt, W, U, decon, out);
+  for (int p = f.npass - 2; p >= 0; --p) {
+    const int R = pick(f.rad, p), m = pick(f.stride, p);
+    with_radix<MAXR>(R, [&](auto r) {
+      fft_pass_pad<decltype(r)::value>(s, L, m, p == 0 ? 0 : m1 / (R * m), anc + 2 * pick(f.tw_off, p), NTH);
+    });
+    if (p > 0) __syncthreads();
+  }
+  cluster_sync_all();  // both halves transformed and visible to the partner
+  pair_unpack<NTH>(f, s, c, a, f.npass > 1 ? m1 : 0, W, U, decon, out);
 }
 
 // Stages (a2)-(c) in one launch with the grid row resident in shared
@@ -808,9 +930,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
   spread_resident<NT, NTH>(off, rb0, rd, rv, sp, poly, sub, f, mr, a, PairCells{c}, s,
                            smem_raw + anchor_offset(f.nl));
   load_anchors<NTH>(f, tw, anc);
-  const RevTab rt = build_rev_tables<NTH>(f, smem_raw, mr, f.nl);  // none: decimation in time
   __syncthreads();
-  pair_finish<NTH, true>(f, s, anc, c, a, rt, W, U, decon, out);
+  pair_finish<NTH, true>(f, s, anc, c, a, W, U, decon, out);
 }
 
 // Twiddle anchors of each pass: row j < m_p holds w^1..w^4 of w = w_{L_p}^j,
@@ -844,7 +965,7 @@ bool asset_fft_radix_ok(int R) {
 }
 
 static size_t asset_rows_smem(const AssetFft& f, int rows) {
-  return anchor_offset(rows * f.nl) + (size_t)f.tw_rows * 32 + (f.dif ? (size_t)(f.rev_lo + f.rev_hi) * 4 : 0);
+  return anchor_offset(f.pair ? pair_points(f) : rows * f.nl) + (size_t)f.tw_rows * 32 + (f.dif ? (size_t)(f.rev_lo + f.rev_hi) * 4 : 0);
 }
 
 size_t asset_fft_smem(const AssetFft& f) { return asset_rows_smem(f, 1); }
@@ -945,8 +1066,12 @@ cudaError_t launch_fft_asset(const float* grid, const AssetFft& f, int D, const 
   // measured fastest with 512 threads and radices up to 32.
   const bool big = asset_fft_max_radix(f) > 16;
   if (f.pair) {
-    if (big) return go(k_fft_asset_pair<kPairThreads, true>, dim3(2, D), kPairThreads);
-    return go(k_fft_asset_pair<kPairThreads, false>, dim3(2, D), kPairThreads);
+    // three passes of 24, 24 and 25 points (14,400) are 576 to 600 butterflies:
+    // one round of 608 threads
+    const int maxr = asset_fft_max_radix(f);
+    if (maxr > 25) return go(k_fft_asset_pair<kPairThreads, 32>, dim3(2, D), kPairThreads);
+    if (maxr > 16) return go(k_fft_asset_pair<608, 25>, dim3(2, D), 608);
+    return go(k_fft_asset_pair<kPairThreads, 16>, dim3(2, D), kPairThreads);
   }
   const int rows = asset_rows(f, D);
   if (rows > 1) {
