@@ -359,11 +359,13 @@ struct mm_plan_s {
   void* s_sigma = nullptr;
   void* s_R = nullptr;
   int* h_status = nullptr;        // pinned: the host-buffer entry point's status read-back
+  int* row_exp = nullptr;         // FP64: each asset's largest exponent field of a return
   int* asset_order = nullptr;     // spreading dispatch order (single problems of D <= kOrderMaxAssets)
   int64_t workspace = 0;
   // per-cutoff configuration
   int cfg_N = -1;
   int tab_N = -1;
+  bool tab_pair = false;          // tables in float pairs
   // autotuned choices (-1 = library default); applied by configure()
   int tune_algo = -1;     // 0 scatter, 1 gather, 2 fused
   int tune_tile = -1;     // spreading cells per block
@@ -435,7 +437,7 @@ void free_all(mm_plan p) {
   void* ptrs[] = {p->grid, p->rec_b0, p->rec_d, p->rec_v, p->W, p->atw, p->U, p->decon, p->es, p->bounds, p->gscale, p->status, p->gapbits, p->wsq,
                   p->partial, p->acc[0], p->acc[1], p->gram_done, p->pw_N, p->pw_sig, p->pw_A,
                   p->pw_V, p->pw_clip, p->s_off, p->s_t, p->s_p, p->s_coef,
-                  p->s_sigma, p->s_R, p->asset_order, p->tma_hi, p->tma_lo, p->pw_sync, p->pw_part, p->pw_log};
+                  p->s_sigma, p->s_R, p->row_exp, p->asset_order, p->tma_hi, p->tma_lo, p->pw_sync, p->pw_part, p->pw_log};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   if (p->h_status) cudaFreeHost(p->h_status);
@@ -667,6 +669,7 @@ mm_status configure(mm_plan p, int N) {
     }
   }
   if (want_fused && !p->res_sub && fits && p->G == 1) s.fused = 1;
+  if (s.fused) p->pair_ok = false;  // the one-CTA kernel spreads and transforms in float64
   p->afft = af;
   p->use_afft = afft && !s.fused;
   p->fft = f;
@@ -679,11 +682,13 @@ mm_status configure(mm_plan p, int N) {
 }
 
 mm_status ensure_tables(mm_plan p, int N, cudaStream_t st) {
-  if (p->tab_N == N) return MM_OK;
+  if (p->tab_N == N && p->tab_pair == p->pair_ok) return MM_OK;
   StageScope sc(p, MM_STAGE_SETUP, st);
   MM_CUDA(launch_setup_tables(p->desc.kernel, p->msp, p->Mr, N, p->fft.n, p->sp, p->tau, p->es,
-                              p->es + kEsNodes, p->es + 2 * kEsNodes, p->W, p->U, p->decon, p->fp64, st));
+                              p->es + kEsNodes, p->es + 2 * kEsNodes, p->W, p->U, p->decon, p->pair_ok ? 2 : (p->fp64 ? 1 : 0),
+                              st));
   p->tab_N = N;
+  p->tab_pair = p->pair_ok;
   return MM_OK;
 }
 
@@ -769,7 +774,7 @@ mm_status coeffs_impl(mm_plan p, const int64_t* off, const double* t, const doub
     StageScope sc(p, MM_STAGE_PREP, st);
     // a batch's cell scales come from launch_group_scales below, a thread each
     MM_CUDA(launch_bounds(off, t, D, p->gsize, p->desc.max_events, t0, t1, p->G > 1 ? 0 : Mr_known, p->bounds,
-                          p->status, use_order ? p->asset_order : nullptr, st));
+                          p->status, use_order ? p->asset_order : nullptr, p->row_exp, st));
   }
   if (N <= 0 && p->G > 1) return MM_ERR_CUTOFF;  // a batch sweeps given cutoffs
   if (N <= 0) {
@@ -805,7 +810,8 @@ mm_status coeffs_impl(mm_plan p, const int64_t* off, const double* t, const doub
     {
       StageScope sc(p, MM_STAGE_PREP, st);
       if (p->fp64)
-        MM_CUDA(launch_prep_f64(off, t, logp, p->bounds, gsc, p->gsize, D, p->Mr, p->desc.max_events, p->pair_ok,
+        MM_CUDA(launch_prep_f64(off, t, logp, p->bounds, gsc, p->gsize, D, p->Mr, p->desc.max_events,
+                                p->pair_ok ? p->row_exp : nullptr,
                                 p->rec_b0, p->rec_d, p->rec_v, p->status, st));
       else
         MM_CUDA(launch_prep_f32(off, t, logp, p->bounds, gsc, p->gsize, D, p->Mr, p->desc.max_events, p->rec_b0,
@@ -822,8 +828,8 @@ mm_status coeffs_impl(mm_plan p, const int64_t* off, const double* t, const doub
       StageScope sc(p, MM_STAGE_SPREAD, st);
       p->sp.order = use_order ? p->asset_order : nullptr;
       if (p->pair_ok)
-        MM_CUDA(launch_spread_pair(off, p->rec_b0, p->rec_d, p->rec_v, p->sp, p->pair_poly, (double*)p->grid,
-                                   p->status, st));
+        MM_CUDA(launch_spread_pair(off, p->rec_b0, p->rec_d, p->rec_v, p->sp, p->pair_poly, p->row_exp,
+                                   p->grid, p->status, st));
       else if (p->fp64)
         MM_CUDA(launch_spread_f64(off, p->rec_b0, p->rec_d, p->rec_v, p->sp, (double*)p->grid, p->status, st));
       else if (p->poly_ok)
@@ -839,12 +845,15 @@ mm_status coeffs_impl(mm_plan p, const int64_t* off, const double* t, const doub
     } else {
     {
       StageScope sc(p, MM_STAGE_FFT_COLS, st);
-      if (p->fp64) MM_CUDA(launch_fft_cols_f64((double*)p->grid, p->fft, D, p->W, p->status, st));
+      if (p->pair_ok) MM_CUDA(launch_fft_cols_pair(p->grid, p->fft, D, p->W, p->status, st));
+      else if (p->fp64) MM_CUDA(launch_fft_cols_f64((double*)p->grid, p->fft, D, p->W, p->status, st));
       else MM_CUDA(launch_fft_cols_f32((float*)p->grid, p->fft, D, p->W, p->status, st));
     }
     {
       StageScope sc(p, MM_STAGE_FFT_ROWS, st);
-      if (p->fp64)
+      if (p->pair_ok)
+        MM_CUDA(launch_fft_rows_pair(p->grid, p->fft, D, p->W, p->U, p->decon, p->row_exp, coeffs, p->status, st));
+      else if (p->fp64)
         MM_CUDA(launch_fft_rows_f64((const double*)p->grid, p->fft, D, p->W, p->U, p->decon, coeffs, p->status, st));
       else
         MM_CUDA(launch_fft_rows_f32((const float*)p->grid, p->fft, D, p->W, p->U, p->decon, coeffs, p->status, st));
@@ -935,7 +944,7 @@ mm_status estimate_eager(mm_plan p, const int64_t* off, const double* t, const d
 mm_status estimate_impl(mm_plan p, const int64_t* off, const double* t, const double* logp, int N, double t0,
                         double t1, void* coeffs, void* sigma, void* R, int32_t* N_used, cudaStream_t st) {
   const bool steady = p->graphs && !p->prof && N > 0 && p->G == 1 && p->cfg_N == N && p->cfg_D == p->D &&
-                      p->tab_N == N && p->w_N == N && p->w_basis == (int)p->desc.basis &&
+                      p->tab_N == N && p->tab_pair == p->pair_ok && p->w_N == N && p->w_basis == (int)p->desc.basis &&
                       (p->fp64 || (!p->acc_dirty && p->acc_D == p->D));
   if (!steady) return estimate_eager(p, off, t, logp, N, t0, t1, coeffs, sigma, R, N_used, st);
   mm_plan_s::EstGraph& G = p->eg[p->fp64 ? 0 : p->acc_sel];
@@ -1089,6 +1098,7 @@ mm_status plan_create_impl(const mm_plan_desc* desc, int gsize, bool batch, mm_p
   A(&p->decon, Np1 * p->rs);
   A((void**)&p->es, (2 * kEsNodes + kEsChebMax) * sizeof(double));
   A((void**)&p->bounds, (size_t)p->G * sizeof(Rescale));
+  if (p->fp64) A((void**)&p->row_exp, std::max<size_t>(D, 1) * sizeof(int));
   if (!batch && D <= (size_t)kOrderMaxAssets) A((void**)&p->asset_order, std::max<size_t>(D, 1) * sizeof(int));
   if (p->G > 1) A(&p->gscale, (size_t)p->G * group_scale_bytes());
   A((void**)&p->status, 4 * sizeof(int));
@@ -1446,7 +1456,7 @@ mm_status mm_nyquist(mm_plan p, const int64_t* d_offsets, const double* d_t, dou
   {
     StageScope sc(p, MM_STAGE_PREP, st);
     MM_CUDA(launch_bounds(d_offsets, d_t, p->D, p->gsize, p->desc.max_events, t0, t1, 0, p->bounds, p->status,
-                          nullptr, st));
+                          nullptr, nullptr, st));
   }
   {
     StageScope sc(p, MM_STAGE_PREP, st, 2);

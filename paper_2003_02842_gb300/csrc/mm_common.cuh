@@ -34,6 +34,33 @@ struct __align__(2 * sizeof(T)) Cplx {
   T x, y;
 };
 
+// Float pairs h + l for the FP64 path's tolerances: about 47 significant bits
+// from float32 operations, which GB300 issues some 64 times faster than float64
+// ones. A sum is Knuth's two-sum of the high parts plus the low parts (8
+// operations), a product the rounded one of the high parts, its error by a fused
+// multiply-add and the cross terms (4); the low part stays within a few units in
+// the last place of the high one and is not renormalised.
+struct __align__(8) FloatPair {
+  float h, l;
+  FloatPair() = default;
+  __host__ __device__ __forceinline__ constexpr FloatPair(float a, float b) : h(a), l(b) {}
+  __host__ __device__ __forceinline__ constexpr explicit FloatPair(double x)
+      : h((float)x), l((float)(x - (double)(float)x)) {}
+  __host__ __device__ __forceinline__ constexpr explicit FloatPair(int x) : h((float)x), l(0.0f) {}
+  __device__ __forceinline__ explicit operator double() const { return (double)h + (double)l; }
+};
+__device__ __forceinline__ FloatPair operator-(FloatPair a) { return FloatPair(-a.h, -a.l); }
+__device__ __forceinline__ FloatPair operator+(FloatPair a, FloatPair b) {
+  const float s = __fadd_rn(a.h, b.h), t = __fsub_rn(s, a.h);
+  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
+  return FloatPair(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ FloatPair operator-(FloatPair a, FloatPair b) { return a + (-b); }
+__device__ __forceinline__ FloatPair operator*(FloatPair a, FloatPair b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return FloatPair(p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p))));
+}
+
 template <typename T>
 __device__ __forceinline__ Cplx<T> cmul(Cplx<T> a, Cplx<T> b) {
   return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
@@ -191,7 +218,8 @@ constexpr int kMaxEppsAssets = 12;
 // order != NULL (a single problem of D <= kOrderMaxAssets): also ranks the
 // assets by event count, heaviest first, into order[0..D-1].
 cudaError_t launch_bounds(const int64_t* off, const double* t, int D, int gsize, int64_t max_events,
-                          double w0, double w1, int64_t Mr, Rescale* rs, int* status, int* order, cudaStream_t s);
+                          double w0, double w1, int64_t Mr, Rescale* rs, int* status, int* order, int* row_exp,
+                          cudaStream_t s);  // row_exp != NULL: cleared, for launch_prep_f64
 cudaError_t launch_group_scales(const Rescale* rs, int G, int64_t Mr, GroupScale* out, const int* status,
                                 cudaStream_t s);
 size_t group_scale_bytes();
@@ -200,9 +228,10 @@ cudaError_t launch_min_gap(const int64_t* off, const double* t, int D, const Res
 cudaError_t launch_prep_f32(const int64_t* off, const double* t, const double* logp, const Rescale* rs,
                             const GroupScale* gsc, int gsize, int D, int64_t Mr, int64_t max_events, int* rb0,
                             void* rd, void* rv, int* status, cudaStream_t s);
-// pair: the records' offsets d as float pairs z = d - 1/2 (launch_spread_pair)
+// row_exp != NULL: records for launch_spread_pair, the offsets d as float pairs
+// z = d - 1/2, and each asset's largest exponent field of a return
 cudaError_t launch_prep_f64(const int64_t* off, const double* t, const double* logp, const Rescale* rs,
-                            const GroupScale* gsc, int gsize, int D, int64_t Mr, int64_t max_events, bool pair,
+                            const GroupScale* gsc, int gsize, int D, int64_t Mr, int64_t max_events, int* row_exp,
                             int* rb0, void* rd, void* rv, int* status, cudaStream_t s);
 cudaError_t launch_spread_f32(const int64_t* off, const int* rb0, const void* rd, const void* rv,
                               const SpreadParams& p, float* grid, const int* status, cudaStream_t s);
@@ -213,10 +242,11 @@ bool spread_poly_supported(int ntaps);
 cudaError_t launch_spread_poly(const int64_t* off, const int* rb0, const void* rd, const void* rv,
                                const SpreadParams& p, const KernelPoly& poly, float* grid, const int* status,
                                cudaStream_t s);
-// FP64 scatter with the taps in float pairs and three-word integer accumulation
+// FP64 scatter with the taps in float pairs and three-word integer accumulation; the
+// grid in float pairs, a row scaled by 2^-(row_exp - 1022) (undone by launch_fft_rows_pair)
 cudaError_t launch_spread_pair(const int64_t* off, const int* rb0, const void* rd, const void* rv,
-                               const SpreadParams& p, const PairPoly& poly, double* grid, const int* status,
-                               cudaStream_t s);
+                               const SpreadParams& p, const PairPoly& poly, const int* row_exp, void* grid,
+                               const int* status, cudaStream_t s);
 cudaError_t launch_spread_f64(const int64_t* off, const int* rb0, const void* rd, const void* rv,
                               const SpreadParams& p, double* grid, const int* status, cudaStream_t s);
 
@@ -229,8 +259,13 @@ cudaError_t launch_es_fit(int msp, const double* y, const double* f, double* che
 cudaError_t launch_setup_tables(int kernel, int msp, int64_t Mr, int N, int64_t n,
                                 const SpreadParams& sp, double tau, const double* esy,
                                 const double* esf, const double* cheb, void* W, void* U, void* decon,
-                                bool fp64, cudaStream_t s);
+                                int kind, cudaStream_t s);  // 0: float32 tables, 1: float64, 2: float pairs
 cudaError_t launch_fft_cols_f32(float* grid, const FftParams& f, int D, const void* W, const int* status, cudaStream_t s);
+// the FP64 path on a grid and tables of float pairs
+cudaError_t launch_fft_cols_pair(void* grid, const FftParams& f, int D, const void* W, const int* status, cudaStream_t s);
+cudaError_t launch_fft_rows_pair(const void* grid, const FftParams& f, int D, const void* W, const void* U,
+                                 const void* decon, const int* row_exp, void* coeffs, const int* status,
+                                 cudaStream_t s);
 cudaError_t launch_fft_cols_f64(double* grid, const FftParams& f, int D, const void* W, const int* status, cudaStream_t s);
 cudaError_t launch_fft_rows_f32(const float* grid, const FftParams& f, int D, const void* W,
                                 const void* U, const void* decon, void* coeffs, const int* status, cudaStream_t s);

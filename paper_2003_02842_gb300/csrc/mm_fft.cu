@@ -14,7 +14,16 @@
 //     and F(k) = G(k) * decon(k) for k <= N, written with coalesced stores.
 // Both passes keep their rows in shared memory and ping-pong between two
 // buffers (autosorting Stockham), so no bit reversal is needed.
+//
+// FP64 plans run these passes in float pairs where their tolerance allows
+// (FloatPair; mm_spread.cu's scatter leaves such a grid): some 80 float64
+// operations per point set both passes' time on the float64 pipe, 179 + 222 us at
+// 100 rows of 20,250 points; in float pairs 55 + 67 us. The pairs' rounding
+// (2^-47 an operation) adds about 1e-14 to coefficients whose truncation is
+// 1e-12 at the tightest tolerance that takes this path.
 #include <math.h>
+
+#include <type_traits>
 
 #include "mm_common.cuh"
 #include "mm_fft_dev.cuh"
@@ -30,9 +39,13 @@ constexpr int kFftPer = 16;
 // ------------------------------------------------------------ pass 1
 // Every global load of a block (its column values and the write-back
 // twiddles) is issued in one batch into registers before the first barrier,
-// so the block waits for memory once.
+// so the block waits for memory once. Float pairs are bound by issue instead of
+// the float64 pipe and read their tables where they use them: two blocks an SM.
 template <typename T>
-__global__ void __launch_bounds__(kFftThreads) k_fft_cols(Cplx<T>* __restrict__ z, FftParams f,
+constexpr bool kTablesEarly = !std::is_same<T, FloatPair>::value;
+
+template <typename T>
+__global__ void __launch_bounds__(kFftThreads, kTablesEarly<T> ? 1 : 2) k_fft_cols(Cplx<T>* __restrict__ z, FftParams f,
                                                           const Cplx<T>* __restrict__ W, const int* __restrict__ gate) {
   if (*gate) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -53,7 +66,7 @@ __global__ void __launch_bounds__(kFftThreads) k_fft_cols(Cplx<T>* __restrict__ 
       const int j1 = idx >> lgB, j2 = j20 + (idx & (B - 1));
       if (j2 < Q) {
         v[i] = za[Q * j1 + j2];
-        wt[i] = W[j2 * j1];  // j2 k1 <= (Q-1)(P-1) < n: no reduction
+        if (kTablesEarly<T>) wt[i] = W[j2 * j1];  // j2 k1 <= (Q-1)(P-1) < n: no reduction
       }
     }
   }
@@ -70,7 +83,7 @@ __global__ void __launch_bounds__(kFftThreads) k_fft_cols(Cplx<T>* __restrict__ 
     const int idx = threadIdx.x + i * kFftThreads;
     if (idx < total) {
       const int k1 = idx >> lgB, c = idx & (B - 1), j2 = j20 + c;
-      if (j2 < Q) za[Q * k1 + j2] = cmul(X[swz(k1, c, lgB)], wt[i]);
+      if (j2 < Q) za[Q * k1 + j2] = cmul(X[swz(k1, c, lgB)], kTablesEarly<T> ? wt[i] : W[j2 * k1]);
     }
   }
 }
@@ -106,12 +119,19 @@ __device__ __forceinline__ int partner_of(const RowSet& r, int ri, int P, int H)
   return (r.mlo + (ri - r.nlow)) - r.r0;
 }
 
+// Type of the coefficients: float pairs leave as float64.
+template <typename T> struct Coef { using type = T; };
+template <> struct Coef<FloatPair> { using type = double; };
+
 // ------------------------------------------------------------ pass 2
 template <typename T>
-__global__ void __launch_bounds__(kFftThreads) k_fft_rows(const Cplx<T>* __restrict__ z, FftParams f,
+__global__ void __launch_bounds__(kFftThreads, kTablesEarly<T> ? 1 : 2) k_fft_rows(const Cplx<T>* __restrict__ z, FftParams f,
                                                           const Cplx<T>* __restrict__ W, const Cplx<T>* __restrict__ U,
-                                                          const T* __restrict__ decon, Cplx<T>* __restrict__ out,
+                                                          const T* __restrict__ decon,
+                                                          const int* __restrict__ row_exp,
+                                                          Cplx<typename Coef<T>::type>* __restrict__ out,
                                                           const int* __restrict__ gate) {
+  using TO = typename Coef<T>::type;
   if (*gate) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int P = f.P, Q = f.Q;
@@ -140,7 +160,7 @@ __global__ void __launch_bounds__(kFftThreads) k_fft_rows(const Cplx<T>* __restr
       const int k2 = idx >> lgB, ro = idx & (B - 1);
       const int k1 = row_of(rs, ro, P);
       const int k = k1 + P * k2;
-      if (k1 >= 0 && k <= f.N) {
+      if (kTablesEarly<T> && k1 >= 0 && k <= f.N) {
         uk[i] = U[k];
         dk[i] = decon[k];
       }
@@ -157,7 +177,10 @@ __global__ void __launch_bounds__(kFftThreads) k_fft_rows(const Cplx<T>* __restr
   }
   __syncthreads();
   const Cplx<T>* X = stockham_fft(buf0, buf1, tw, Q, lgB, f.rad_q, f.nrad_q);
-  Cplx<T>* oa = out + (int64_t)blockIdx.y * (f.N + 1);
+  Cplx<TO>* oa = out + (int64_t)blockIdx.y * (f.N + 1);
+  double unscale = 1.0;  // 2^(row_exp - 1022)
+  if constexpr (std::is_same<T, FloatPair>::value)
+    unscale = __longlong_as_double((long long)(row_exp[blockIdx.y] + 1) << 52);
 #pragma unroll
   for (int i = 0; i < kFftPer; ++i) {
     const int idx = threadIdx.x + i * kFftThreads;
@@ -168,13 +191,20 @@ __global__ void __launch_bounds__(kFftThreads) k_fft_rows(const Cplx<T>* __restr
     if (k1 < 0 || k > f.N) continue;
     const int pri = partner_of(rs, ri, P, f.H);
     const int pk2 = (k1 == 0) ? ((k2 == 0) ? 0 : Q - k2) : Q - 1 - k2;
+    if (!kTablesEarly<T>) {
+      uk[i] = U[k];
+      dk[i] = decon[k];
+    }
     const Cplx<T> Zk = X[swz(k2, ri, lgB)];
     const Cplx<T> Zc = cconj(X[swz(pk2, pri, lgB)]);
     const Cplx<T> E = {(T)0.5 * (Zk.x + Zc.x), (T)0.5 * (Zk.y + Zc.y)};
     const Cplx<T> dlt = csub(Zk, Zc);
     const Cplx<T> O = {(T)0.5 * dlt.y, (T)-0.5 * dlt.x};  // (Zk - Zc) / (2i)
     const Cplx<T> G = cadd(E, cmul(uk[i], O));
-    oa[k] = Cplx<T>{G.x * dk[i], G.y * dk[i]};
+    if constexpr (std::is_same<T, FloatPair>::value)
+      oa[k] = Cplx<TO>{(TO)(G.x * dk[i]) * unscale, (TO)(G.y * dk[i]) * unscale};
+    else
+      oa[k] = Cplx<TO>{G.x * dk[i], G.y * dk[i]};
   }
 }
 
@@ -290,7 +320,7 @@ __global__ void k_setup_tables(int kernel, int msp, int64_t Mr, int N, int64_t n
     } else {
       const double alpha = kPi * 2.0 * msp / (double)Mr;
       double acc = 0.0;
-      if constexpr (sizeof(T) == 4) {
+      if constexpr (std::is_same<T, float>::value) {
         // Clenshaw's recurrence at x = 2 (theta / theta_max)^2 - 1,
         // theta / theta_max = 4 k / M_r
         const double r = 4.0 * k / (double)Mr, x2 = 4.0 * r * r - 2.0;  // 2 x
@@ -313,17 +343,19 @@ __global__ void k_setup_tables(int kernel, int msp, int64_t Mr, int N, int64_t n
 
 cudaError_t launch_setup_tables(int kernel, int msp, int64_t Mr, int N, int64_t n, const SpreadParams& sp,
                                 double tau, const double* esy, const double* esf, const double* cheb,
-                                void* W, void* U, void* decon, bool fp64, cudaStream_t s) {
+                                void* W, void* U, void* decon, int kind, cudaStream_t s) {
   const int64_t m = n > (int64_t)N + 1 ? n : (int64_t)N + 1;
   const int nth = 128;
   const int blocks = (int)((m + nth - 1) / nth);
   const int nt = es_cheb_terms(msp);
-  if (fp64)
-    k_setup_tables<double><<<blocks, nth, 0, s>>>(kernel, msp, Mr, N, n, sp.kb_b, sp.kb_inv_phi0, tau, esy, esf,
-                                                  cheb, nt, (Cplx<double>*)W, (Cplx<double>*)U, (double*)decon);
-  else
-    k_setup_tables<float><<<blocks, nth, 0, s>>>(kernel, msp, Mr, N, n, sp.kb_b, sp.kb_inv_phi0, tau, esy, esf,
-                                                 cheb, nt, (Cplx<float>*)W, (Cplx<float>*)U, (float*)decon);
+  auto go = [&](auto t) {
+    using T = decltype(t);
+    k_setup_tables<T><<<blocks, nth, 0, s>>>(kernel, msp, Mr, N, n, sp.kb_b, sp.kb_inv_phi0, tau, esy, esf, cheb, nt,
+                                             (Cplx<T>*)W, (Cplx<T>*)U, (T*)decon);
+  };
+  if (kind == 2) go(FloatPair{});
+  else if (kind == 1) go(double{});
+  else go(float{});
   return cudaGetLastError();
 }
 
@@ -353,7 +385,8 @@ static cudaError_t launch_cols_t(T* grid, const FftParams& f, int D, const void*
 
 template <typename T>
 static cudaError_t launch_rows_t(const T* grid, const FftParams& f, int D, const void* W, const void* U,
-                                 const void* decon, void* coeffs, const int* status, cudaStream_t s) {
+                                 const void* decon, const int* row_exp, void* coeffs, const int* status,
+                                 cudaStream_t s) {
   const size_t smem = fft_rows_smem(f, sizeof(T) == 8);
   auto fn = k_fft_rows<T>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -361,7 +394,7 @@ static cudaError_t launch_rows_t(const T* grid, const FftParams& f, int D, const
   dim3 grd((f.H + f.rowblk - 1) / f.rowblk, D);
   if (((1 << f.lg_rowcols) * f.Q) > kFftThreads * kFftPer) return cudaErrorInvalidValue;
   fn<<<grd, kFftThreads, smem, s>>>(reinterpret_cast<const Cplx<T>*>(grid), f, (const Cplx<T>*)W, (const Cplx<T>*)U,
-                            (const T*)decon, (Cplx<T>*)coeffs, status + 1);
+                            (const T*)decon, row_exp, (Cplx<typename Coef<T>::type>*)coeffs, status + 1);
   return cudaGetLastError();
 }
 
@@ -373,13 +406,22 @@ cudaError_t launch_fft_cols_f64(double* grid, const FftParams& f, int D, const v
                                 cudaStream_t s) {
   return launch_cols_t<double>(grid, f, D, W, status, s);
 }
+cudaError_t launch_fft_cols_pair(void* grid, const FftParams& f, int D, const void* W, const int* status,
+                                 cudaStream_t s) {
+  return launch_cols_t<FloatPair>((FloatPair*)grid, f, D, W, status, s);
+}
+cudaError_t launch_fft_rows_pair(const void* grid, const FftParams& f, int D, const void* W, const void* U,
+                                 const void* decon, const int* row_exp, void* coeffs, const int* status,
+                                 cudaStream_t s) {
+  return launch_rows_t<FloatPair>((const FloatPair*)grid, f, D, W, U, decon, row_exp, coeffs, status, s);
+}
 cudaError_t launch_fft_rows_f32(const float* grid, const FftParams& f, int D, const void* W, const void* U,
                                 const void* decon, void* coeffs, const int* status, cudaStream_t s) {
-  return launch_rows_t<float>(grid, f, D, W, U, decon, coeffs, status, s);
+  return launch_rows_t<float>(grid, f, D, W, U, decon, nullptr, coeffs, status, s);
 }
 cudaError_t launch_fft_rows_f64(const double* grid, const FftParams& f, int D, const void* W, const void* U,
                                 const void* decon, void* coeffs, const int* status, cudaStream_t s) {
-  return launch_rows_t<double>(grid, f, D, W, U, decon, coeffs, status, s);
+  return launch_rows_t<double>(grid, f, D, W, U, decon, nullptr, coeffs, status, s);
 }
 
 }  // namespace mmgpu

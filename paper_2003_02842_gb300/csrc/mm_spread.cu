@@ -44,7 +44,7 @@ namespace mmgpu {
 // anywhere leaves every read in bounds.
 __global__ void k_bounds(const int64_t* __restrict__ off, const double* __restrict__ t, int D, int gsize,
                          int64_t max_events, double w0, double w1, int64_t Mr, Rescale* rs, int* status,
-                         int* __restrict__ order) {
+                         int* __restrict__ order, int* __restrict__ row_exp) {
   __shared__ double s_lo[8], s_hi[8];
   __shared__ int s_bad;
   pdl_wait();     // the previous call's kernels may still read the gate
@@ -57,8 +57,10 @@ __global__ void k_bounds(const int64_t* __restrict__ off, const double* __restri
   // 1) the offsets alone: non-decreasing from 0 up to at most max_events.
   //    Only when all of them hold is any event time read.
   int bad = 0;
-  for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x)
+  for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
     if (off[i + 1] < off[i]) bad = 1;
+    if (row_exp) row_exp[i] = 0;  // the prep kernel raises it
+  }
   if (threadIdx.x == 0 && (off[i0] < 0 || off[i1] > max_events || (g == 0 && off[0] != 0))) bad = 1;
   if (bad) atomicOr(&s_bad, 1);
   __syncthreads();
@@ -176,7 +178,8 @@ __global__ void k_bounds(const int64_t* __restrict__ off, const double* __restri
 }
 
 cudaError_t launch_bounds(const int64_t* off, const double* t, int D, int gsize, int64_t max_events, double w0,
-                          double w1, int64_t Mr, Rescale* rs, int* status, int* order, cudaStream_t s) {
+                          double w1, int64_t Mr, Rescale* rs, int* status, int* order, int* row_exp,
+                          cudaStream_t s) {
   const int G = (D + gsize - 1) / gsize;
   if (order && (G != 1 || D > kOrderMaxAssets)) return cudaErrorInvalidValue;
   if (G > 1) {
@@ -189,7 +192,7 @@ cudaError_t launch_bounds(const int64_t* off, const double* t, int D, int gsize,
   // k_group_scales
   const int nth = gsize <= 32 && !order ? 32 : 256;
   return launch_pdl(k_bounds, dim3(G), dim3(nth), 0, s, off, t, D, gsize, max_events, w0, w1, Mr, rs, status,
-                    order);
+                    order, row_exp);
 }
 
 // Per-problem fixed-point cell scales for the grid size of this call.
@@ -306,7 +309,9 @@ __device__ __forceinline__ double offset_pair(unsigned long long frac) {
   return __hiloint2double(__float_as_int(zh), __float_as_int(zl));
 }
 
-// PAIR (float64): the offset as the float pair of offset_pair in its 8 bytes.
+// PAIR (float64): the offset as the float pair of offset_pair in its 8 bytes, and
+// each asset's largest exponent field of a return into row_exp (its grid row, in
+// float pairs, is scaled by it).
 template <typename T, bool PAIR>
 __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(const int64_t* __restrict__ off, const double* __restrict__ t,
                                                        const double* __restrict__ logp,
@@ -314,7 +319,7 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(const int64_t* __restr
                                                        const GroupScale* __restrict__ gsc, int gsize,
                                                        const int* __restrict__ gate, int D, int64_t Mr,
                                                        int* __restrict__ rb0, T* __restrict__ rd,
-                                                       T* __restrict__ rv, int* status) {
+                                                       T* __restrict__ rv, int* __restrict__ row_exp, int* status) {
   static_assert(kPrepE == 4, "records are stored as 4-vectors");
   __shared__ UScale s_us;
   __shared__ UScaleF s_usf;
@@ -391,6 +396,7 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(const int64_t* __restr
   int b0v[kPrepE];
   T dv[kPrepE], vv[kPrepE];
   int lo = s_a0;
+  int ex_asset = -1, ex_top = 0;  // PAIR: the asset of the thread's records so far and their largest exponent
 #pragma unroll
   for (int j = 0; j < kPrepE; ++j) {
     const int64_t h = h0 + j;
@@ -450,6 +456,24 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(const int64_t* __restr
     dv[j] = cd;
     if (sizeof(T) == 8) vv[j] = (T)(pv[j + 1] - pv[j]);
     else vv[j] = (T)((ph[j + 1] - ph[j]) + (pl[j + 1] - pl[j]));
+    if (PAIR) {
+      if (lo != ex_asset && ex_asset >= 0) {
+        atomicMax(row_exp + ex_asset, ex_top);
+        ex_top = 0;
+      }
+      ex_asset = lo;
+      ex_top = max(ex_top, (__double2hiint((double)vv[j]) >> 20) & 0x7FF);
+    }
+  }
+  if (PAIR) {
+    // one update a warp when its threads' last records are of one asset
+    const int a0 = __shfl_sync(0xffffffffu, ex_asset, 0);
+    if (__all_sync(0xffffffffu, ex_asset == a0)) {
+      ex_top = __reduce_max_sync(0xffffffffu, ex_top);
+      if ((threadIdx.x & 31) == 0 && a0 >= 0) atomicMax(row_exp + a0, ex_top);
+    } else if (ex_asset >= 0) {
+      atomicMax(row_exp + ex_asset, ex_top);
+    }
   }
   if (h0 + kPrepE <= ntot) {
     // h0 is a multiple of 4 and the record arrays are the plan's own
@@ -476,13 +500,13 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(const int64_t* __restr
 template <typename T, bool PAIR>
 static cudaError_t launch_prep_t(const int64_t* off, const double* t, const double* logp, const Rescale* rs,
                                  const GroupScale* gsc, int gsize, int D, int64_t Mr, int64_t max_events, int* rb0,
-                                 T* rd, T* rv, int* status, cudaStream_t s) {
+                                 T* rd, T* rv, int* row_exp, int* status, cudaStream_t s) {
   if (max_events <= 0) return cudaSuccess;
   if ((((uintptr_t)rb0) | ((uintptr_t)rd) | ((uintptr_t)rv)) & 15) return cudaErrorMisalignedAddress;
   const int64_t per_block = (int64_t)kPrepThreads * kPrepE;
   const int64_t blocks = (max_events + per_block - 1) / per_block;
   return launch_pdl(k_prep<T, PAIR>, dim3((unsigned)blocks), dim3(kPrepThreads), 0, s, off, t, logp, rs, gsc, gsize,
-                    status + 1, D, Mr, rb0, rd, rv, status);
+                    status + 1, D, Mr, rb0, rd, rv, row_exp, status);
 }
 
 cudaError_t launch_prep_f32(const int64_t* off, const double* t, const double* logp, const Rescale* rs,
@@ -490,16 +514,16 @@ cudaError_t launch_prep_f32(const int64_t* off, const double* t, const double* l
                             int64_t Mr, int64_t max_events, int* rb0, void* rd, void* rv, int* status,
                             cudaStream_t s) {
   return launch_prep_t<float, false>(off, t, logp, rs, gsc, gsize, D, Mr, max_events, rb0, (float*)rd, (float*)rv,
-                                     status, s);
+                                     nullptr, status, s);
 }
 cudaError_t launch_prep_f64(const int64_t* off, const double* t, const double* logp, const Rescale* rs,
                             const GroupScale* gsc, int gsize, int D,
-                            int64_t Mr, int64_t max_events, bool pair, int* rb0, void* rd, void* rv, int* status,
+                            int64_t Mr, int64_t max_events, int* row_exp, int* rb0, void* rd, void* rv, int* status,
                             cudaStream_t s) {
   auto go = [&](auto fn) {
-    return fn(off, t, logp, rs, gsc, gsize, D, Mr, max_events, rb0, (double*)rd, (double*)rv, status, s);
+    return fn(off, t, logp, rs, gsc, gsize, D, Mr, max_events, rb0, (double*)rd, (double*)rv, row_exp, status, s);
   };
-  return pair ? go(launch_prep_t<double, true>) : go(launch_prep_t<double, false>);
+  return row_exp ? go(launch_prep_t<double, true>) : go(launch_prep_t<double, false>);
 }
 
 // ------------------------------------------------------------------ spread
@@ -936,8 +960,8 @@ cudaError_t launch_spread_poly(const int64_t* off, const int* rb0, const void* r
 // 100 float32 operations instead: the even and odd polynomials of PairPoly (two
 // taps each) by Horner's rule in float pairs h + l, the leading coefficients of
 // which need one float only; the product with the return; and an accumulation
-// that stays exact in three int32 words, as k_spread_poly's in two. Now 77 us and
-// 97 us.
+// that stays exact in three int32 words, as k_spread_poly's in two. Now 75 us and
+// 97 us. The grid leaves as float pairs, which the FFT passes keep.
 //
 // Error: against the kernel in 64 bits a tap is off by at most 7e-15 of the peak
 // (8e-16 rms; measured for the three kernels at tol 1e-12), so the path is taken
@@ -953,9 +977,6 @@ cudaError_t launch_spread_poly(const int64_t* off, const int* rb0, const void* r
 // records of a staged chunk keeps a chunk's mid and lo sums below 2^31; between
 // chunks lo carries into mid and mid into hi. The quantum is 2^-(eh + 2k) (V 2^-60
 // for tiles of up to 511 records, V 2^-53 at 30,000), and no sum rounds.
-struct FloatPair {
-  float h, l;
-};
 // c + r y
 __device__ __forceinline__ FloatPair pair_step(FloatPair r, FloatPair y, float ch, float cl) {
   const float p = __fmul_rn(r.h, y.h), e = __fmaf_rn(r.h, y.h, -p);
@@ -998,7 +1019,8 @@ __global__ void __launch_bounds__(kSpreadThreads, 4) k_spread_pair(const int64_t
                                                                const double* __restrict__ rv,
                                                                const int* __restrict__ gate, SpreadParams p,
                                                                const __grid_constant__ PairPoly poly,
-                                                               double* __restrict__ grid) {
+                                                               const int* __restrict__ row_exp,
+                                                               FloatPair* __restrict__ grid) {
   constexpr int EC = kPairChunk;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* ev_d = reinterpret_cast<double*>(smem_raw);
@@ -1105,35 +1127,33 @@ __global__ void __launch_bounds__(kSpreadThreads, 4) k_spread_pair(const int64_t
     }
   }
   __syncthreads();
-  // cells: (hi 2^k + mid) 2^-(eh + k) + lo 2^-(eh + 2k), each term built as a
-  // float64 with its integer in the low mantissa bits (no conversions)
-  double* g = grid + (int64_t)a * p.Mr + L;
-  const int xa = 0x433 - (eh + kk), xl = 0x433 - (eh + 2 * kk);
-  const bool plain = xl >= 1 && xa <= 0x7FE && top != 0x7FF;
-  const long long ba = ((long long)xa << 52) + (1ll << 51), bl = ((long long)xl << 52) + (1ll << 51);
+  // cells: (hi + (mid + lo 2^-k) 2^-k) 2^-eh as float pairs, scaled by the row's
+  // largest exponent, from the exact integers: the leading 24 bits of A = hi 2^k +
+  // mid, then the rest and lo
+  FloatPair* g = grid + (int64_t)a * p.Mr + L;
+  const int sa = -(eh + kk) - (row_exp[a] - 1022);  // returns of the row scaled below 1
+  const bool plain = sa >= -80;
+  const float unit = plain ? __int_as_float((127 + sa) << 23) : 1.0f;
   for (int c = threadIdx.x; c < Tlen; c += kSpreadThreads) {
     const long long A = ((long long)tile[c] << kk) + tile[c + tpad];
-    const int lo = tile[c + 2 * tpad];
-    if (plain) {
-      g[c] = (__longlong_as_double(ba + A) - __longlong_as_double(ba)) +
-             (__longlong_as_double(bl + lo) - __longlong_as_double(bl));
-    } else if (top == 0x7FF) {
-      g[c] = __longlong_as_double(0x7ff8000000000000ll);  // an infinite return
-    } else {
-      g[c] = ldexp((double)A + ldexp((double)lo, -kk), -(eh + kk));
-    }
+    const float below = (float)tile[c + 2 * tpad] * __int_as_float((127 - kk) << 23);
+    const float h = (float)A;  // rounded to 24 bits: A - h is exact in 63 bits and has few left
+    const float l = (float)(A - (long long)h) + below;
+    if (plain) g[c] = FloatPair(h * unit, l * unit);
+    else g[c] = FloatPair(top == 0x7FF ? __int_as_float(0x7fc00000) : ldexpf(h, sa), ldexpf(l, sa));
   }
 }
 
 cudaError_t launch_spread_pair(const int64_t* off, const int* rb0, const void* rd, const void* rv,
-                               const SpreadParams& p, const PairPoly& poly, double* grid, const int* status,
+                               const SpreadParams& p, const PairPoly& poly, const int* row_exp, void* grid,
+                               const int* status,
                                cudaStream_t s) {
   if (p.tile > spread_max_tile(true)) return cudaErrorInvalidValue;
   const size_t smem = (size_t)kPairChunk * (2 * sizeof(double) + sizeof(int)) + 3 * (((size_t)p.tile + 3) / 4 * 16);
   const cudaError_t e = cudaFuncSetAttribute(k_spread_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   return launch_pdl(k_spread_pair, dim3(p.ntiles, p.D), dim3(kSpreadThreads), smem, s, off, rb0, (const double*)rd,
-                    (const double*)rv, (const int*)(status + 1), p, poly, grid);
+                    (const double*)rv, (const int*)(status + 1), p, poly, row_exp, (FloatPair*)grid);
 }
 
 template <typename T, int K>
