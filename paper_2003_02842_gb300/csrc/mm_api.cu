@@ -386,6 +386,8 @@ struct mm_plan_s {
   int w_N = -1, w_basis = -1;
   GramParams gram{};
   KernelPoly poly{};
+  double poly_err = -1.0;  // its fit error (< 0: not fitted yet) and the constants it was fitted for
+  double poly_t1 = 0.0, poly_b = 0.0;
   bool poly_ok = false;   // float32 spreading with polynomial taps and integer accumulation
   PairPoly pair_poly{};
   bool pair_ok = false;   // FP64 spreading in float pairs
@@ -575,9 +577,17 @@ mm_status configure(mm_plan p, int N) {
   p->tau = kPi * lam / ((double)Mr * (double)Mr);
   p->poly_ok = false;
   if (!p->fp64 && s.algo == 0 && p->tune_poly != 0 && spread_poly_supported(s.khi - s.klo + 1)) {
-    // the fit must stay far below the NUFFT tolerance and near float32 rounding
-    const double err = fit_kernel_poly(s, &p->poly);
-    p->poly_ok = err <= std::max(3.0e-7, 0.1 * p->desc.tol);
+    // the fit must stay far below the NUFFT tolerance and near float32 rounding.
+    // It depends on the cutoff through sigma alone (Gaussian, Kaiser-Bessel; the
+    // ES taps not at all) and costs some 70 us of host time, more than the rest of
+    // a serving request's set-up, so it is kept while its constants are.
+    if (!(p->poly_err >= 0.0 && p->poly_t1 == s.g_t1 && p->poly_b == s.kb_b) &&
+        !(p->poly_err >= 0.0 && s.kernel == MM_KERNEL_ES)) {
+      p->poly_err = fit_kernel_poly(s, &p->poly);
+      p->poly_t1 = s.g_t1;
+      p->poly_b = s.kb_b;
+    }
+    p->poly_ok = p->poly_err <= std::max(3.0e-7, 0.1 * p->desc.tol);
   }
   // FP64: taps in float pairs where their error (at most 1e-14) and the fit's
   // are 50 times below the NUFFT tolerance; float64 throughout otherwise
@@ -1580,6 +1590,33 @@ mm_status plan_set_active_assets(mm_plan p, int D) {
 }
 
 int* plan_status_word(mm_plan p) { return p ? p->status : nullptr; }
+
+mm_status plan_nyquist_enqueue(mm_plan p, const int64_t* off, const double* t, double t0, double t1, int* h3,
+                               cudaStream_t st) {
+  const mm_status r = check_plan(p);
+  if (r != MM_OK) return r;
+  if (!(isfinite(t0) && isfinite(t1))) return MM_ERR_INVALID_ARG;
+  p->last = st;
+  {
+    StageScope sc(p, MM_STAGE_PREP, st);
+    MM_CUDA(launch_bounds(off, t, p->D, p->gsize, p->desc.max_events, t0, t1, 0, p->bounds, p->status, nullptr,
+                          nullptr, st));
+  }
+  {
+    StageScope sc(p, MM_STAGE_PREP, st, 2);
+    MM_CUDA(launch_min_gap(off, t, p->D, p->bounds, p->gapbits, p->status + 2, p->status, st));
+  }
+  MM_CUDA(cudaMemcpyAsync(h3, p->status, 3 * sizeof(int), cudaMemcpyDeviceToHost, st));
+  return MM_OK;
+}
+
+mm_status plan_nyquist_result(mm_plan p, const int* h3, int32_t* N) {
+  if (h3[1]) return h3[0] ? flags_to_status(h3[0]) : MM_ERR_INVALID_ARG;
+  if (h3[2] < 0) return MM_ERR_CUTOFF;
+  if (p->desc.basis == MM_BASIS_FEJER && h3[2] < 1) return MM_ERR_CUTOFF;
+  *N = h3[2];
+  return MM_OK;
+}
 
 mm_status plan_flags_to_status(int flags) { return flags_to_status(flags); }
 

@@ -322,6 +322,12 @@ int epps_max_assets();
 mm_status plan_create_no_staging(const mm_plan_desc* desc, mm_plan* out);  // no host-buffer entry staging
 mm_status plan_set_active_assets(mm_plan p, int D);
 int* plan_status_word(mm_plan p);
+// The window's Nyquist cutoff in two halves: kernels and an asynchronous copy of
+// three status words to h3 (pinned), then, when the stream has passed it, the
+// cutoff or the error mm_nyquist's coefficients would give.
+mm_status plan_nyquist_enqueue(mm_plan p, const int64_t* off, const double* t, double t0, double t1, int* h3,
+                               cudaStream_t st);
+mm_status plan_nyquist_result(mm_plan p, const int* h3, int32_t* N);
 mm_status plan_flags_to_status(int flags);
 // The cutoff sweep of a batch (mm_epps.cu): G problems of Dg assets, splits
 // CTAs per problem (epps_splits) with their partial sums and zeroed arrival
