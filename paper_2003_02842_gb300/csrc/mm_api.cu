@@ -333,7 +333,7 @@ struct mm_plan_s {
   Rescale* bounds = nullptr;       // one per problem
   void* gscale = nullptr;          // per-problem cell scales (batched form)
   int* status = nullptr;  // [0] sticky flags, [1] gate, [2] Nyquist N
-  unsigned long long* gapbits = nullptr;
+  unsigned long long* gapbits = nullptr;  // [D] smallest gaps and an arrival counter (launch_min_gap)
   void* wsq = nullptr;
   void* partial = nullptr;        // FP64 path: per-split partial tiles
   float* acc[2] = {nullptr, nullptr};  // mixed path: FP32 accumulators, used alternately
@@ -789,8 +789,9 @@ mm_status coeffs_impl(mm_plan p, const int64_t* off, const double* t, const doub
   if (N <= 0 && p->G > 1) return MM_ERR_CUTOFF;  // a batch sweeps given cutoffs
   if (N <= 0) {
     {
-      StageScope sc(p, MM_STAGE_PREP, st, 2);
-      MM_CUDA(launch_min_gap(off, t, D, p->bounds, p->gapbits, p->status + 2, p->status, st));
+      StageScope sc(p, MM_STAGE_PREP, st);
+      MM_CUDA(launch_min_gap(off, t, D, p->desc.max_events / p->desc.D, p->bounds, p->gapbits, p->status + 2,
+                             p->status, st));
     }
     int hv[3];
     MM_CUDA(cudaMemcpyAsync(hv, p->status, sizeof(hv), cudaMemcpyDeviceToHost, st));
@@ -1112,7 +1113,7 @@ mm_status plan_create_impl(const mm_plan_desc* desc, int gsize, bool batch, mm_p
   if (!batch && D <= (size_t)kOrderMaxAssets) A((void**)&p->asset_order, std::max<size_t>(D, 1) * sizeof(int));
   if (p->G > 1) A(&p->gscale, (size_t)p->G * group_scale_bytes());
   A((void**)&p->status, 4 * sizeof(int));
-  A((void**)&p->gapbits, sizeof(unsigned long long));
+  A((void**)&p->gapbits, (size_t)(D + 1) * sizeof(unsigned long long));
   A(&p->wsq, Np1 * p->rs);
   if (!batch) {
     GramParams g = gram_params(p, d.N_max);
@@ -1142,6 +1143,8 @@ mm_status plan_create_impl(const mm_plan_desc* desc, int gsize, bool batch, mm_p
   }
   if (r == MM_OK) {
     if (cudaMemset(p->status, 0, 4 * sizeof(int)) != cudaSuccess) r = MM_ERR_CUDA;
+    if (r == MM_OK && cudaMemset(p->gapbits, 0, (size_t)(D + 1) * sizeof(unsigned long long)) != cudaSuccess)
+      r = MM_ERR_CUDA;
     if (p->gram_done && cudaMemset(p->gram_done, 0, sizeof(int)) != cudaSuccess) r = MM_ERR_CUDA;
   }
   if (r == MM_OK && d.kernel == MM_KERNEL_ES) {
@@ -1469,8 +1472,9 @@ mm_status mm_nyquist(mm_plan p, const int64_t* d_offsets, const double* d_t, dou
                           nullptr, nullptr, st));
   }
   {
-    StageScope sc(p, MM_STAGE_PREP, st, 2);
-    MM_CUDA(launch_min_gap(d_offsets, d_t, p->D, p->bounds, p->gapbits, p->status + 2, p->status, st));
+    StageScope sc(p, MM_STAGE_PREP, st);
+    MM_CUDA(launch_min_gap(d_offsets, d_t, p->D, p->desc.max_events / p->desc.D, p->bounds, p->gapbits, p->status + 2,
+                           p->status, st));
   }
   int hv[3];
   MM_CUDA(cudaMemcpyAsync(hv, p->status, sizeof(hv), cudaMemcpyDeviceToHost, st));
@@ -1603,8 +1607,9 @@ mm_status plan_nyquist_enqueue(mm_plan p, const int64_t* off, const double* t, d
                           nullptr, st));
   }
   {
-    StageScope sc(p, MM_STAGE_PREP, st, 2);
-    MM_CUDA(launch_min_gap(off, t, p->D, p->bounds, p->gapbits, p->status + 2, p->status, st));
+    StageScope sc(p, MM_STAGE_PREP, st);
+    MM_CUDA(launch_min_gap(off, t, p->D, p->desc.max_events / p->desc.D, p->bounds, p->gapbits, p->status + 2,
+                           p->status, st));
   }
   MM_CUDA(cudaMemcpyAsync(h3, p->status, 3 * sizeof(int), cudaMemcpyDeviceToHost, st));
   return MM_OK;

@@ -223,8 +223,8 @@ cudaError_t launch_bounds(const int64_t* off, const double* t, int D, int gsize,
 cudaError_t launch_group_scales(const Rescale* rs, int G, int64_t Mr, GroupScale* out, const int* status,
                                 cudaStream_t s);
 size_t group_scale_bytes();
-cudaError_t launch_min_gap(const int64_t* off, const double* t, int D, const Rescale* rs,
-                           unsigned long long* gapbits, int* nyq, int* status, cudaStream_t s);
+cudaError_t launch_min_gap(const int64_t* off, const double* t, int D, int64_t asset_events, const Rescale* rs,
+                           unsigned long long* gap, int* nyq, int* status, cudaStream_t s);
 cudaError_t launch_prep_f32(const int64_t* off, const double* t, const double* logp, const Rescale* rs,
                             const GroupScale* gsc, int gsize, int D, int64_t Mr, int64_t max_events, int* rb0,
                             void* rd, void* rv, int* status, cudaStream_t s);
