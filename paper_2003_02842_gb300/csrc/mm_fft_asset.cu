@@ -708,7 +708,11 @@ __device__ __forceinline__ void pair_finish(const AssetFft& f, Cplx<float>* s, c
 // latency counts: the row is fetched straight into the first pass's registers
 // (a copy into digit-reversed slots first cost 5 of 22.6 us), the slots are padded
 // against bank conflicts, and a thread unpacks two modes from the same values.
-// 5120 rows of 28,800 points: 1595 us before, 1059 us with these.
+// 5120 rows of 28,800 points: 1595 us before, 1059 us with these. While a row is
+// worked on, the one that follows it on these SMs is brought from memory into L2
+// (kPairAhead rows on, half by each CTA: no registers, no waiting): 1059 -> 1045 us.
+constexpr uint32_t kPrefetchChunk = 4096;
+constexpr int kPairAhead = 76;  // pairs the chip holds (152 SMs, a CTA each)
 template <int NTH, int MAXR>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTH, 1)
     k_fft_asset_pair(const float* __restrict__ grid, AssetFft f, const Cplx<float>* __restrict__ W,
@@ -737,6 +741,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTH, 1)
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
   const Cplx<float>* z = reinterpret_cast<const Cplx<float>*>(grid) + (size_t)a * f.n + c;
+  if (threadIdx.x < 32 && a + kPairAhead < (int)gridDim.y) {
+    // 16-byte aligned chunks of this CTA's half of the row (n is even)
+    const uint32_t all = (uint32_t)f.n * 8u, mid = (all / 2) & ~15u;
+    const uint32_t b0 = c == 0 ? 0u : mid, b1 = c == 0 ? mid : all;
+    const unsigned char* src = reinterpret_cast<const unsigned char*>(grid) + (size_t)(a + kPairAhead) * all;
+    for (uint32_t o = b0 + threadIdx.x * kPrefetchChunk; o < b1; o += 32 * kPrefetchChunk) {
+      const uint32_t cb = b1 - o < kPrefetchChunk ? b1 - o : kPrefetchChunk;
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src + o), "r"(cb) : "memory");
+    }
+  }
   // a position below m_1 times q_0 is padded by q_0, the first digit of u
   with_radix<MAXR>(pick(f.rad, f.npass - 1), [&](auto r) {
     fft_first_pass<decltype(r)::value>(s, z, L, NTH, [&](int u) {
