@@ -43,10 +43,14 @@ constexpr int kFftPer = 16;
 // the float64 pipe and read their tables where they use them: two blocks an SM.
 template <typename T>
 constexpr bool kTablesEarly = !std::is_same<T, FloatPair>::value;
+// Two blocks an SM but in float64 (with one block asked for, ptxas gave the float32
+// passes up to 152 registers and one block: 61 -> 103 us at 64 rows of 80,000 points).
+template <typename T>
+constexpr int kFftBlocks = std::is_same<T, double>::value ? 1 : 2;
 
 template <typename T>
-__global__ void __launch_bounds__(kFftThreads, kTablesEarly<T> ? 1 : 2) k_fft_cols(Cplx<T>* __restrict__ z, FftParams f,
-                                                          const Cplx<T>* __restrict__ W, const int* __restrict__ gate) {
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks<T>) k_fft_cols(Cplx<T>* __restrict__ z, FftParams f,
+                                                                         const Cplx<T>* __restrict__ W, const int* __restrict__ gate) {
   if (*gate) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int P = f.P, Q = f.Q, lgB = f.lg_cols, B = 1 << lgB;
@@ -125,7 +129,7 @@ template <> struct Coef<FloatPair> { using type = double; };
 
 // ------------------------------------------------------------ pass 2
 template <typename T>
-__global__ void __launch_bounds__(kFftThreads, kTablesEarly<T> ? 1 : 2) k_fft_rows(const Cplx<T>* __restrict__ z, FftParams f,
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks<T>) k_fft_rows(const Cplx<T>* __restrict__ z, FftParams f,
                                                           const Cplx<T>* __restrict__ W, const Cplx<T>* __restrict__ U,
                                                           const T* __restrict__ decon,
                                                           const int* __restrict__ row_exp,
