@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kJacobiThreads) k_psd_jacobi(const double* __r
   W* A = reinterpret_cast<W*>(rot + 2 * nh);                // two copies of four planes
   __shared__ double s_red[kJacobiThreads / 32];
   __shared__ int s_neg;
-  const int tid = threadIdx.x, nth = kJacobiThreads;
+  const int tid = threadIdx.x, nth = (int)blockDim.x;
   auto block_red = [&](double v, bool max) -> double {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -771,7 +771,10 @@ static cudaError_t launch_psd_one_cta(double* sig, double* A, W* V, int D, int* 
   auto* info = reinterpret_cast<PsdInfo*>(sync);
   cudaError_t e = cudaFuncSetAttribute(k_psd_jacobi<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_psd_jacobi<W><<<1, kJacobiThreads, smem, s>>>(sig, D, lg, A, info, clipped);
+  // a thread per block where that many fit: barriers and sums over idle warps are
+  // a tenth of the time at three assets
+  const int threads = std::min(kJacobiThreads, ((nh + 31) & ~31) + ((fold_size(nh) + 31) & ~31));
+  k_psd_jacobi<W><<<1, threads, smem, s>>>(sig, D, lg, A, info, clipped);
   switch ((m / 2 + 31) / 32) {
     case 1: k_psd_vectors<W, 1><<<D, 32, 0, s>>>(lg, info, D, V); break;
     case 2: k_psd_vectors<W, 2><<<D, 32, 0, s>>>(lg, info, D, V); break;
