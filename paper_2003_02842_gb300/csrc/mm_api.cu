@@ -547,8 +547,11 @@ mm_status configure(mm_plan p, int N) {
   // default tile: the largest (measured on GB300 with the polynomial scatter:
   // 4096 cells beat 2048 on both the block and the batched workloads), or half
   // of it where the assets' mean density says that tiles will be dense (a cell
-  // then takes two words, and one tile fills the shared memory of 4096 words)
-  const bool dense = !p->fp64 && 2.0 * (double)p->desc.max_events > (double)Mr * p->desc.D;
+  // then takes two words, and one tile fills the shared memory of 4096 words):
+  // from a quarter of a record a cell, where the busiest assets' stencils hold
+  // more than kOneRun (238 assets of 0.28 a cell: 29.5 us in full tiles, 14.3 in halves)
+  const bool dense = !p->fp64 && 4.0 * (double)p->desc.max_events > (double)Mr * p->desc.D;
+  s.dense = dense;
   int tile = p->desc.spread_tile > 0 ? std::min(p->desc.spread_tile, tmax) : (dense ? tmax / 2 : tmax);
   if (p->tune_tile > 0) tile = std::min(p->tune_tile, tmax);
   if (Mr <= (int64_t)tile) {
@@ -820,13 +823,13 @@ mm_status coeffs_impl(mm_plan p, const int64_t* off, const double* t, const doub
     }
     {
       StageScope sc(p, MM_STAGE_PREP, st);
+      const bool spare = p->G == 1 && D < p->desc.D;
       if (p->fp64)
-        MM_CUDA(launch_prep_f64(off, t, logp, p->bounds, gsc, p->gsize, D, p->Mr, p->desc.max_events,
-                                p->pair_ok ? p->row_exp : nullptr,
-                                p->rec_b0, p->rec_d, p->rec_v, p->status, st));
+        MM_CUDA(launch_prep_f64(off, t, logp, p->bounds, gsc, p->gsize, D, p->Mr, p->desc.max_events, spare,
+                                p->pair_ok ? p->row_exp : nullptr, p->rec_b0, p->rec_d, p->rec_v, p->status, st));
       else
-        MM_CUDA(launch_prep_f32(off, t, logp, p->bounds, gsc, p->gsize, D, p->Mr, p->desc.max_events, p->rec_b0,
-                                p->rec_d, p->rec_v, p->status, st));
+        MM_CUDA(launch_prep_f32(off, t, logp, p->bounds, gsc, p->gsize, D, p->Mr, p->desc.max_events, spare,
+                                p->rec_b0, p->rec_d, p->rec_v, p->status, st));
     }
     if (p->res_sub > 0) {
       StageScope sc(p, MM_STAGE_FUSED, st);

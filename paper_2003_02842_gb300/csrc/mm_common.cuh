@@ -107,6 +107,7 @@ struct SpreadParams {
   double kb_inv_phi0;// KB: 1 / phi(0) (kernel normalised to peak 1)
   int64_t max_events;
   int64_t asset_events;  // capacity per asset of the plan (max_events over its assets)
+  int dense;             // float32: tiles are likely dense at that density (configure)
   // spreading tiles are dispatched asset by asset in this order (the assets
   // ranked by event count, heaviest first, written by k_bounds), or in index
   // order when null
@@ -150,8 +151,7 @@ struct Rescale {
   unsigned long long S;      // cell scale of grid scale_Mr: 64-bit multiplier, in [2^63, 2^64)
   int F;                     // fractional bits of the time fixed point
   int sh;                    // right shift of the 128-bit product, 0..127
-  float s_hi, s_lo;          // the float-pair cell scale of the same grid
-  long long scale_Mr;        // grid size the cell scales belong to (0: not computed)
+  long long scale_Mr;        // grid size the cell scale belongs to (0: not computed)
 };
 constexpr int kUFrac = 40;   // fractional bits of u_fix
 
@@ -225,14 +225,15 @@ cudaError_t launch_group_scales(const Rescale* rs, int G, int64_t Mr, GroupScale
 size_t group_scale_bytes();
 cudaError_t launch_min_gap(const int64_t* off, const double* t, int D, int64_t asset_events, const Rescale* rs,
                            unsigned long long* gap, int* nyq, int* status, cudaStream_t s);
+// spare: the call's events may be far fewer than max_events (k_prep)
 cudaError_t launch_prep_f32(const int64_t* off, const double* t, const double* logp, const Rescale* rs,
-                            const GroupScale* gsc, int gsize, int D, int64_t Mr, int64_t max_events, int* rb0,
-                            void* rd, void* rv, int* status, cudaStream_t s);
+                            const GroupScale* gsc, int gsize, int D, int64_t Mr, int64_t max_events, bool spare,
+                            int* rb0, void* rd, void* rv, int* status, cudaStream_t s);
 // row_exp != NULL: records for launch_spread_pair, the offsets d as float pairs
 // z = d - 1/2, and each asset's largest exponent field of a return
 cudaError_t launch_prep_f64(const int64_t* off, const double* t, const double* logp, const Rescale* rs,
-                            const GroupScale* gsc, int gsize, int D, int64_t Mr, int64_t max_events, int* row_exp,
-                            int* rb0, void* rd, void* rv, int* status, cudaStream_t s);
+                            const GroupScale* gsc, int gsize, int D, int64_t Mr, int64_t max_events, bool spare,
+                            int* row_exp, int* rb0, void* rd, void* rv, int* status, cudaStream_t s);
 cudaError_t launch_spread_f32(const int64_t* off, const int* rb0, const void* rd, const void* rv,
                               const SpreadParams& p, float* grid, const int* status, cudaStream_t s);
 // float32 scatter with the polynomial taps and int32 fixed-point shared

@@ -30,7 +30,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
   __shared__ int s_row[64], s_partner[64];
   __shared__ int s_nrows, s_flags;
   __shared__ UScale s_us;
-  __shared__ UScaleF s_usf;
   if (*gate) return;  // uniform: the whole block leaves
   const int P = f.P, Q = f.Q;
   const int Mr = (int)sp.Mr;
@@ -55,8 +54,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
   for (int j = threadIdx.x; j < Q; j += kFusedThreads) twQ[j] = W[j * P];
   if (threadIdx.x == 0) {
     s_flags = 0;
-    if (sizeof(T) == 8) s_us = make_uscale(rs, sp.Mr);
-    else s_usf = make_uscale_f(rs, sp.Mr);
+    s_us = make_uscale(rs, sp.Mr);
   }
   __syncthreads();
 
@@ -76,17 +74,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
       continue;
     }
     const long long dt = to_fix(th, rs.F) - rs.t0_fix;
-    int b0;
-    T d;
-    if (sizeof(T) == 8) {
-      const unsigned long long uf = u_fix_of(th, rs.t0_fix, rs.F, s_us);
-      b0 = (int)(uf >> kUFrac);
-      d = frac_to<T>(uf & ((1ull << kUFrac) - 1));
-    } else {
-      float fd;
-      cell_f32(dt, s_usf, b0, fd);
-      d = (T)fd;
-    }
+    const unsigned long long uf = u_fix_of(dt, s_us);
+    const int b0 = (int)(uf >> kUFrac);
+    const T d = frac_to<T>(uf & ((1ull << kUFrac) - 1));
     if (dt < 0 || b0 > Mr || (b0 == Mr && d > (T)0)) {
       flags |= ST_OUT_OF_WINDOW;
       continue;

@@ -161,13 +161,10 @@ __global__ void k_bounds(const int64_t* __restrict__ off, const double* __restri
       r.F = 62 - (ex + 1);                   // |t_fix| < 2^61
       r.t0_fix = to_fix(t0, r.F);
       if (Mr > 0) {
-        // the cell scales of this call's grid, once (float64 is slow here)
+        // the cell scale of this call's grid, once (float64 is slow here)
         const UScale us = make_uscale(r, Mr);
-        const UScaleF usf = make_uscale_f(r, Mr);
         r.S = us.S;
         r.sh = us.sh;
-        r.s_hi = usf.s_hi;
-        r.s_lo = usf.s_lo;
         r.scale_Mr = Mr;
       }
     }
@@ -203,7 +200,6 @@ __global__ void k_group_scales(const Rescale* __restrict__ rs, int G, int64_t Mr
   const Rescale r = rs[g];
   GroupScale q;
   q.us = make_uscale(r, Mr);
-  q.usf = make_uscale_f(r, Mr);
   q.t0_fix = r.t0_fix;
   q.F = r.F;
   out[g] = q;
@@ -322,11 +318,25 @@ constexpr int kSpreadThreads = 256;
 // last event of an asset carries no return and its record is never read
 // (it holds kNoCell or is left as it was).
 //
+// Bound by the integer pipe (51 % of its rate, and 70 % of the SMs' time at 1.03
+// waves of the former 256-thread blocks): the cell and its offset of both paths come
+// from one 64 x 64 -> 128-bit product (float32 offsets rounded to 2^-24 of a cell;
+// a float-pair product took twice the instructions), the end of the asset is kept
+// as a count instead of read for each event, a problem's scale is read once per
+// asset of a thread, whole stretches come by 16-byte loads. 128 threads leave 56
+// registers at nine blocks an SM, without the spills of 48. 9.2e6 events in 512
+// problems: 146 -> 120 us; 100 assets of some 7,700: 16.4 -> 14.4 us.
+//
 // Each thread takes kPrepE consecutive events: it loads kPrepE + 1 times and
 // log-prices, orders, checks and splits each value once (every value but the
 // last serves two returns), and writes its records with vector stores.
 constexpr int kPrepE = 4;
-constexpr int kPrepThreads = 256;
+constexpr int kPrepThreads = 128;
+// SPARE: a call for fewer assets than the plan's, whose grid by the plan's capacity
+// would be mostly empty blocks (a server's requests: 34 -> 29.6 us each): two
+// waves of blocks at most and a loop. Where the capacity is the call's own size the
+// loop costs more than it gives (16.4 -> 19.2 us at 100 assets).
+constexpr int64_t kPrepSpareBlocks = 152 * 9 * 2;
 
 template <typename T> struct Rec4;
 template <> struct Rec4<float> {
@@ -355,17 +365,14 @@ __device__ __forceinline__ double offset_pair(unsigned long long frac) {
 // PAIR (float64): the offset as the float pair of offset_pair in its 8 bytes, and
 // each asset's largest exponent field of a return into row_exp (its grid row, in
 // float pairs, is scaled by it).
-template <typename T, bool PAIR>
-__global__ void __launch_bounds__(kPrepThreads, 5) k_prep(const int64_t* __restrict__ off, const double* __restrict__ t,
-                                                       const double* __restrict__ logp,
-                                                       const Rescale* __restrict__ rsp,
-                                                       const GroupScale* __restrict__ gsc, int gsize,
-                                                       const int* __restrict__ gate, int D, int64_t Mr,
-                                                       int* __restrict__ rb0, T* __restrict__ rd,
-                                                       T* __restrict__ rv, int* __restrict__ row_exp, int* status) {
+template <typename T, bool PAIR, bool SPARE>
+__global__ void __launch_bounds__(kPrepThreads, 9)
+    k_prep(const int64_t* __restrict__ off, const double* __restrict__ t, const double* __restrict__ logp,
+           const Rescale* __restrict__ rsp, const GroupScale* __restrict__ gsc, int gsize,
+           const int* __restrict__ gate, int D, int64_t Mr, int* __restrict__ rb0, T* __restrict__ rd,
+           T* __restrict__ rv, int* __restrict__ row_exp, int* status) {
   static_assert(kPrepE == 4, "records are stored as 4-vectors");
   __shared__ UScale s_us;
-  __shared__ UScaleF s_usf;
   __shared__ int s_flags;
   __shared__ int s_a0;
   // one round of loads: the gate, the event count and the call's rescaling
@@ -379,192 +386,189 @@ __global__ void __launch_bounds__(kPrepThreads, 5) k_prep(const int64_t* __restr
   if (!gsc) rs0 = *rsp;
   if (gated) return;  // uniform
   const bool scales = gsc || rs0.scale_Mr == Mr;  // uniform
-  const int64_t hb = (int64_t)blockIdx.x * (kPrepThreads * kPrepE);
-  const int64_t h0 = hb + (int64_t)threadIdx.x * kPrepE;
-  double tv[kPrepE + 1], pv[kPrepE + 1];
+  const bool vec = ((reinterpret_cast<uintptr_t>(t) | reinterpret_cast<uintptr_t>(logp)) & 15) == 0;
+  for (int64_t hb = (int64_t)blockIdx.x * (kPrepThreads * kPrepE); hb < ntot;
+       hb += (int64_t)gridDim.x * (kPrepThreads * kPrepE)) {
+    const int64_t h0 = hb + (int64_t)threadIdx.x * kPrepE;
+    double tv[kPrepE + 1], pv[kPrepE + 1];
+    if (vec && h0 + kPrepE < ntot) {
+      // 16-byte loads (h0 is a multiple of 4)
+      const double2* t2 = reinterpret_cast<const double2*>(t + h0);
+      const double2* p2 = reinterpret_cast<const double2*>(logp + h0);
+      const double2 ta = __ldg(t2), tb = __ldg(t2 + 1), pa = __ldg(p2), pb = __ldg(p2 + 1);
+      tv[0] = ta.x, tv[1] = ta.y, tv[2] = tb.x, tv[3] = tb.y, tv[4] = __ldg(t + h0 + 4);
+      pv[0] = pa.x, pv[1] = pa.y, pv[2] = pb.x, pv[3] = pb.y, pv[4] = __ldg(logp + h0 + 4);
+    } else {
 #pragma unroll
-  for (int j = 0; j <= kPrepE; ++j) {
-    tv[j] = 0.0;
-    pv[j] = 0.0;
-    if (h0 + j < ntot) {
-      tv[j] = t[h0 + j];
-      pv[j] = logp[h0 + j];
-    }
-  }
-  if (threadIdx.x == 0) {
-    if (!scales) {
-      if (sizeof(T) == 8) s_us = make_uscale(rs0, Mr);
-      else s_usf = make_uscale_f(rs0, Mr);
-    }
-    s_flags = 0;
-  }
-  // asset of the block's first event (a 32-ary search by warp 0, a couple of
-  // dependent loads), then each thread walks forward to its own events' assets
-  if (threadIdx.x < 32) {
-    const int64_t hs = min(hb, ntot > 0 ? ntot - 1 : 0);
-    // first index in [1, D] with off[idx] > hs (D when none): the asset is idx - 1
-    const int lane = threadIdx.x;
-    int64_t lo = 1, hi = D;
-    for (int it = 0; it < 16 && hi > lo; ++it) {
-      const int64_t len = hi - lo;
-      const int64_t stride = (len + 31) / 32;
-      const int64_t o = (int64_t)lane * stride;
-      const bool below = o < len && off[lo + o] <= hs;
-      const int cnt = __popc(__ballot_sync(0xffffffffu, below));
-      if (cnt == 0) {
-        hi = lo;
-      } else {
-        const int64_t nlo = lo + (int64_t)(cnt - 1) * stride + 1;
-        const int64_t nhi = min(lo + (int64_t)cnt * stride, hi);
-        lo = min(nlo, nhi);
-        hi = nhi;
+      for (int j = 0; j <= kPrepE; ++j) {
+        tv[j] = 0.0;
+        pv[j] = 0.0;
+        if (h0 + j < ntot) {
+          tv[j] = t[h0 + j];
+          pv[j] = logp[h0 + j];
+        }
       }
     }
-    if (lane == 0) s_a0 = (int)lo - 1;
-  }
-  // per value, once: order key, finiteness and (float32 path) the exact
-  // hi + lo split of the log-price
-  long long key[kPrepE + 1];
-  bool fin_t[kPrepE + 1], fin_p[kPrepE + 1];
-  float ph[kPrepE + 1], pl[kPrepE + 1];
-#pragma unroll
-  for (int j = 0; j <= kPrepE; ++j) {
-    key[j] = order_key(tv[j]);
-    fin_t[j] = finite_bits(tv[j]);
-    fin_p[j] = finite_bits(pv[j]);
-    if (sizeof(T) == 4) split_f64(pv[j], ph[j], pl[j]);
-  }
-  __syncthreads();
-  int flags = 0;
-  int b0v[kPrepE];
-  T dv[kPrepE], vv[kPrepE];
-  int lo = s_a0;
-  int ex_asset = -1, ex_top = 0;  // PAIR: the asset of the thread's records so far and their largest exponent
-#pragma unroll
-  for (int j = 0; j < kPrepE; ++j) {
-    const int64_t h = h0 + j;
-    b0v[j] = kNoCell;
-    dv[j] = (T)0;
-    vv[j] = (T)0;
-    if (h >= ntot) continue;
-    while (lo + 1 < D && off[lo + 1] <= h) ++lo;
-    if (!(h + 1 < off[lo + 1])) continue;  // the asset's last event: no return
-    // this event's problem: its fixed-point scale (batched form) or the
-    // call's single one
-    Rescale rs = rs0;
-    UScale us;
-    UScaleF usf;
-    if (gsc) {
-      const GroupScale q = gsc[lo / gsize];
-      rs.t0_fix = q.t0_fix;
-      rs.F = q.F;
-      us = q.us;
-      usf = q.usf;
-    } else if (scales) {
-      us.S = rs0.S;
-      us.sh = rs0.sh;
-      usf.s_hi = rs0.s_hi;
-      usf.s_lo = rs0.s_lo;
-    } else {
-      us = s_us;
-      usf = s_usf;
+    if (threadIdx.x == 0) {
+      if (!scales) s_us = make_uscale(rs0, Mr);  // (the same on each pass)
+      s_flags = 0;
     }
-    if (!(key[j] < key[j + 1])) flags |= (key[j] == key[j + 1]) ? ST_DUPLICATE : ST_UNSORTED;
-    if (!(fin_t[j] && fin_p[j] && fin_p[j + 1])) {
-      flags |= ST_NONFINITE;
-      continue;
-    }
-    const long long dt = to_fix(tv[j], rs.F) - rs.t0_fix;
-    int cb;
-    T cd;
-    bool past;  // beyond the cell's start
-    if (sizeof(T) == 8) {
-      const unsigned long long uf = u_fix_of(tv[j], rs.t0_fix, rs.F, us);
-      cb = (int)(uf >> kUFrac);
-      const unsigned long long frac = uf & ((1ull << kUFrac) - 1);
-      if (PAIR) cd = (T)offset_pair(frac);
-      else cd = frac_to<T>(frac);
-      past = frac != 0ull;
-    } else {
-      float fd;
-      cell_f32(dt, usf, cb, fd);
-      cd = (T)fd;
-      past = fd > 0.0f;
-    }
-    if (dt < 0 || cb > Mr || (cb == Mr && past)) {
-      flags |= ST_OUT_OF_WINDOW;
-      continue;
-    }
-    b0v[j] = cb;
-    dv[j] = cd;
-    if (sizeof(T) == 8) vv[j] = (T)(pv[j + 1] - pv[j]);
-    else vv[j] = (T)((ph[j + 1] - ph[j]) + (pl[j + 1] - pl[j]));
-    if (PAIR) {
-      if (lo != ex_asset && ex_asset >= 0) {
-        atomicMax(row_exp + ex_asset, ex_top);
-        ex_top = 0;
+    // asset of the block's first event (a 32-ary search by warp 0, a couple of
+    // dependent loads), then each thread walks forward to its own events' assets
+    if (threadIdx.x < 32) {
+      // first index in [1, D] with off[idx] > hb (D when none): the asset is idx - 1
+      const int lane = threadIdx.x;
+      int64_t lo = 1, hi = D;
+      for (int it = 0; it < 16 && hi > lo; ++it) {
+        const int64_t len = hi - lo;
+        const int64_t stride = (len + 31) / 32;
+        const int64_t o = (int64_t)lane * stride;
+        const bool below = o < len && off[lo + o] <= hb;
+        const int cnt = __popc(__ballot_sync(0xffffffffu, below));
+        if (cnt == 0) {
+          hi = lo;
+        } else {
+          const int64_t nlo = lo + (int64_t)(cnt - 1) * stride + 1;
+          const int64_t nhi = min(lo + (int64_t)cnt * stride, hi);
+          lo = min(nlo, nhi);
+          hi = nhi;
+        }
       }
-      ex_asset = lo;
-      ex_top = max(ex_top, (__double2hiint((double)vv[j]) >> 20) & 0x7FF);
+      if (lane == 0) s_a0 = (int)lo - 1;
     }
-  }
-  if (PAIR) {
-    // one update a warp when its threads' last records are of one asset
-    const int a0 = __shfl_sync(0xffffffffu, ex_asset, 0);
-    if (__all_sync(0xffffffffu, ex_asset == a0)) {
-      ex_top = __reduce_max_sync(0xffffffffu, ex_top);
-      if ((threadIdx.x & 31) == 0 && a0 >= 0) atomicMax(row_exp + a0, ex_top);
-    } else if (ex_asset >= 0) {
-      atomicMax(row_exp + ex_asset, ex_top);
-    }
-  }
-  if (h0 + kPrepE <= ntot) {
-    // h0 is a multiple of 4 and the record arrays are the plan's own
-    // (256-byte aligned) allocations: 16-byte vector stores
-    *reinterpret_cast<int4*>(rb0 + h0) = make_int4(b0v[0], b0v[1], b0v[2], b0v[3]);
-    Rec4<T>::store(rd + h0, dv);
-    Rec4<T>::store(rv + h0, vv);
-  } else {
+    __syncthreads();
+    int flags = 0;
+    int b0v[kPrepE];
+    T dv[kPrepE], vv[kPrepE];
+    int lo = s_a0;
+    // events of asset lo from h0 on (a thread looks at five)
+    auto left = [&](int a) {
+      const int64_t r = off[a + 1] - h0;
+      return r > kPrepE + 1 ? kPrepE + 2 : r < 0 ? 0 : (int)r;
+    };
+    int rem = left(lo);
+    int cur = -1;  // asset of the scale in use (batched form)
+    long long t0_fix = rs0.t0_fix;
+    int F = rs0.F;
+    UScale us{rs0.S, rs0.sh};
+    if (!scales) us = s_us;
+    int ex_asset = -1, ex_top = 0;  // PAIR: the asset of the thread's records so far and their largest exponent
+    // per value, once: order key, finiteness and (float32 path) the exact hi + lo
+    // split of the log-price
+    long long key = order_key(tv[0]);
+    bool fin_p = finite_bits(pv[0]);
+    float ph = 0.f, pl = 0.f;
+    if (sizeof(T) == 4) split_f64(pv[0], ph, pl);
 #pragma unroll
     for (int j = 0; j < kPrepE; ++j) {
-      if (h0 + j < ntot) {
-        rb0[h0 + j] = b0v[j];
-        rd[h0 + j] = dv[j];
-        rv[h0 + j] = vv[j];
+      const long long key0 = key;
+      const bool fin_p0 = fin_p;
+      const float ph0 = ph, pl0 = pl;
+      key = order_key(tv[j + 1]);
+      fin_p = finite_bits(pv[j + 1]);
+      if (sizeof(T) == 4) split_f64(pv[j + 1], ph, pl);
+      b0v[j] = kNoCell;
+      dv[j] = (T)0;
+      vv[j] = (T)0;
+      while (j >= rem && lo + 1 < D) rem = left(++lo);
+      if (!(j + 1 < rem)) continue;  // the asset's last event: no return
+      // this event's problem: its fixed-point scale (batched form), kept while
+      // the asset is the same, or the call's single one
+      if (gsc && lo != cur) {
+        const GroupScale q = gsc[lo / gsize];
+        t0_fix = q.t0_fix;
+        F = q.F;
+        us = q.us;
+        cur = lo;
+      }
+      if (!(key0 < key)) flags |= (key0 == key) ? ST_DUPLICATE : ST_UNSORTED;
+      if (!(finite_bits(tv[j]) && fin_p0 && fin_p)) {
+        flags |= ST_NONFINITE;
+        continue;
+      }
+      const long long dt = to_fix(tv[j], F) - t0_fix;
+      const unsigned long long uf = u_fix_of(dt, us);
+      const int cb = (int)(uf >> kUFrac);
+      const unsigned long long frac = uf & ((1ull << kUFrac) - 1);
+      if (dt < 0 || cb > Mr || (cb == Mr && frac != 0ull)) {  // beyond the last cell's start
+        flags |= ST_OUT_OF_WINDOW;
+        continue;
+      }
+      b0v[j] = cb;
+      if (PAIR) dv[j] = (T)offset_pair(frac);
+      else dv[j] = frac_to<T>(frac);
+      if (sizeof(T) == 8) vv[j] = (T)(pv[j + 1] - pv[j]);
+      else vv[j] = (T)((ph - ph0) + (pl - pl0));
+      if (PAIR) {
+        if (lo != ex_asset && ex_asset >= 0) {
+          atomicMax(row_exp + ex_asset, ex_top);
+          ex_top = 0;
+        }
+        ex_asset = lo;
+        ex_top = max(ex_top, (__double2hiint((double)vv[j]) >> 20) & 0x7FF);
       }
     }
+    if (PAIR) {
+      // one update a warp when its threads' last records are of one asset
+      const int a0 = __shfl_sync(0xffffffffu, ex_asset, 0);
+      if (__all_sync(0xffffffffu, ex_asset == a0)) {
+        ex_top = __reduce_max_sync(0xffffffffu, ex_top);
+        if ((threadIdx.x & 31) == 0 && a0 >= 0) atomicMax(row_exp + a0, ex_top);
+      } else if (ex_asset >= 0) {
+        atomicMax(row_exp + ex_asset, ex_top);
+      }
+    }
+    if (h0 + kPrepE <= ntot) {
+      // h0 is a multiple of 4 and the record arrays are the plan's own
+      // (256-byte aligned) allocations: 16-byte vector stores
+      *reinterpret_cast<int4*>(rb0 + h0) = make_int4(b0v[0], b0v[1], b0v[2], b0v[3]);
+      Rec4<T>::store(rd + h0, dv);
+      Rec4<T>::store(rv + h0, vv);
+    } else {
+#pragma unroll
+      for (int j = 0; j < kPrepE; ++j) {
+        if (h0 + j < ntot) {
+          rb0[h0 + j] = b0v[j];
+          rd[h0 + j] = dv[j];
+          rv[h0 + j] = vv[j];
+        }
+      }
+    }
+    if (flags) atomicOr(&s_flags, flags);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_flags) atomicOr(status, s_flags);
+    if (!SPARE) break;
   }
-  if (flags) atomicOr(&s_flags, flags);
-  __syncthreads();
-  if (threadIdx.x == 0 && s_flags) atomicOr(status, s_flags);
   pdl_trigger();
 }
 
 template <typename T, bool PAIR>
 static cudaError_t launch_prep_t(const int64_t* off, const double* t, const double* logp, const Rescale* rs,
-                                 const GroupScale* gsc, int gsize, int D, int64_t Mr, int64_t max_events, int* rb0,
-                                 T* rd, T* rv, int* row_exp, int* status, cudaStream_t s) {
+                                 const GroupScale* gsc, int gsize, int D, int64_t Mr, int64_t max_events, bool spare,
+                                 int* rb0, T* rd, T* rv, int* row_exp, int* status, cudaStream_t s) {
   if (max_events <= 0) return cudaSuccess;
   if ((((uintptr_t)rb0) | ((uintptr_t)rd) | ((uintptr_t)rv)) & 15) return cudaErrorMisalignedAddress;
   const int64_t per_block = (int64_t)kPrepThreads * kPrepE;
-  const int64_t blocks = (max_events + per_block - 1) / per_block;
-  return launch_pdl(k_prep<T, PAIR>, dim3((unsigned)blocks), dim3(kPrepThreads), 0, s, off, t, logp, rs, gsc, gsize,
-                    status + 1, D, Mr, rb0, rd, rv, row_exp, status);
+  int64_t blocks = (max_events + per_block - 1) / per_block;
+  if (spare) blocks = std::min(blocks, kPrepSpareBlocks);
+  return launch_pdl(spare ? k_prep<T, PAIR, true> : k_prep<T, PAIR, false>, dim3((unsigned)blocks),
+                    dim3(kPrepThreads), 0, s, off, t, logp, rs, gsc, gsize, status + 1, D, Mr, rb0, rd, rv, row_exp,
+                    status);
 }
 
 cudaError_t launch_prep_f32(const int64_t* off, const double* t, const double* logp, const Rescale* rs,
                             const GroupScale* gsc, int gsize, int D,
-                            int64_t Mr, int64_t max_events, int* rb0, void* rd, void* rv, int* status,
+                            int64_t Mr, int64_t max_events, bool spare, int* rb0, void* rd, void* rv, int* status,
                             cudaStream_t s) {
-  return launch_prep_t<float, false>(off, t, logp, rs, gsc, gsize, D, Mr, max_events, rb0, (float*)rd, (float*)rv,
+  return launch_prep_t<float, false>(off, t, logp, rs, gsc, gsize, D, Mr, max_events, spare, rb0, (float*)rd, (float*)rv,
                                      nullptr, status, s);
 }
 cudaError_t launch_prep_f64(const int64_t* off, const double* t, const double* logp, const Rescale* rs,
                             const GroupScale* gsc, int gsize, int D,
-                            int64_t Mr, int64_t max_events, int* row_exp, int* rb0, void* rd, void* rv, int* status,
-                            cudaStream_t s) {
+                            int64_t Mr, int64_t max_events, bool spare, int* row_exp, int* rb0, void* rd, void* rv,
+                            int* status, cudaStream_t s) {
   auto go = [&](auto fn) {
-    return fn(off, t, logp, rs, gsc, gsize, D, Mr, max_events, rb0, (double*)rd, (double*)rv, row_exp, status, s);
+    return fn(off, t, logp, rs, gsc, gsize, D, Mr, max_events, spare, rb0, (double*)rd, (double*)rv, row_exp, status, s);
   };
   return row_exp ? go(launch_prep_t<double, true>) : go(launch_prep_t<double, false>);
 }
@@ -716,11 +720,12 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread_scatter(const int64_t
 // Threads of a polynomial-scatter block and records it stages at a time. A block is
 // a chain of dependent latencies (offsets, search, records, barriers), which other
 // blocks hide when there are many: 128 threads and eight blocks an SM from
-// kPolyBlocksMany tiles up (512 replications of ten assets: 463 us against 609 us
+// kPolyBlocksMany tiles up (512 replications of ten assets: 474 us against 609 us
 // with 256 threads), 256 threads and six blocks down to kPolyBlocksSome (the block
-// workload's 1000 tiles: 17.6 us against 20.7 us with 128), else 512 threads. 512 also where the assets' capacity gives a tile more than
-// kPolyManyRecords (a busy day in the one tile of a low cutoff's grid): a thread
-// then sums runs of several records of a cell before it reduces.
+// workload's 1000 tiles: 18.4 us against 20.7 us with 128), else 512 threads. 512 also
+// where the assets' capacity gives a tile more than kPolyManyRecords (a busy day in
+// the one tile of a low cutoff's grid): a thread then sums runs of several records
+// of a cell before it reduces.
 template <int NTH> struct PolyBlock;
 template <> struct PolyBlock<128> { static constexpr int chunk = 896, per_sm = 8; };
 template <> struct PolyBlock<256> { static constexpr int chunk = 1536, per_sm = 6; };
@@ -738,8 +743,8 @@ constexpr int kPolyManyRecords = 4096;
 // that at most and 2^-27 rms, as its float32 product's own rounding. That halves
 // the shared-memory reductions, which bound the taps, and the tile. With the shorter
 // taps below, the guessed search and the block sizes above the block workload's
-// spreading took 17.6 us (20.2 us with two words a cell in every tile), 500 stocks'
-// day 127 us (143 us), 512 replications of ten assets 463 us (715 us).
+// spreading took 18.4 us (20.2 us with two words a cell in every tile), 500 stocks'
+// day 128 us (143 us), 512 replications of ten assets 474 us (715 us).
 constexpr int kOneRun = 20;
 
 // Taps k and 1 - k of a record are phi(a - z) and phi(a + z), a = k - 1/2,
@@ -837,7 +842,7 @@ __global__ void __launch_bounds__(NTH, PolyBlock<NTH>::per_sm) k_spread_poly(con
                                                                const int* __restrict__ gate, SpreadParams p,
                                                                const __grid_constant__ KernelPoly poly,
                                                                const __grid_constant__ PairTaps taps, int cells,
-                                                               float* __restrict__ grid) {
+                                                               int widths_first, float* __restrict__ grid) {
   constexpr int EC = PolyBlock<NTH>::chunk;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   int* ev_p = reinterpret_cast<int*>(smem_raw);
@@ -863,7 +868,10 @@ __global__ void __launch_bounds__(NTH, PolyBlock<NTH>::per_sm) k_spread_poly(con
       load_record<float>(rb0, rd, rv, p, tr, L, c0 + i, ev_p[i], ev_d[i], ev_v[i]);
   };
   // at most kOneRun records in any stencil's width, and their sums of |v|;
-  // chunks overlap by a run, and the last one stays staged
+  // chunks overlap by a run, and the last one stays staged. Where the assets'
+  // density makes dense tiles likely the widths are looked at first, so that such
+  // a tile leaves before the sums, which cost half its taps (a barrier more: 1.5 us
+  // of the block workload's spreading)
   bool sparse = Tlen <= cells;
   float run = 0.f;
   int64_t cs = 0;
@@ -874,6 +882,12 @@ __global__ void __launch_bounds__(NTH, PolyBlock<NTH>::per_sm) k_spread_poly(con
     __syncthreads();
     const bool last = cs + n == ntot;
     const int lim = last ? n : n - kOneRun;
+    if (widths_first) {
+      for (int i = threadIdx.x; i + kOneRun < n; i += NTH)
+        sparse = sparse && ev_p[i + kOneRun] - ev_p[i] > 2 * NP;
+      sparse = __syncthreads_and(sparse);
+      if (!sparse) break;
+    }
     for (int i = threadIdx.x; i < lim; i += NTH) {
       if (i + kOneRun < n) sparse = sparse && ev_p[i + kOneRun] - ev_p[i] > 2 * NP;
       float w = 0.f;
@@ -882,17 +896,17 @@ __global__ void __launch_bounds__(NTH, PolyBlock<NTH>::per_sm) k_spread_poly(con
       run = fmaxf(run, w);
     }
     if (last) break;
-    cs += EC - kOneRun;
-    if (!__syncthreads_and(sparse)) {  // dense already: the rest does not matter
+    if (!__syncthreads_and(sparse)) {
       sparse = false;
       break;
     }
+    cs += EC - kOneRun;
   }
   run = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(run)));  // not negative
   if ((threadIdx.x & 31) == 0) s_run[threadIdx.x >> 5] = run;
   sparse = __syncthreads_and(sparse);
 #pragma unroll
-  for (int w = 0; w < NTH / 32; ++w) run = fmaxf(run, s_run[w]);
+  for (int w = 0; w < NTH / 32; ++w) run = sparse ? fmaxf(run, s_run[w]) : 0.f;
   // 2^e and 2^-e have to be normal floats
   if (sparse && run < 1.0e30f && (run > 1.0e-27f || run == 0.f)) {
     int ex = 0;
@@ -912,9 +926,15 @@ __global__ void __launch_bounds__(NTH, PolyBlock<NTH>::per_sm) k_spread_poly(con
     pdl_trigger();
     return;
   }
-  // the tile's scales: sum and maximum of |v| over its records
+  // the tile's scales: sum and maximum of |v| over its records, those of the first
+  // chunk from where they are staged
+  const int first = cs == 0 ? n : 0;
   float part = 0.f, pmax = 0.f;
-  for (int64_t i = threadIdx.x; i < ntot; i += NTH) {
+  for (int i = threadIdx.x; i < first; i += NTH) {
+    part += fabsf(ev_v[i]);
+    pmax = fmaxf(pmax, fabsf(ev_v[i]));
+  }
+  for (int64_t i = first + threadIdx.x; i < ntot; i += NTH) {
     int pp;
     float dd, vv;
     load_record<float>(rb0, rd, rv, p, tr, L, i, pp, dd, vv);
@@ -932,8 +952,10 @@ __global__ void __launch_bounds__(NTH, PolyBlock<NTH>::per_sm) k_spread_poly(con
     }
     for (int64_t c0 = 0; c0 < ntot; c0 += EC) {
       const int m = (int)min((int64_t)EC, ntot - c0);
-      __syncthreads();
-      stage(c0, m);
+      if (c0 > 0 || (s0 > 0 ? ntot > EC : first == 0)) {  // else staged already
+        __syncthreads();
+        stage(c0, m);
+      }
       __syncthreads();
       spread_chunk<NT, NTH>(ev_p, ev_d, ev_v, m, len, p.klo - s0, poly, ts, tile_s, tile_s + 4u * half, AllCells{});
     }
@@ -976,7 +998,7 @@ cudaError_t launch_spread_poly(const int64_t* off, const int* rb0, const void* r
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     return launch_pdl(fn, grd, dim3(nth), smem, s, off, rb0, (const float*)rd, (const float*)rv,
-                      (const int*)(status + 1), p, poly, taps, cells, grid);
+                      (const int*)(status + 1), p, poly, taps, cells, p.dense, grid);
   };
   // tap counts without an instantiation: the next one up, padded with zero taps
   auto pick = [&](auto w) -> cudaError_t {
