@@ -37,18 +37,18 @@ L2_FLUSH_BYTES = 256 << 20  # > 129 MB L2
 # summarised in profiles/ (a kernel changed since its capture has no entry)
 NCU_TRAFFIC = {
     # the block workload in its default configuration
-    # (profiles/c3_block_D100_N10000_kernels_ncu.md)
-    ("fft", "c3", "bf16x3", "es"): 16438016,
-    ("spread", "c3", "bf16x3", "es"): 9236224,
-    ("prep", "c3", "bf16x3", "es"): 12287488,
-    ("gram", "c3", "bf16x3", "es"): 8115712,
+    # (profiles/c3_and_c4_R256_kernels_ncu.md)
+    ("fft", "c3", "bf16x3", "es"): 16438528,
+    ("spread", "c3", "bf16x3", "es"): 9264896,
+    ("prep", "c3", "bf16x3", "es"): 12286208,
+    ("gram", "c3", "bf16x3", "es"): 8112640,
     # the pre-split contraction alone at D = 500, N = 14400
     # (profiles/gram_D500_N14400_kernel_ncu.md)
     ("gram", "gram_D500_N14400", "bf16x3", "es", "tma"): 60790272,
 }
 NCU_SOURCE = {
-    "c3": "profiles/c3_block_D100_N10000_kernels_ncu.md",
-    "c4": "profiles/c4_batch_R256_D10_kernels_ncu.md",
+    "c3": "profiles/c3_and_c4_R256_kernels_ncu.md",
+    "c4": "profiles/c3_and_c4_R256_kernels_ncu.md",
     "gram_D500_N14400": "profiles/gram_D500_N14400_kernel_ncu.md",
 }
 # the batched workload is too large for a full ncu capture: dram bytes per
@@ -56,7 +56,7 @@ NCU_SOURCE = {
 # M_r = 57600), scaled by the rows of a launch (the traffic is the rows' grid
 # reads and coefficient writes, so it grows with them)
 NCU_TRAFFIC_PER_ROW = {
-    ("fft", "c4", "bf16x3", "es", 57600): (590240768 + 264606464) / 2560.0,
+    ("fft", "c4", "bf16x3", "es", 57600): (590388480 + 262378240) / 2560.0,
 }
 
 # Stages (a)-(c) of the hot path, as the library's profiler names them.

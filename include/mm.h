@@ -79,7 +79,9 @@ typedef enum { MM_BASIS_DIRICHLET = 0, MM_BASIS_FEJER = 1 } mm_basis;
  * Sec. 2.2.5. */
 typedef enum { MM_KERNEL_GAUSS = 0, MM_KERNEL_KB = 1, MM_KERNEL_ES = 2 } mm_kernel;
 
-/* MM_PREC_FP64: every stage in float64. MM_PREC_MIXED_*: rescaling, phase
+/* MM_PREC_FP64: float64 data and results; spreading and FFT in float pairs (47
+ * bits) where their error is 50 times below the tolerance (tol >= 5e-13), every
+ * stage in float64 below that. MM_PREC_MIXED_*: rescaling, phase
  * reduction to grid offsets, differencing into returns and the diagonal
  * normalisation in float64; spreading, FFT and deconvolution in float32; the
  * contraction on the tensor cores as split bf16 (hi*hi + hi*lo + lo*hi) or
