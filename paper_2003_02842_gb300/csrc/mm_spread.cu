@@ -1154,10 +1154,16 @@ __global__ void __launch_bounds__(kSpreadThreads, 4) k_spread_pair(const int64_t
       if (live) {
         const double zz = ev_d[e];
         z = {__int_as_float(__double2hiint(zz)), __int_as_float(__double2loint(zz))};
-        // v 2^eh from the exponent field; more than 2^1000 below V: zero
-        const long long b = __double_as_longlong(ev_v[e]);
-        const int ex = (int)((b >> 52) & 0x7FF);
-        if (ex > 0 && ex + eh > 0) split_f64(__longlong_as_double(b + ((long long)eh << 52)), v.h, v.l);
+        // v 2^eh from the exponent field (a subnormal return's after 54 binary
+        // places up); more than 2^1000 below V: zero
+        long long b = __double_as_longlong(ev_v[e]);
+        int ex = (int)((b >> 52) & 0x7FF), up = eh;
+        if (ex == 0) {
+          b = __double_as_longlong(ev_v[e] * 18014398509481984.0);  // 2^54
+          ex = (int)((b >> 52) & 0x7FF);
+          up = eh - 54;
+        }
+        if (ex > 0 && ex + up > 0) split_f64(__longlong_as_double(b + ((long long)up << 52)), v.h, v.l);
       }
       const float yh = __fmul_rn(z.h, z.h);
       const FloatPair y{yh, __fmaf_rn(z.l, z.l, __fmaf_rn(__fadd_rn(z.h, z.h), z.l, __fmaf_rn(z.h, z.h, -yh)))};
@@ -1205,7 +1211,7 @@ __global__ void __launch_bounds__(kSpreadThreads, 4) k_spread_pair(const int64_t
     const float h = (float)A;  // rounded to 24 bits: A - h is exact in 63 bits and has few left
     const float l = (float)(A - (long long)h) + below;
     if (plain) g[c] = FloatPair(h * unit, l * unit);
-    else g[c] = FloatPair(top == 0x7FF ? __int_as_float(0x7fc00000) : ldexpf(h, sa), ldexpf(l, sa));
+    else g[c] = FloatPair(ldexpf(h, sa), ldexpf(l, sa));
   }
 }
 

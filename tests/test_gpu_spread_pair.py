@@ -12,7 +12,7 @@ import pytest
 import oracle
 from paper_2003_02842_gb300 import synth
 
-from gpu_helpers import rel_l2_rows, run
+from gpu_helpers import rel_l2_rows, run, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -66,3 +66,45 @@ def test_tight_tolerances_keep_float64_taps():
     ev = synth.random_events(9, D=2, n_range=(100, 500), T=1000.0)
     F, G = _both(ev, 300, "es", 0, tol=1e-14)
     assert rel_l2_rows(F, G).max() <= 2e-15
+
+
+def _coeffs(ev, N, algo):
+    import paper_2003_02842_gb300 as mm
+    plan = mm.mm_plan_create(D=ev.D, N_max=N, max_events=ev.n_events, tol=1e-12, kernel="es", prec="fp64",
+                             spread_algo=algo)
+    F, _ = mm.mm_coeffs(plan, *to_dev(ev), N)
+    mm.mm_plan_sync(plan)
+    F = F.cpu().numpy()
+    mm.mm_destroy(plan)
+    return F
+
+
+@pytest.mark.parametrize("size", [0.9 * 2.0**1023, 1.2 * 2.0**1023, 1.9 * 2.0**1023])
+def test_returns_at_the_top_of_float64(size):
+    # four returns of +-size (their exponent's power, 2^1024, is beyond float64 from 2^1023 on);
+    # a coefficient is at most 4 size / (2 pi), finite. The oracle works on 2^-1000 of them
+    t = np.array([0.0, 130.0, 377.0, 781.5, 1000.0])
+    ev = synth.from_lists([t], [0.5 * size * (-1.0) ** np.arange(5)])
+    F = _coeffs(ev, 60, "scatter")
+    ref = oracle.coeffs_F(ev.offsets, ev.t, ev.logp * 2.0**-1000, 60)
+    assert np.isfinite(F).all()
+    assert rel_l2_rows(F * 2.0**-1000, ref).max() <= 1e-11
+
+
+def test_a_return_beyond_float64_gives_nan():
+    ev = synth.random_events(11, D=2, n_range=(60, 90), T=1000.0)
+    p = ev.logp.copy()
+    p[10], p[11] = 1.7e308, -1.7e308  # the first asset's return overflows
+    ev = synth.Events(ev.offsets, ev.t, p)
+    F, G = _coeffs(ev, 40, "scatter"), _coeffs(ev, 40, "gather")
+    assert np.isnan(F[0]).all() and not np.isfinite(G[0]).any()
+    assert rel_l2_rows(F[1:], G[1:]).max() <= 1e-13
+
+
+def test_subnormal_returns():
+    # returns below 2^-1022, some 40 bits above float64's last place (2^-1074)
+    ev = synth.random_events(12, D=2, n_range=(60, 90), T=1000.0)
+    ev = synth.Events(ev.offsets, ev.t, (ev.logp - 4.6) * 2.0**-1024)
+    assert np.abs(np.diff(ev.logp)).max() < 2.0**-1022
+    F, G = _coeffs(ev, 40, "scatter") * 2.0**1000, _coeffs(ev, 40, "gather") * 2.0**1000
+    assert np.linalg.norm(G) > 0 and rel_l2_rows(F, G).max() <= 1e-9
