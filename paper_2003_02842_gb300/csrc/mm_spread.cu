@@ -738,14 +738,18 @@ constexpr int kPolyManyRecords = 4096;
 // holds more than kOneRun records, a cell's sum is at most the largest sum W of
 // |v| over kOneRun records in a row, not that of the tile: with x = v phi 2^e,
 // e = 30 - ex(W), every cell's sum of the rounded x stays below 2^30 (1 + 1e-6)
-// + kOneRun / 2 < 2^31 in one int32, with a quantum of at most W 2^-29. A run's W
-// is some 16 times the typical return at 20 records, so a tap is off by 2^-25 of
-// that at most and 2^-27 rms, as its float32 product's own rounding. That halves
-// the shared-memory reductions, which bound the taps, and the tile. With the shorter
+// + kOneRun / 2 < 2^31 in one int32, with a quantum of at most W 2^-29. The tile is
+// taken so only where W is at most kOneEven times the mean sum of a run, kOneRun
+// times the mean |v|: a tap is then off by at most 80 2^-30 of the mean |v|, 2^-24.5
+// of it rms, as the float32 product of a tap is, and a return that dwarfs the
+// others does not cost them their digits (they keep two words; Brownian returns
+// at Poisson times stay at about twice the mean). One word halves the
+// shared-memory reductions, which bound the taps, and the tile. With the shorter
 // taps below, the guessed search and the block sizes above the block workload's
 // spreading took 18.4 us (20.2 us with two words a cell in every tile), 500 stocks'
 // day 128 us (143 us), 512 replications of ten assets 474 us (715 us).
 constexpr int kOneRun = 20;
+constexpr float kOneEven = 4.0f;
 
 // Taps k and 1 - k of a record are phi(a - z) and phi(a + z), a = k - 1/2,
 // z = d - 1/2: with tap k's polynomial E(z^2) + z O(z^2), tap 1 - k is
@@ -850,7 +854,7 @@ __global__ void __launch_bounds__(NTH, PolyBlock<NTH>::per_sm) k_spread_poly(con
   float* ev_v = ev_d + EC;
   int* tile = reinterpret_cast<int*>(ev_v + EC);
   const uint32_t tile_s = (uint32_t)__cvta_generic_to_shared(tile);
-  __shared__ float s_sum[NTH / 32], s_max[NTH / 32], s_run[NTH / 32];
+  __shared__ float s_sum[NTH / 32], s_max[NTH / 32], s_run[NTH / 32], s_all[NTH / 32];
   const int64_t L = (int64_t)blockIdx.x * p.tile;
   const int Tlen = (int)min((int64_t)p.tile, p.Mr - L);
   auto clear = [&] {
@@ -867,13 +871,13 @@ __global__ void __launch_bounds__(NTH, PolyBlock<NTH>::per_sm) k_spread_poly(con
     for (int i = threadIdx.x; i < n; i += NTH)
       load_record<float>(rb0, rd, rv, p, tr, L, c0 + i, ev_p[i], ev_d[i], ev_v[i]);
   };
-  // at most kOneRun records in any stencil's width, and their sums of |v|;
+  // at most kOneRun records in any stencil's width, and the sums of |v|;
   // chunks overlap by a run, and the last one stays staged. Where the assets'
   // density makes dense tiles likely the widths are looked at first, so that such
   // a tile leaves before the sums, which cost half its taps (a barrier more: 1.5 us
   // of the block workload's spreading)
   bool sparse = Tlen <= cells;
-  float run = 0.f;
+  float run = 0.f, all = 0.f;  // largest sum over a run, sum over the tile
   int64_t cs = 0;
   int n = 0;
   while (true) {
@@ -894,6 +898,7 @@ __global__ void __launch_bounds__(NTH, PolyBlock<NTH>::per_sm) k_spread_poly(con
 #pragma unroll
       for (int j = 0; j < kOneRun; ++j) w += i + j < n ? fabsf(ev_v[i + j]) : 0.f;
       run = fmaxf(run, w);
+      all += fabsf(ev_v[i]);
     }
     if (last) break;
     if (!__syncthreads_and(sparse)) {
@@ -903,12 +908,22 @@ __global__ void __launch_bounds__(NTH, PolyBlock<NTH>::per_sm) k_spread_poly(con
     cs += EC - kOneRun;
   }
   run = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(run)));  // not negative
-  if ((threadIdx.x & 31) == 0) s_run[threadIdx.x >> 5] = run;
-  sparse = __syncthreads_and(sparse);
 #pragma unroll
-  for (int w = 0; w < NTH / 32; ++w) run = sparse ? fmaxf(run, s_run[w]) : 0.f;
+  for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
+  if ((threadIdx.x & 31) == 0) {
+    s_run[threadIdx.x >> 5] = run;
+    s_all[threadIdx.x >> 5] = all;
+  }
+  sparse = __syncthreads_and(sparse);
+  all = 0.f;
+#pragma unroll
+  for (int w = 0; w < NTH / 32; ++w) {
+    run = sparse ? fmaxf(run, s_run[w]) : 0.f;
+    all += s_all[w];
+  }
+  const bool even = run * (float)ntot <= kOneEven * (float)kOneRun * all;
   // 2^e and 2^-e have to be normal floats
-  if (sparse && run < 1.0e30f && (run > 1.0e-27f || run == 0.f)) {
+  if (sparse && even && run < 1.0e30f && (run > 1.0e-27f || run == 0.f)) {
     int ex = 0;
     if (run > 0.f) frexpf(run, &ex);  // run < 2^ex
     const int e = 30 - ex;

@@ -81,3 +81,27 @@ def test_one_return_dwarfs_the_others():
     lp = ev.logp.copy()
     lp[100:] += 1.0e4
     _check(synth.Events(ev.offsets, ev.t, lp), 700)
+
+
+def test_small_returns_beside_a_large_one_keep_their_digits():
+    # One return of 1 among 5300 of 2^-32 to 2^-30.4, all of one sign, in one tile of 4096 cells
+    # with at most 20 records in any stencil's width. Each is below half the quantum that the
+    # large one would set for one word a cell (2^-29); together they are 2.5e-6 of it, 20 times
+    # the float32 rounding of the transform of both. What they add to the coefficients is
+    # taken against the large return alone.
+    n, N = 5300, 1020
+    u = (np.arange(n + 1) + 0.25 * np.sin(np.arange(n + 1))) / n
+    u[0], u[-1] = 0.0, 1.0
+    v = 2.0**-31 * (1.0 + 0.5 * np.cos(6.0 * np.pi * u[:-1]))
+    one = np.zeros(n)
+    one[n // 3] = 1.0
+
+    def coeffs(r):
+        ev = synth.from_lists([u * 1000.0], [np.concatenate([[0.0], np.cumsum(r)])])
+        return ev, _coeffs(ev, N, "es", "bf16x3", tile=4096)[0]
+
+    ev, F = coeffs(one + v)
+    _, F1 = coeffs(one)
+    small = synth.Events(ev.offsets, ev.t, np.concatenate([[0.0], np.cumsum(v)]))
+    ref = oracle.coeffs_F(small.offsets, small.t, small.logp, N)[0]
+    assert np.abs((F - F1 - ref)[:6]).max() <= 0.3 * abs(ref[0])
