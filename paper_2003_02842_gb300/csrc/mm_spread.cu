@@ -320,7 +320,7 @@ constexpr int kSpreadThreads = 256;
 //
 // Bound by the integer pipe (51 % of its rate, and 70 % of the SMs' time at 1.03
 // waves of the former 256-thread blocks): the cell and its offset of both paths come
-// from one 64 x 64 -> 128-bit product (float32 offsets rounded to 2^-24 of a cell;
+// from one 64 x 64 -> 128-bit product (float32 offsets to 24 significant bits;
 // a float-pair product took twice the instructions), the end of the asset is kept
 // as a count instead of read for each event, a problem's scale is read once per
 // asset of a thread, whole stretches come by 16-byte loads. 128 threads leave 56

@@ -157,8 +157,8 @@ __device__ __forceinline__ T kernel_value(T x, const SpreadParams& p) {
 
 template <typename T> __device__ __forceinline__ T frac_to(unsigned long long frac);
 template <> __device__ __forceinline__ float frac_to<float>(unsigned long long frac) {
-  // 24 bits, rounded
-  return __uint2float_rn((unsigned)((frac + (1ull << (kUFrac - 25))) >> (kUFrac - 24))) * 5.9604644775390625e-8f;
+  // to 24 significant bits, from 32
+  return __uint2float_rn((unsigned)(frac >> (kUFrac - 32))) * 2.3283064365386963e-10f;
 }
 template <> __device__ __forceinline__ double frac_to<double>(unsigned long long frac) {
   return (double)frac * 9.094947017729282e-13;  // * 2^-40

@@ -85,3 +85,33 @@ def test_time_far_beyond_the_window(prec, far):
                  torch.from_numpy(ev.logp).cuda(), 100)
     assert mm.mm_plan_sync(plan) == 1  # invalid argument, before "unsorted"
     mm.mm_destroy(plan)
+
+
+def test_float32_offsets_keep_24_significant_bits():
+    # One return an asset at cell b + d of 4096 cells of width 1, d in [1/4, 1/2) a multiple of
+    # 2^-24, then the same 2^-25 later: the coefficients' phases, -2 pi k (b + d) / 4096, have to
+    # turn by 2^-25 of a cell. Rounded to 2^-24 the second set turns by twice that. A tap's
+    # float32 rounding moves a single asset by some 1e-7 of a cell, the mean of 4096 by 2.5e-9;
+    # the bound is three times that.
+    import torch
+
+    import paper_2003_02842_gb300 as mm
+    D, N, M = 4096, 1020, 4096.0
+    rng = np.random.default_rng(41)
+    u = rng.integers(64, 4000, D) + rng.integers(2**22, 2**23, D) * 2.0**-24
+    turned = []
+    for add in (0.0, 2.0**-25):
+        t = np.stack([u + add, np.full(D, M - 1.0)], 1).ravel()
+        p = np.tile([0.0, 1.0], D)
+        off = np.arange(0, 2 * D + 1, 2, dtype=np.int64)
+        plan = mm.mm_plan_create(D=D, N_max=N, max_events=2 * D, tol=1e-6)
+        F, _ = mm.mm_coeffs(plan, *[torch.from_numpy(x).cuda() for x in (off, t, p)], N, window=(0.0, M))
+        assert mm.mm_plan_sync(plan) == 0 and mm.mm_plan_get_info(plan)["Mr"] == 4096
+        mm.mm_destroy(plan)
+        k = torch.arange(N + 1, device="cuda", dtype=torch.float64)
+        x = torch.from_numpy(u).cuda()
+        ref = torch.polar(torch.ones(D, N + 1, device="cuda", dtype=torch.float64),
+                          2.0 * np.pi * (torch.frac(x[:, None] * k / M)))
+        phase = (F.to(torch.complex128) * ref * 2.0 * np.pi).imag  # -2 pi k (shift) / M
+        turned.append(-(phase * k).sum() / (k * k).sum() / D * M / (2.0 * np.pi))
+    assert abs(float(turned[1] - turned[0]) - 2.0**-25) <= 2.0**-27
