@@ -837,7 +837,10 @@ __device__ __forceinline__ void write_cells(const SpreadParams& p, float* __rest
 
 // One block per tile. `cells` int32 of shared memory: a sparse tile has one word
 // per cell, a dense one (by the records themselves) is taken in parts of cells / 2
-// with a hi and a lo word each.
+// with a hi and a lo word each. A part stages and evaluates the records that reach it,
+// from its first on (every part going through all of the tile's: one asset of 40,000
+// records among 99 of 2,000 on 40,500 cells 44.6 us, now 38.2; 25 of 500 assets with
+// 100,000 on 57,600 cells 166 us, now 133).
 template <int NT, int NP, int NTH>
 __global__ void __launch_bounds__(NTH, PolyBlock<NTH>::per_sm) k_spread_poly(const int64_t* __restrict__ off,
                                                                const int* __restrict__ rb0,
@@ -894,6 +897,7 @@ __global__ void __launch_bounds__(NTH, PolyBlock<NTH>::per_sm) k_spread_poly(con
     }
     for (int i = threadIdx.x; i < lim; i += NTH) {
       if (i + kOneRun < n) sparse = sparse && ev_p[i + kOneRun] - ev_p[i] > 2 * NP;
+      if (!sparse) break;  // the sums are not wanted
       float w = 0.f;
 #pragma unroll
       for (int j = 0; j < kOneRun; ++j) w += i + j < n ? fabsf(ev_v[i + j]) : 0.f;
@@ -959,21 +963,42 @@ __global__ void __launch_bounds__(NTH, PolyBlock<NTH>::per_sm) k_spread_poly(con
   const TileScales ts = tile_scales<NTH>(part, pmax, ntot, s_sum, s_max);
   const float inv_h = ts.inv_h, inv_l = ts.inv_l;
   const int half = cells / 2 & ~3;
+  // records of the staged chunk before `cell` (they are sorted)
+  auto before = [&](int cell, int m) {
+    int lo = 0, hi = m;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (ev_p[mid] < cell) lo = mid + 1;
+      else hi = mid;
+    }
+    return lo;
+  };
+  int64_t from = 0;  // the part's first record
   for (int s0 = 0; s0 < Tlen; s0 += half) {
     const int len = min(half, Tlen - s0);
+    const bool more = s0 + half < Tlen;  // another part follows
+    int64_t next = ntot;
     if (s0 > 0) {
       __syncthreads();
       clear();
     }
-    for (int64_t c0 = 0; c0 < ntot; c0 += EC) {
-      const int m = (int)min((int64_t)EC, ntot - c0);
-      if (c0 > 0 || (s0 > 0 ? ntot > EC : first == 0)) {  // else staged already
+    for (int64_t c0 = from; c0 < ntot; c0 += EC) {
+      int m = (int)min((int64_t)EC, ntot - c0);
+      if (c0 > 0 || s0 > 0 || first == 0) {  // else staged already
         __syncthreads();
         stage(c0, m);
       }
       __syncthreads();
+      const int all = m;
+      if (more) {
+        const int q = before(s0 + half - p.khi, all);
+        if (q < all && next == ntot) next = c0 + q;
+        m = before(s0 + half - p.klo, all);
+      }
       spread_chunk<NT, NTH>(ev_p, ev_d, ev_v, m, len, p.klo - s0, poly, ts, tile_s, tile_s + 4u * half, AllCells{});
+      if (m < all) break;  // uniform: the rest lies beyond the part
     }
+    from = next;
     __syncthreads();
     write_cells<NTH>(p, grid, a, L, s0, len,
                      [&](int c) { return fmaf((float)tile[half + c], inv_l, (float)tile[c] * inv_h); });
