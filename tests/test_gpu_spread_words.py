@@ -105,3 +105,18 @@ def test_small_returns_beside_a_large_one_keep_their_digits():
     small = synth.Events(ev.offsets, ev.t, np.concatenate([[0.0], np.cumsum(v)]))
     ref = oracle.coeffs_F(small.offsets, small.t, small.logp, N)[0]
     assert np.abs((F - F1 - ref)[:6]).max() <= 0.3 * abs(ref[0])
+
+
+@pytest.mark.parametrize("kernel,tol,msp", [("gauss", 1e-8, 9), ("gauss", 1e-11, 12), ("gauss", 1e-12, 13), ("es", 1e-12, 9)])
+@pytest.mark.parametrize("n", [300, 9000])
+def test_wide_stencils(kernel, tol, msp, n):
+    # 18 to 26 taps (24 and 25 on both sides of an instantiation), sparse and dense tiles
+    import paper_2003_02842_gb300 as mm
+    ev = synth.random_events(n, D=2, n_range=(n, n), T=5000.0)
+    plan = mm.mm_plan_create(D=2, N_max=1000, max_events=ev.n_events, tol=tol, kernel=kernel)
+    F, _ = mm.mm_coeffs(plan, *to_dev(ev), 1000)
+    info = mm.mm_plan_get_info(plan)
+    assert mm.mm_plan_sync(plan) == 0 and info["msp"] == msp and info["spread_poly"] == 1
+    F = F.cpu().numpy().astype(np.complex128)
+    mm.mm_destroy(plan)
+    assert rel_l2_rows(F, _coeffs(ev, 1000, kernel, "fp64", tol=tol)).max() <= 1e-6
