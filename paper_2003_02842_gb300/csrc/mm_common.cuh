@@ -194,7 +194,7 @@ struct GramParams {
   int D;
   int N;             // modes k = 0..N
   int ld;            // leading dimension (complex elements) of the coefficients
-  int tile;          // output tile edge (128 tensor path, 4 fp64 path)
+  int tile;          // output tile edge (128 tensor path, 4 or 64 fp64 path)
   int ntiles;        // ceil(D / tile)
   int npairs;        // ntiles (ntiles+1) / 2
   int splits;        // split-K factor

@@ -25,6 +25,8 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include "mm_async.cuh"
 #include "mm_common.cuh"
 #include "mm_tc.cuh"
@@ -135,10 +137,71 @@ __global__ void __launch_bounds__(32 * kF64Warps, 2)
   }
 }
 
-// Tiles, chunks and splits of the FP64 contraction: about eight CTAs per SM
+// The same over 64 x 64 tiles, for many assets: 256 threads with a 4 x 4 micro-tile
+// each, K in chunks of 16 complex modes staged with their weights. Its CTAs are few and
+// long (34 us a chunk and wave), so it wins where they fill whole waves of the SMs and
+// where the 4 x 4 tiles are so many that their CTAs' fixed time counts (gram_f64_shape).
+__global__ void __launch_bounds__(256) k_gram_f64_wide(const double2* __restrict__ F, GramParams g,
+                                                       const double* __restrict__ wsq, double* __restrict__ partial) {
+  __shared__ double As[32][65];
+  __shared__ double Bs[32][65];
+  int I, J;
+  pair_of(blockIdx.x, g.ntiles, I, J);
+  const int s = blockIdx.y;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  double acc[4][4] = {};
+  const int c0 = s * g.chunks_per_split;
+  const int c1 = min(c0 + g.chunks_per_split, g.nchunks);
+  for (int c = c0; c < c1; ++c) {
+    const int kb = c * 16;
+    for (int idx = threadIdx.x; idx < 2 * 64 * 16; idx += 256) {
+      const int which = idx >> 10;  // 0: A rows, 1: B rows
+      const int r = (idx >> 4) & 63, kk = idx & 15;
+      const int row = (which ? J : I) * 64 + r;
+      const int k = kb + kk;
+      double2 v = {0.0, 0.0};
+      if (row < g.D && k <= g.N) {
+        v = F[(int64_t)row * g.ld + k];
+        const double sc = wsq[k];
+        v.x *= sc;
+        v.y *= sc;
+      }
+      if (which) { Bs[2 * kk][r] = v.x; Bs[2 * kk + 1][r] = v.y; }
+      else { As[2 * kk][r] = v.x; As[2 * kk + 1][r] = v.y; }
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int kr = 0; kr < 32; ++kr) {
+      double a[4], b[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) { a[q] = As[kr][ty * 4 + q]; b[q] = Bs[kr][tx * 4 + q]; }
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y) acc[x][y] = fma(a[x], b[y], acc[x][y]);
+    }
+    __syncthreads();
+  }
+  double* out = partial + ((int64_t)blockIdx.x * g.splits + s) * 64 * 64;
+#pragma unroll
+  for (int x = 0; x < 4; ++x)
+#pragma unroll
+    for (int y = 0; y < 4; ++y) out[(ty * 4 + x) * 64 + tx * 4 + y] = acc[x][y];
+}
+
+constexpr int kF64WideMin = 256;           // assets; with fewer the 4 x 4 tiles were always faster
+constexpr int kF64WideCtas = 2 * 152;
+
+// Tiles, chunks and splits of the FP64 contraction. 4 x 4 tiles: about eight CTAs per SM
 // (the float64 pipe is busy from two on; eight keep the last wave short), at
 // least four chunks per warp (a CTA's reductions cost about as much as two),
-// at most max_splits.
+// at most max_splits. 64 x 64 tiles: CTAs for two waves, partial tiles a small
+// fraction of the operand's bytes. Between the two by the multiply-adds that fit into
+// the time each takes: whole waves of 16-mode chunks at 0.83 of the pipe's cycles
+// against the wanted products and 8900 a CTA (its launch, tile search and sums). With
+// the other form and with the one taken: D = 1000, N = 30: 579 and 108 us; D = 2000,
+// N = 30: 2861 and 382; D = 1000, N = 2000: 4624 and 4235; D = 320, N = 8000: 1854 and
+// 1755; D = 600, N = 2000: 2820 and 1682; D = 700, N = 500: 1113 and 702.
 void gram_f64_shape(GramParams* g, int max_splits) {
   constexpr int kTargetCtas = 8 * 152;
   g->tile = 4;
@@ -151,17 +214,41 @@ void gram_f64_shape(GramParams* g, int max_splits) {
   S = S < max_splits ? S : max_splits;
   g->splits = S > 1 ? S : 1;
   g->chunks_per_split = (g->nchunks + g->splits - 1) / g->splits;
+  if (g->D < kF64WideMin) return;
+  GramParams w = *g;
+  w.tile = 64;
+  w.ntiles = (w.D + 63) / 64;
+  w.npairs = w.ntiles * (w.ntiles + 1) / 2;
+  w.chunk = 16;
+  w.nchunks = (w.N + 1 + 15) / 16;
+  const double operand = (double)w.D * 2.0 * (w.N + 1) * 8.0, tile_bytes = 64.0 * 64.0 * 8.0;
+  const int by_bytes = (int)std::max(1.0, ceil(operand / (4.0 * w.npairs * tile_bytes)));
+  S = std::max(1, std::min({w.nchunks, std::max(1, kF64WideCtas / w.npairs), by_bytes}));
+  w.chunks_per_split = (w.nchunks + S - 1) / S;
+  w.splits = (w.nchunks + w.chunks_per_split - 1) / w.chunks_per_split;
+  const int64_t waves = ((int64_t)w.npairs * w.splits + 151) / 152;
+  const double wide = 0.83 * (double)waves * w.chunks_per_split * 152.0 * (2.0 * 16.0 * 64.0 * 64.0);
+  const double narrow = 1.03 * (double)g->npairs * (32.0 * (g->N + 1) + 8900.0);
+  if (wide < narrow) *g = w;
 }
 
 size_t gram_f64_partial_bytes(int D) {
-  // splits <= target CTAs / pairs + 1, 16 sums each
+  // 4 x 4: splits <= target CTAs / pairs + 1, 16 sums each; 64 x 64: as many CTAs as
+  // aimed at, or a pair each
   const size_t nt = ((size_t)D + 3) / 4, np = nt * (nt + 1) / 2;
-  return (np + 8 * 152) * 16 * sizeof(double);
+  const size_t narrow = (np + 8 * 152) * 16 * sizeof(double);
+  if (D < kF64WideMin) return narrow;
+  const size_t wt = ((size_t)D + 63) / 64, wp = wt * (wt + 1) / 2;
+  return std::max(narrow, std::max(wp, (size_t)kF64WideCtas) * 64 * 64 * sizeof(double));
 }
 
 cudaError_t launch_gram_f64(const void* coeffs, const GramParams& g, const double* wsq, double* partial,
                             cudaStream_t s) {
   dim3 grd(g.npairs, g.splits);
+  if (g.tile == 64) {
+    k_gram_f64_wide<<<grd, 256, 0, s>>>((const double2*)coeffs, g, wsq, partial);
+    return cudaGetLastError();
+  }
   k_gram_f64<<<grd, 32 * kF64Warps, 0, s>>>((const double2*)coeffs, g, wsq, partial);
   return cudaGetLastError();
 }
