@@ -607,6 +607,7 @@ __device__ __forceinline__ double sum_splits(const TP* __restrict__ partial, con
   const int p = I * g.ntiles - I * (I - 1) / 2 + (J - I);
   const int64_t base = (int64_t)p * g.splits * g.tile * g.tile + (int64_t)(i % g.tile) * g.tile + (j % g.tile);
   const int64_t step = (int64_t)g.tile * g.tile;
+  if (g.splits == 1) return (double)partial[base];  // float64 additions are slow: 13 us of 4e6 entries
   double acc[4] = {};
   int s = 0;
   for (; s + 4 <= g.splits; s += 4)
