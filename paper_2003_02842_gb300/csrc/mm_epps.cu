@@ -37,8 +37,8 @@
 // problems of 10 assets, 64 cutoffs to 14,399 (590 MB), and 232 us at 16
 // problems on one CTA each; now 206 us and 73 us.
 //
-// Small problems (k_epps_small: float32, at most 4 assets and 511 modes) take a
-// warp each: one mode a lane, prefix sums over k by a warp scan in float pairs
+// Small problems (k_epps_small: float32, at most 4 assets and 511 modes, epps_small)
+// take a warp each: one mode a lane, prefix sums over k by a warp scan in float pairs
 // (48 bits, as the float64 pipe would bound it), for Fejer the prefix of the
 // prefix (sum_{k<=N} (N - k) q_k = sum_{m<N} P(m)); the lane of a cutoff writes
 // its Sigma and R. 8192 problems of two assets and 50 cutoffs:
@@ -426,12 +426,29 @@ __global__ void __launch_bounds__(kEppsThreads) k_epps_small(const float2* __res
   if (zero_var) atomicOr(status, ST_ZERO_VAR);
 }
 
+// A warp a problem is a chain of 32-mode steps, each a scan per pair of assets: 7 us
+// to 250 us by its length, however few the problems. So it is taken for short chains,
+// and for long ones from as many problems on as keep CTAs of the other form busy for
+// longer. Steps times (pairs + 1), both forms measured at 1 to 4 assets, 20 to 511 modes
+// and 4 to 8192 problems (us, a warp each against CTAs): 4 assets, 511 modes, 32 problems
+// 74 against 15; 2 assets, 200 modes, 150 problems 25 against 14; 3 assets, 50 modes, 600
+// problems 12 against 18; 2 assets, 350 modes, 2500 problems 30 against 41.
+constexpr int kSmallShort = 12;      // chains that are always shorter
+constexpr int kSmallLong = 128;      // and never
+constexpr int kSmallPerStep = 28;    // problems per step between the two
+
+bool epps_small(int Dg, int ld, int G) {
+  if (Dg > kSmallAssets || ld > kSmallModes) return false;
+  const int chain = (Dg * (Dg + 1) / 2 + 1) * ((ld + 31) / 32);
+  return chain <= kSmallShort || (chain <= kSmallLong && G >= kSmallPerStep * chain);
+}
+
 template <typename T, int DG>
 cudaError_t launch_dg(bool fejer, const EppsArgs& a, cudaStream_t s) {
   constexpr int NP = Pairs<DG>::n;
   const int* gate = a.status + 1;
   if constexpr (sizeof(T) == 4 && DG <= kSmallAssets) {
-    if (a.ld <= kSmallModes) {
+    if (epps_small(DG, a.ld, a.G)) {
       const int grid = std::min((a.G + 7) / 8, 6 * 152);
       auto small = [&](auto fn) {
         fn<<<grid, kEppsThreads, 0, s>>>((const float2*)a.coef, a.ld, a.cut, a.ncut, a.G, (float*)a.sigma,
