@@ -79,9 +79,15 @@ typedef enum { MM_BASIS_DIRICHLET = 0, MM_BASIS_FEJER = 1 } mm_basis;
  * Sec. 2.2.5. */
 typedef enum { MM_KERNEL_GAUSS = 0, MM_KERNEL_KB = 1, MM_KERNEL_ES = 2 } mm_kernel;
 
-/* MM_PREC_FP64: float64 data and results; spreading and FFT in float pairs (47
- * bits) where their error is 50 times below the tolerance (tol >= 5e-13), every
- * stage in float64 below that. MM_PREC_MIXED_*: rescaling, phase
+/* MM_PREC_FP64: float64 data and results. Phases are kept to 2^-40 of a grid cell
+ * and the cell scale to float64: together some 1e-12 of a row's rms at N = 5000,
+ * 3e-12 at N = 20,000. At tolerances of 1e-12 and more, spreading, FFT and
+ * deconvolution run in float pairs (47 bits), which add 3e-14 to 8e-14 of a row in
+ * the norm of Eq. (15) and at most half the tolerance to the modes next to the
+ * cutoff, where the deconvolution is largest (at 1e-12: 3e-13 rms for the Gaussian
+ * kernel, 1e-13 for the others). Tolerances below 1e-12 keep every stage in float64
+ * (9e-13, say, with the stencil of 1e-12 for the ES and Kaiser-Bessel kernels).
+ * MM_PREC_MIXED_*: rescaling, phase
  * reduction to grid offsets, differencing into returns and the diagonal
  * normalisation in float64; spreading, FFT and deconvolution in float32; the
  * contraction on the tensor cores as split bf16 (hi*hi + hi*lo + lo*hi) or
@@ -363,9 +369,10 @@ typedef struct {
   mm_precision prec;     /* MM_PREC_MIXED_*: stages (a)-(c) in float32; the sweep
                             contraction accumulates in float32 on the CUDA cores
                             (D <= 12 makes it memory-bound), normalised in float64.
-                            MM_PREC_FP64: the same form in float64 throughout
-                            (complex128 coefficients, float64 Sigma and R): the
-                            mixed form's comparator */
+                            MM_PREC_FP64: the same form with complex128
+                            coefficients (by stages as mm_precision says), a float64
+                            sweep and float64 Sigma and R: the mixed form's
+                            comparator */
   int32_t spread_algo;   /* stages (a)-(c) as mm_plan_desc.spread_algo (0 .. 3) */
   int32_t reserved[4];   /* must be zero */
 } mm_batch_desc;

@@ -280,6 +280,27 @@ double fit_pair_poly(const SpreadParams& s, PairPoly* out) {
   return worst;
 }
 
+// Rounding of the float-pair spreading and FFT in a coefficient where the averaging
+// kernel's transform is at its peak, relative to the rms of its row: 0.9e-14 to 1.1e-14
+// measured against float64 throughout (three kernels, tolerances 1e-6 to 1e-12, 30 to
+// 20,000 modes; roll-offs of 2 to 30 raise it by just that factor at the modes next to
+// the cutoff: 2.7e-13 rms for the Gaussian kernel at 1e-12, 1.1e-13 ES, 7e-14
+// Kaiser-Bessel).
+constexpr double kPairRounding = 1.2e-14;
+
+// Largest ratio of the kernel's transform at mode 0 to that at a mode k <= N, k < M_r / 4
+// (trapezoidal rule on the kernel as spread; a few per cent are enough).
+double kernel_rolloff(const SpreadParams& s) {
+  const int m = 8, last = s.msp * m;
+  double at_0 = 0.0, at_N = 0.0;
+  for (int i = -last; i <= last; ++i) {
+    const double x = (double)i / m, v = kernel_at(s, x);
+    at_0 += v;
+    at_N += v * cos(0.5 * kPi * x);
+  }
+  return at_0 / at_N;
+}
+
 // M_sp rules of Sec. 2.2.5 (sigma = 2).
 int msp_rule(mm_kernel k, double eps) {
   const double sigma = 2.0;
@@ -592,11 +613,13 @@ mm_status configure(mm_plan p, int N) {
     }
     p->poly_ok = p->poly_err <= std::max(3.0e-7, 0.1 * p->desc.tol);
   }
-  // FP64: taps in float pairs where their error (at most 1e-14) and the fit's
-  // are 50 times below the NUFFT tolerance; float64 throughout otherwise
+  // FP64: spreading and FFT in float pairs down to a tolerance of 1e-12, where what they
+  // add to a coefficient next to the cutoff stays below half the tolerance: the pairs'
+  // rounding and the taps' fit error, raised by the deconvolution's largest factor.
+  // Float64 throughout below 1e-12 and where that does not hold.
   p->pair_ok = false;
-  if (p->fp64 && s.algo == 0 && p->tune_poly != 0 && p->desc.tol >= 5.0e-13)
-    p->pair_ok = fit_pair_poly(s, &p->pair_poly) + 1.0e-14 <= 0.02 * p->desc.tol;
+  if (p->fp64 && s.algo == 0 && p->tune_poly != 0 && p->desc.tol >= 1.0e-12)
+    p->pair_ok = kernel_rolloff(s) * (fit_pair_poly(s, &p->pair_poly) + kPairRounding) <= 0.5 * p->desc.tol;
   // per-asset FFT: mixed path, the complex grid fits in shared memory and n
   // factors into at most kMaxAssetPasses compiled radices
   AssetFft af{};

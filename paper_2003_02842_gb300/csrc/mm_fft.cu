@@ -19,8 +19,8 @@
 // (FloatPair; mm_spread.cu's scatter leaves such a grid): some 80 float64
 // operations per point set both passes' time on the float64 pipe, 179 + 222 us at
 // 100 rows of 20,250 points; in float pairs 55 + 67 us. The pairs' rounding
-// (2^-47 an operation) adds about 1e-14 to coefficients whose truncation is
-// 1e-12 at the tightest tolerance that takes this path.
+// (2^-47 an operation) adds about 1e-14 to a coefficient before the deconvolution
+// (kPairRounding), for a tolerance of 1e-12 at the tightest.
 #include <math.h>
 
 #include <type_traits>

@@ -1075,9 +1075,10 @@ cudaError_t launch_spread_poly(const int64_t* off, const int* rb0, const void* r
 // 97 us. The grid leaves as float pairs, which the FFT passes keep.
 //
 // Error: against the kernel in 64 bits a tap is off by at most 7e-15 of the peak
-// (8e-16 rms; measured for the three kernels at tol 1e-12), so the path is taken
-// for tolerances from 5e-13 up, where the kernel's own truncation is at least 100
-// times that; tighter tolerances keep float64 throughout.
+// (8e-16 rms; measured for the three kernels at tol 1e-12). With the FFT's rounding
+// that is some 1e-14 of a coefficient before the deconvolution, whose largest factor
+// decides where the path is taken (configure); tolerances below 1e-12 keep
+// float64 throughout.
 //
 // Scales: V = max |v| < 2^exV over the tile's n records (from exponent fields:
 // returns of any float64 magnitude), eh = 21 - exV - max(0, bitlen(n) - 9), so

@@ -68,9 +68,9 @@ def test_tight_tolerances_keep_float64_taps():
     assert rel_l2_rows(F, G).max() <= 2e-15
 
 
-def _coeffs(ev, N, algo):
+def _coeffs(ev, N, algo, kernel="es", tol=1e-12):
     import paper_2003_02842_gb300 as mm
-    plan = mm.mm_plan_create(D=ev.D, N_max=N, max_events=ev.n_events, tol=1e-12, kernel="es", prec="fp64",
+    plan = mm.mm_plan_create(D=ev.D, N_max=N, max_events=ev.n_events, tol=tol, kernel=kernel, prec="fp64",
                              spread_algo=algo)
     F, _ = mm.mm_coeffs(plan, *to_dev(ev), N)
     mm.mm_plan_sync(plan)
@@ -108,3 +108,32 @@ def test_subnormal_returns():
     assert np.abs(np.diff(ev.logp)).max() < 2.0**-1022
     F, G = _coeffs(ev, 40, "scatter") * 2.0**1000, _coeffs(ev, 40, "gather") * 2.0**1000
     assert np.linalg.norm(G) > 0 and rel_l2_rows(F, G).max() <= 1e-9
+
+
+def _mode_errors(ev, N, kernel, tol):
+    """|scatter - gather| (float64 throughout) of each mode, rms over the rows, in units of a row's rms."""
+    F, G = _coeffs(ev, N, "scatter", kernel, tol), _coeffs(ev, N, "gather", kernel, tol)
+    rms = np.sqrt((np.abs(G) ** 2).mean(1, keepdims=True))
+    return np.sqrt(((np.abs(F - G) / rms) ** 2).mean(0))
+
+
+@pytest.mark.parametrize("kernel", ["es", "kb", "gauss"])
+@pytest.mark.parametrize("N", [30, 700, 4096, 10124, 20000])
+def test_modes_next_to_the_cutoff(kernel, N):
+    # The deconvolution raises the pairs' rounding most there; what is promised is half the
+    # tolerance, rms over the last fiftieth of the modes, and a tenth of it over a row
+    ev = synth.random_events(70 + N, D=6, n_range=(200, 6000), T=28800.0)
+    for tol in (1e-10, 1e-12):
+        e = _mode_errors(ev, N, kernel, tol)
+        assert np.sqrt((e[-max(1, (N + 1) // 50):] ** 2).mean()) <= 0.5 * tol
+        assert np.sqrt((e**2).mean()) <= 1e-13
+
+
+@pytest.mark.parametrize("kernel", ["es", "kb", "gauss"])
+@pytest.mark.parametrize("N", [30, 700, 1000, 5000])
+def test_pairs_from_a_tolerance_of_1e_12(kernel, N):
+    # Two float64 paths that only add in another order agree to some 1e-15 of a row's rms, the
+    # pairs differ by 1e-14 and more: which one ran shows on both sides of the line
+    ev = synth.random_events(90 + N, D=4, n_range=(200, 3000), T=28800.0)
+    rms = {tol: float(np.sqrt((_mode_errors(ev, N, kernel, tol) ** 2).mean())) for tol in (1e-12, 9.9e-13)}
+    assert rms[1e-12] > 4e-15 and rms[9.9e-13] < 3e-15
