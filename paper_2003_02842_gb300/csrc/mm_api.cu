@@ -213,8 +213,10 @@ double fit_pair_poly(const SpreadParams& s, PairPoly* out) {
   if (last > kPairMax) return 1e300;
   out->npair = last;
   out->one_sided = last > s.khi ? 1 : 0;
-  double node[n], T[n][n];
+  double node[n], T[n][n], C[n][n];  // C: T_i at the nodes (1274 cosines a fit at 13 pairs otherwise)
   for (int m = 0; m < n; ++m) node[m] = cos(kPi * (m + 0.5) / n);
+  for (int i = 0; i < n; ++i)
+    for (int m = 0; m < n; ++m) C[i][m] = cos(kPi * i * (m + 0.5) / n);
   memset(T, 0, sizeof(T));
   T[0][0] = 1.0;
   T[1][1] = 1.0;
@@ -234,7 +236,7 @@ double fit_pair_poly(const SpreadParams& s, PairPoly* out) {
       double in_t[n] = {};  // powers of t = 8 y - 1
       for (int i = 0; i < n; ++i) {
         double acc = 0.0;
-        for (int m = 0; m < n; ++m) acc += v[h][m] * cos(kPi * i * (m + 0.5) / n);
+        for (int m = 0; m < n; ++m) acc += v[h][m] * C[i][m];
         acc *= (i == 0 ? 1.0 : 2.0) / n;
         for (int q = 0; q < n; ++q) in_t[q] += acc * T[i][q];
       }
@@ -254,8 +256,8 @@ double fit_pair_poly(const SpreadParams& s, PairPoly* out) {
         }
       }
     }
-    for (int q = 0; q <= 32; ++q) {
-      const double z = q / 64.0, y = z * z;
+    for (int q = 0; q <= 16; ++q) {
+      const double z = q / 32.0, y = z * z;
       double E = 0.0, O = 0.0;
       for (int i = n - 1; i >= 0; --i) {
         E = E * y + mono[0][i];
@@ -288,17 +290,18 @@ double fit_pair_poly(const SpreadParams& s, PairPoly* out) {
 // Kaiser-Bessel).
 constexpr double kPairRounding = 1.2e-14;
 
-// Largest ratio of the kernel's transform at mode 0 to that at a mode k <= N, k < M_r / 4
-// (trapezoidal rule on the kernel as spread; a few per cent are enough).
-double kernel_rolloff(const SpreadParams& s) {
-  const int m = 8, last = s.msp * m;
-  double at_0 = 0.0, at_N = 0.0;
+// Ratio of the kernel's transform at mode 0 to that at a mode of `turns` turns a cell
+// (k / M_r; below a quarter for every k <= N), by the trapezoidal rule on the kernel as
+// spread, two points a cell; a few per cent are enough.
+double kernel_rolloff(const SpreadParams& s, double turns) {
+  const int m = 2, last = s.msp * m;
+  double at_0 = 0.0, at_k = 0.0;
   for (int i = -last; i <= last; ++i) {
     const double x = (double)i / m, v = kernel_at(s, x);
     at_0 += v;
-    at_N += v * cos(0.5 * kPi * x);
+    at_k += v * cos(2.0 * kPi * turns * x);
   }
-  return at_0 / at_N;
+  return at_0 / at_k;
 }
 
 // M_sp rules of Sec. 2.2.5 (sigma = 2).
@@ -411,6 +414,8 @@ struct mm_plan_s {
   double poly_t1 = 0.0, poly_b = 0.0;
   bool poly_ok = false;   // float32 spreading with polynomial taps and integer accumulation
   PairPoly pair_poly{};
+  double pair_err = -1.0;  // its part of a coefficient's error next to the cutoff (< 0: not fitted yet)
+  double pair_t1 = 0.0, pair_b = 0.0;
   bool pair_ok = false;   // FP64 spreading in float pairs
   int tune_poly = -1;     // autotuner override: 0 off
   cudaStream_t last = nullptr;
@@ -618,8 +623,18 @@ mm_status configure(mm_plan p, int N) {
   // rounding and the taps' fit error, raised by the deconvolution's largest factor.
   // Float64 throughout below 1e-12 and where that does not hold.
   p->pair_ok = false;
-  if (p->fp64 && s.algo == 0 && p->tune_poly != 0 && p->desc.tol >= 1.0e-12)
-    p->pair_ok = kernel_rolloff(s) * (fit_pair_poly(s, &p->pair_poly) + kPairRounding) <= 0.5 * p->desc.tol;
+  if (p->fp64 && s.algo == 0 && p->tune_poly != 0 && p->desc.tol >= 1.0e-12) {
+    // kept as the float32 fit is: the ES taps do not depend on the cutoff (28.8 us of
+    // host time a call with another cutoff each; 40.3 with a fit in each)
+    if (!(p->pair_err >= 0.0 && p->pair_t1 == s.g_t1 && p->pair_b == s.kb_b) &&
+        !(p->pair_err >= 0.0 && s.kernel == MM_KERNEL_ES)) {
+      const double turns = s.kernel == MM_KERNEL_ES ? 0.25 : (double)N / (double)Mr;
+      p->pair_err = kernel_rolloff(s, turns) * (fit_pair_poly(s, &p->pair_poly) + kPairRounding);
+      p->pair_t1 = s.g_t1;
+      p->pair_b = s.kb_b;
+    }
+    p->pair_ok = p->pair_err <= 0.5 * p->desc.tol;
+  }
   // per-asset FFT: mixed path, the complex grid fits in shared memory and n
   // factors into at most kMaxAssetPasses compiled radices
   AssetFft af{};

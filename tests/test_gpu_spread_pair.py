@@ -137,3 +137,18 @@ def test_pairs_from_a_tolerance_of_1e_12(kernel, N):
     ev = synth.random_events(90 + N, D=4, n_range=(200, 3000), T=28800.0)
     rms = {tol: float(np.sqrt((_mode_errors(ev, N, kernel, tol) ** 2).mean())) for tol in (1e-12, 9.9e-13)}
     assert rms[1e-12] > 4e-15 and rms[9.9e-13] < 3e-15
+
+
+@pytest.mark.parametrize("kernel", ["es", "kb", "gauss"])
+def test_a_plan_at_one_cutoff_after_another(kernel):
+    # the fit that a plan keeps over cutoffs is the one that each cutoff needs: a new plan's
+    # coefficients, bit for bit (integer sums, a transform in a fixed order)
+    import paper_2003_02842_gb300 as mm
+    ev = synth.random_events(13, D=2, n_range=(100, 900), T=5000.0)
+    x = to_dev(ev)
+    plan = mm.mm_plan_create(D=2, N_max=3000, max_events=ev.n_events, tol=1e-12, kernel=kernel, prec="fp64")
+    for N in (700, 701, 31, 3000, 700, 1024):
+        F, _ = mm.mm_coeffs(plan, *x, N)
+        assert mm.mm_plan_sync(plan) == 0
+        assert np.array_equal(F.cpu().numpy(), _coeffs(ev, N, "scatter", kernel))
+    mm.mm_destroy(plan)
