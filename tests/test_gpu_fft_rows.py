@@ -42,3 +42,12 @@ def test_batch_rows_per_cta():
     for r in (0, 1, 151, 152, 303, 499):
         ref = oracle.coeffs_F(evs[r].offsets, evs[r].t, evs[r].logp, N)
         assert rel_l2_rows(F[r * D:(r + 1) * D], ref).max() <= 1e-5
+
+
+@pytest.mark.parametrize("D,N", [(305, 6000), (306, 6000), (456, 6000), (457, 6000), (608, 5000), (609, 4500)])
+def test_long_rows_in_several_waves(D, N):
+    # both sides of the line between two rows a CTA and a CTA a row
+    ev = synth.random_events(600 + D, D=D, n_range=(2, 12), T=900.0)
+    out = run(dict(tol=1e-6, kernel="es", basis="dirichlet", prec="bf16x3"), ev, N)
+    assert out["status"] == 0 and out["info"]["fft_algo"] == 0 and out["info"]["fft_split"] == 1
+    assert rel_l2_rows(out["F"], oracle.coeffs_F(ev.offsets, ev.t, ev.logp, N)).max() <= 1e-5
