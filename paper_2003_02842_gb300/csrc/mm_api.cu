@@ -1283,7 +1283,7 @@ mm_status mm_corr_pairwise(mm_plan p, const void* d_coeffs, int32_t N_coeffs, co
     MM_CUDA(launch_pairwise(p->fp64, p->desc.basis == MM_BASIS_FEJER, d_coeffs, N_coeffs + 1, p->pw_N, D,
                             p->pw_part, p->pw_sig, st));
   }
-  StageScope sc(p, MM_STAGE_REDUCE, st, psd_repair ? 2 : 1);
+  StageScope sc(p, MM_STAGE_REDUCE, st, 1 + (psd_repair ? psd_repair_launches(p->fp64, D) : 0));
   int* clip = d_clipped_or_null ? (int*)d_clipped_or_null : p->pw_clip;
   if (psd_repair) MM_CUDA(launch_psd_repair(p->fp64, p->pw_sig, p->pw_A, p->pw_V, D, clip, p->pw_log, p->pw_sync, p->status,
                                            st));

@@ -362,6 +362,7 @@ cudaError_t launch_pairwise(bool fp64, bool fejer, const void* coeffs, int ld, c
 size_t pairwise_part_bytes(int D);         // split partial sums and zeroed arrival counters
 cudaError_t launch_psd_repair(bool fp64, double* sig, double* A, double* V, int D, int* clipped, void* log,
                               void* sync, int* status, cudaStream_t s);
+int psd_repair_launches(bool fp64, int D);
 size_t psd_log_bytes(bool fp64, int D);    // the one-CTA iteration's rotation log
 size_t psd_sync_bytes();  // the multi-CTA repair's barrier and reduction words
 cudaError_t launch_pairwise_out(bool fp64, const double* sig, int D, void* sigma, void* R, int* status,

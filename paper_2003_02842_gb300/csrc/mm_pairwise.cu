@@ -753,6 +753,9 @@ cudaError_t launch_pairwise(bool fp64, bool fejer, const void* coeffs, int ld, c
 
 static bool psd_one_cta(bool fp64, int D) { return D <= (fp64 ? kPsdMaxD64 : kPsdMaxD); }
 
+// iteration, eigenvectors and product, or the cooperative kernel that does all
+int psd_repair_launches(bool fp64, int D) { return psd_one_cta(fp64, D) ? 3 : 1; }
+
 size_t psd_log_bytes(bool fp64, int D) {
   if (D > kPsdMaxD) D = kPsdMaxD;  // larger matrices use the multi-CTA iteration, which keeps none
   const size_t m = ((size_t)D + 1) & ~(size_t)1;

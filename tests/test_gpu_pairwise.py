@@ -137,3 +137,20 @@ def test_pairwise_rejects_bad_arguments():
     S, R, c = mm.mm_corr_pairwise(plan, F, 8, [8] * D)
     torch.cuda.synchronize()
     mm.mm_destroy(plan)
+
+
+@pytest.mark.parametrize("prec,D,repair", [("bf16x3", 20, 3), ("bf16x3", 159, 1), ("fp64", 20, 3), ("fp64", 113, 1)])
+def test_launches_are_counted(prec, D, repair):
+    # the pairwise sums and the output, and the repair's kernels: iteration, eigenvectors and
+    # product where one CTA iterates, one cooperative kernel beyond that
+    import torch
+
+    import paper_2003_02842_gb300 as mm
+    plan = mm.mm_plan_create(D=D, N_max=30, tol=1e-6, prec=prec)
+    F = torch.randn((D, 31), dtype=torch.complex128 if prec == "fp64" else torch.complex64, device="cuda")
+    for psd, want in ((False, 2), (True, 2 + repair)):
+        before = mm.mm_plan_get_info(plan)["launches"]
+        mm.mm_corr_pairwise(plan, F, 30, [30] * D, psd_repair=psd)
+        assert mm.mm_plan_get_info(plan)["launches"] - before == want
+    mm.mm_plan_sync(plan)
+    mm.mm_destroy(plan)
