@@ -371,7 +371,8 @@ struct mm_plan_s {
   double* pw_V = nullptr;         // (allocated on first use)
   int* pw_clip = nullptr;
   void* pw_sync = nullptr;        // the repair's barrier words and results
-  void* pw_part = nullptr;        // split partial sums
+  void* pw_part = nullptr;        // split partial sums and arrival counters,
+  bool pw_ready = false;          // cleared
   void* pw_log = nullptr;         // the one-CTA repair's rotations
   int acc_sel = 0;
   bool acc_dirty = true;          // clear both before the next contraction
@@ -444,10 +445,14 @@ struct mm_plan_s {
 
 namespace {
 
+// A failed call's error is reported once: it is not left for the next launch's check.
 #define MM_CUDA(call)                                 \
   do {                                                \
     cudaError_t e_ = (call);                          \
-    if (e_ != cudaSuccess) return MM_ERR_CUDA;        \
+    if (e_ != cudaSuccess) {                          \
+      cudaGetLastError();                             \
+      return MM_ERR_CUDA;                             \
+    }                                                 \
   } while (0)
 
 mm_status dalloc(mm_plan p, void** ptr, size_t bytes) {
@@ -1257,7 +1262,7 @@ mm_status mm_corr_pairwise(mm_plan p, const void* d_coeffs, int32_t N_coeffs, co
   for (int i = 0; i < D; ++i)
     if (h_N[i] < lo || h_N[i] > N_coeffs) return MM_ERR_CUTOFF;
   cudaStream_t st = (cudaStream_t)stream;
-  if (!p->pw_part) {  // first use; a failed attempt is resumed by the next call
+  if (!p->pw_ready) {  // first use; a failed attempt is resumed by the next call
     const size_t dd = (size_t)p->desc.D * p->desc.D * sizeof(double);
     const bool psd = p->desc.D <= pairwise_psd_max_assets();
     const size_t part = pairwise_part_bytes(p->desc.D);
@@ -1275,6 +1280,7 @@ mm_status mm_corr_pairwise(mm_plan p, const void* d_coeffs, int32_t N_coeffs, co
     need(&p->pw_part, part);
     if (a != MM_OK) return a;
     MM_CUDA(cudaMemsetAsync(p->pw_part, 0, part, st));
+    p->pw_ready = true;  // the arrival counters will be clear
   }
   p->last = st;
   MM_CUDA(cudaMemcpyAsync(p->pw_N, h_N, (size_t)D * sizeof(int), cudaMemcpyHostToDevice, st));

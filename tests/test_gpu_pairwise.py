@@ -154,3 +154,47 @@ def test_launches_are_counted(prec, D, repair):
         assert mm.mm_plan_get_info(plan)["launches"] - before == want
     mm.mm_plan_sync(plan)
     mm.mm_destroy(plan)
+
+
+def test_first_use_that_fails_to_clear_its_counters_is_repeated():
+    # The first call runs on a stream whose capture has been invalidated (by a host call that
+    # a capture does not allow): its allocations succeed, the clearing of the split sums'
+    # arrival counters is refused. The next call, on a working stream, has to clear them (in
+    # memory that may hold the 0xff bytes written here) and not to meet the first one's error.
+    import ctypes
+
+    import torch
+
+    import paper_2003_02842_gb300 as mm
+    D, N = 40, 4000
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    F = torch.randn((D, N + 1), dtype=torch.complex64, device="cuda", generator=gen)
+    Ns = [N - 10 * i for i in range(D)]
+    fresh = mm.mm_plan_create(D=D, N_max=N, tol=1e-6)
+    S0, R0, _ = mm.mm_corr_pairwise(fresh, F, N, Ns)
+    assert mm.mm_plan_sync(fresh) == 0
+
+    plan = mm.mm_plan_create(D=D, N_max=N, tol=1e-6)
+    R = torch.full((D, D), 7.0, device="cuda")
+    stream = torch.cuda.Stream()
+    x = torch.full((256 << 20,), 255, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    del x
+    torch.cuda.empty_cache()
+    cu = ctypes.CDLL("libcuda.so.1")
+    h = ctypes.c_void_p(stream.cuda_stream)
+    hN = (ctypes.c_int32 * D)(*Ns)
+    assert cu.cuStreamBeginCapture_v2(h, 2) == 0  # relaxed: allocations are allowed
+    try:
+        assert cu.cuStreamSynchronize(h) != 0  # not allowed: invalidates the capture
+        st = mm._lib.load().mm_corr_pairwise(plan.handle, ctypes.c_void_p(F.data_ptr()), N, hN, 0, None,
+                                             ctypes.c_void_p(R.data_ptr()), None, h)
+    finally:
+        graph = ctypes.c_void_p()
+        cu.cuStreamEndCapture(h, ctypes.byref(graph))
+    assert st != 0
+    S1, R1, _ = mm.mm_corr_pairwise(plan, F, N, Ns)
+    assert mm.mm_plan_sync(plan) == 0
+    assert torch.equal(S0, S1) and torch.equal(R0, R1)
+    mm.mm_destroy(plan)
+    mm.mm_destroy(fresh)
