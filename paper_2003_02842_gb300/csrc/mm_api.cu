@@ -1268,7 +1268,7 @@ mm_status mm_corr_pairwise(mm_plan p, const void* d_coeffs, int32_t N_coeffs, co
     const size_t part = pairwise_part_bytes(p->desc.D);
     mm_status a = MM_OK;
     auto need = [&](void** ptr, size_t bytes) {
-      if (a == MM_OK && !*ptr) a = dalloc(p, ptr, bytes);
+      if (a == MM_OK && bytes > 0 && !*ptr) a = dalloc(p, ptr, bytes);
     };
     need((void**)&p->pw_N, (size_t)p->desc.D * sizeof(int));
     need((void**)&p->pw_sig, dd);
@@ -1279,7 +1279,7 @@ mm_status mm_corr_pairwise(mm_plan p, const void* d_coeffs, int32_t N_coeffs, co
     need(&p->pw_log, psd_log_bytes(p->fp64, p->desc.D));
     need(&p->pw_part, part);
     if (a != MM_OK) return a;
-    MM_CUDA(cudaMemsetAsync(p->pw_part, 0, part, st));
+    if (part > 0) MM_CUDA(cudaMemsetAsync(p->pw_part, 0, part, st));
     p->pw_ready = true;  // the arrival counters will be clear
   }
   p->last = st;

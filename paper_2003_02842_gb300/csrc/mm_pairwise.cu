@@ -731,6 +731,7 @@ static int pairwise_splits(int D, int ld) {
 
 size_t pairwise_part_bytes(int D) {
   const size_t nt = ((size_t)D + kPT - 1) / kPT, tiles = nt * (nt + 1) / 2;
+  if (tiles >= (size_t)kPairwiseCtas) return 0;  // a CTA a tile
   return (tiles + kPairwiseCtas) * 256 * sizeof(double) + tiles * sizeof(int);
 }
 
@@ -757,7 +758,7 @@ static bool psd_one_cta(bool fp64, int D) { return D <= (fp64 ? kPsdMaxD64 : kPs
 int psd_repair_launches(bool fp64, int D) { return psd_one_cta(fp64, D) ? 3 : 1; }
 
 size_t psd_log_bytes(bool fp64, int D) {
-  if (D > kPsdMaxD) D = kPsdMaxD;  // larger matrices use the multi-CTA iteration, which keeps none
+  if (!psd_one_cta(fp64, D)) return 0;  // the multi-CTA iteration keeps none
   const size_t m = ((size_t)D + 1) & ~(size_t)1;
   return ((size_t)kJacobiSweeps * (m - 1) + 1) * (m / 2) * 2 * (fp64 ? 8 : 4);
 }

@@ -198,3 +198,20 @@ def test_first_use_that_fails_to_clear_its_counters_is_repeated():
     assert torch.equal(S0, S1) and torch.equal(R0, R1)
     mm.mm_destroy(plan)
     mm.mm_destroy(fresh)
+
+
+@pytest.mark.parametrize("prec,D", [("fp64", 120), ("bf16x3", 159), ("bf16x3", 560)])
+def test_scratch_of_large_matrices(prec, D):
+    # matrix, eigenvectors and estimate (float64 D x D each) and up to 1.4 MB of split sums; no
+    # log of rotations (4.6 MB at 120 assets in float64) where the whole GPU iterates, no
+    # split sums (2.5 MB at 560 assets) where every tile of pairs has one CTA
+    import torch
+
+    import paper_2003_02842_gb300 as mm
+    plan = mm.mm_plan_create(D=D, N_max=30, tol=1e-6, prec=prec)
+    before = mm.mm_plan_get_info(plan)["workspace_bytes"]
+    F = torch.randn((D, 31), dtype=torch.complex128 if prec == "fp64" else torch.complex64, device="cuda")
+    mm.mm_corr_pairwise(plan, F, 30, [30] * D, psd_repair=True)
+    assert mm.mm_plan_sync(plan) == 0
+    assert mm.mm_plan_get_info(plan)["workspace_bytes"] - before < 3 * 8 * D * D + 1500000
+    mm.mm_destroy(plan)
