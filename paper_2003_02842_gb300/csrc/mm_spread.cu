@@ -741,19 +741,24 @@ constexpr int kPolyManyRecords = 4096;
 // Sparse tiles, one word per cell. When no stretch of 2 NP cells (a stencil)
 // holds more than kOneRun records, a cell's sum is at most the largest sum W of
 // |v| over kOneRun records in a row, not that of the tile: with x = v phi 2^e,
-// e = 30 - ex(W), every cell's sum of the rounded x stays below 2^30 (1 + 1e-6)
-// + kOneRun / 2 < 2^31 in one int32, with a quantum of at most W 2^-29. The tile is
-// taken so only where W is at most kOneEven times the mean sum of a run, kOneRun
-// times the mean |v|: a tap is then off by at most 80 2^-30 of the mean |v|, 2^-24.5
-// of it rms, as the float32 product of a tap is, and a return that dwarfs the
-// others does not cost them their digits (they keep two words; Brownian returns
-// at Poisson times stay at about twice the mean). One word halves the
-// shared-memory reductions, which bound the taps, and the tile. With the shorter
-// taps below, the guessed search and the block sizes above the block workload's
+// e = 31 - ex(W kOneRoom), every cell's sum of the rounded x stays below 2^31 / kOneRoom
+// times the taps' largest value (1 and their fit error, at most 0.05 at the loosest
+// tolerance) + kOneRun / 2 < 2^31 in one int32, with a quantum of at most W 2^-30 1.07.
+// The tile is taken so only where W is at most kOneEven times the largest run of every
+// warp's records (32 in a row at a time): a tap is then off by at most 170 2^-31 of the
+// mean |v| of a run nearby, 2^-24.4 of it rms, as the float32 product of a tap is, and a
+// return that dwarfs the others does not cost them their digits (they keep two words;
+// Brownian returns at Poisson times stay at about twice; the sum of |v| over the
+// tile, reduced for this, cost 3 % of the kernel with 120 records a tile). Coefficients'
+// float32 rounding is 1 to 3 % above that with two words (1.87e-7 and 1.84e-7 of a row at
+// the block workload, beside a truncation of 3e-6; 2 to 4 % with a quantum of W 2^-29).
+// One word halves the shared-memory reductions, which bound the taps, and the tile. With
+// the shorter taps below, the guessed search and the block sizes above the block workload's
 // spreading took 18.4 us (20.2 us with two words a cell in every tile), 500 stocks'
 // day 128 us (143 us), 512 replications of ten assets 474 us (715 us).
 constexpr int kOneRun = 20;
-constexpr float kOneEven = 4.0f;
+constexpr float kOneEven = 8.0f;
+constexpr float kOneRoom = 1.0625f;
 
 // Taps k and 1 - k of a record are phi(a - z) and phi(a + z), a = k - 1/2,
 // z = d - 1/2: with tap k's polynomial E(z^2) + z O(z^2), tap 1 - k is
@@ -861,7 +866,7 @@ __global__ void __launch_bounds__(NTH, kPolyPerSm<NT, NTH>) k_spread_poly(const 
   float* ev_v = ev_d + EC;
   int* tile = reinterpret_cast<int*>(ev_v + EC);
   const uint32_t tile_s = (uint32_t)__cvta_generic_to_shared(tile);
-  __shared__ float s_sum[NTH / 32], s_max[NTH / 32], s_run[NTH / 32], s_all[NTH / 32];
+  __shared__ float s_sum[NTH / 32], s_max[NTH / 32], s_run[NTH / 32];
   const int64_t L = (int64_t)blockIdx.x * p.tile;
   const int Tlen = (int)min((int64_t)p.tile, p.Mr - L);
   auto clear = [&] {
@@ -878,13 +883,14 @@ __global__ void __launch_bounds__(NTH, kPolyPerSm<NT, NTH>) k_spread_poly(const 
     for (int i = threadIdx.x; i < n; i += NTH)
       load_record<float>(rb0, rd, rv, p, tr, L, c0 + i, ev_p[i], ev_d[i], ev_v[i]);
   };
-  // at most kOneRun records in any stencil's width, and the sums of |v|;
+  // at most kOneRun records in any stencil's width, and the largest sum of |v| over that
+  // many in a row (a shorter run at the end is part of one, or the tile has no longer one);
   // chunks overlap by a run, and the last one stays staged. Where the assets'
   // density makes dense tiles likely the widths are looked at first, so that such
   // a tile leaves before the sums, which cost half its taps (a barrier more: 1.5 us
   // of the block workload's spreading)
   bool sparse = Tlen <= cells;
-  float run = 0.f, all = 0.f;  // largest sum over a run, sum over the tile
+  float run = 0.f;
   int64_t cs = 0;
   int n = 0;
   while (true) {
@@ -892,7 +898,7 @@ __global__ void __launch_bounds__(NTH, kPolyPerSm<NT, NTH>) k_spread_poly(const 
     stage(cs, n);
     __syncthreads();
     const bool last = cs + n == ntot;
-    const int lim = last ? n : n - kOneRun;
+    const int lim = last ? max(min(n, 1), n - kOneRun + 1) : n - kOneRun;
     if (widths_first) {
       for (int i = threadIdx.x; i + kOneRun < n; i += NTH)
         sparse = sparse && ev_p[i + kOneRun] - ev_p[i] > 2 * NP;
@@ -906,7 +912,6 @@ __global__ void __launch_bounds__(NTH, kPolyPerSm<NT, NTH>) k_spread_poly(const 
 #pragma unroll
       for (int j = 0; j < kOneRun; ++j) w += i + j < n ? fabsf(ev_v[i + j]) : 0.f;
       run = fmaxf(run, w);
-      all += fabsf(ev_v[i]);
     }
     if (last) break;
     if (!__syncthreads_and(sparse)) {
@@ -916,25 +921,21 @@ __global__ void __launch_bounds__(NTH, kPolyPerSm<NT, NTH>) k_spread_poly(const 
     cs += EC - kOneRun;
   }
   run = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(run)));  // not negative
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
-  if ((threadIdx.x & 31) == 0) {
-    s_run[threadIdx.x >> 5] = run;
-    s_all[threadIdx.x >> 5] = all;
-  }
+  if ((threadIdx.x & 31) == 0) s_run[threadIdx.x >> 5] = run;
   sparse = __syncthreads_and(sparse);
-  all = 0.f;
+  float low = INFINITY;  // the smallest of the warps' largest runs (of those that are not zero)
 #pragma unroll
   for (int w = 0; w < NTH / 32; ++w) {
-    run = sparse ? fmaxf(run, s_run[w]) : 0.f;
-    all += s_all[w];
+    const float r = s_run[w];
+    run = sparse ? fmaxf(run, r) : 0.f;
+    low = fminf(low, r > 0.f ? r : INFINITY);
   }
-  const bool even = run * (float)ntot <= kOneEven * (float)kOneRun * all;
+  const bool even = run <= kOneEven * low;
   // 2^e and 2^-e have to be normal floats
   if (sparse && even && run < 1.0e30f && (run > 1.0e-27f || run == 0.f)) {
     int ex = 0;
-    if (run > 0.f) frexpf(run, &ex);  // run < 2^ex
-    const int e = 30 - ex;
+    if (run > 0.f) frexpf(run * kOneRoom, &ex);  // run kOneRoom < 2^ex
+    const int e = 31 - ex;
     const float scale = __int_as_float((127 + e) << 23), inv = __int_as_float((127 - e) << 23);
     spread_one_word<NP, NTH>(ev_p, ev_d, ev_v, n, Tlen, taps, scale, tile_s);
     for (int64_t c0 = 0; c0 < cs; c0 += EC) {  // the records before the staged chunk
@@ -993,14 +994,14 @@ __global__ void __launch_bounds__(NTH, kPolyPerSm<NT, NTH>) k_spread_poly(const 
         stage(c0, m);
       }
       __syncthreads();
-      const int all = m;
+      const int staged = m;
       if (more) {
-        const int q = before(s0 + half - p.khi, all);
-        if (q < all && next == ntot) next = c0 + q;
-        m = before(s0 + half - p.klo, all);
+        const int q = before(s0 + half - p.khi, staged);
+        if (q < staged && next == ntot) next = c0 + q;
+        m = before(s0 + half - p.klo, staged);
       }
       spread_chunk<NT, NTH>(ev_p, ev_d, ev_v, m, len, p.klo - s0, poly, ts, tile_s, tile_s + 4u * half, AllCells{});
-      if (m < all) break;  // uniform: the rest lies beyond the part
+      if (m < staged) break;  // uniform: the rest lies beyond the part
     }
     from = next;
     __syncthreads();

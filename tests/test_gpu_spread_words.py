@@ -120,3 +120,27 @@ def test_wide_stencils(kernel, tol, msp, n):
     F = F.cpu().numpy().astype(np.complex128)
     mm.mm_destroy(plan)
     assert rel_l2_rows(F, _coeffs(ev, 1000, kernel, "fp64", tol=tol)).max() <= 1e-6
+
+
+@pytest.mark.parametrize("tol", [1e-6, 1e-3])
+@pytest.mark.parametrize("run", [0.94, 0.9411, 0.9412, 0.9999, 1.0001, 1.88, 1.883])
+def test_one_word_filled_to_its_last_bit(run, tol):
+    # 30 groups of 20 records within a ten-thousandth of a cell, of one sign: a cell gets the
+    # whole sum of a run, `run`, around the powers of two where the word's scale changes
+    # (run times 1.0625 below and above one and two); an overflow would turn the sign
+    import torch
+
+    import paper_2003_02842_gb300 as mm
+    N, T = 1020, 4096.0
+    t = (128.0 * np.arange(1, 31)[:, None] + 1e-5 * np.arange(20)[None, :]).ravel()
+    p = np.arange(len(t) + 1) * (run / 20)
+    off = torch.tensor([0, len(t) + 1]).cuda()
+    x = (off, torch.from_numpy(np.append(t, 4090.0)).cuda(), torch.from_numpy(p).cuda())
+    F = []
+    for prec in ("bf16x3", "fp64"):
+        plan = mm.mm_plan_create(D=1, N_max=N, max_events=len(p), tol=tol, prec=prec)
+        c, _ = mm.mm_coeffs(plan, *x, N, window=(0.0, T))
+        assert mm.mm_plan_sync(plan) == 0 and mm.mm_plan_get_info(plan)["Mr"] == 4096
+        F.append(c.cpu().numpy().astype(np.complex128))
+        mm.mm_destroy(plan)
+    assert rel_l2_rows(F[0], F[1]).max() <= max(1e-6, 0.2 * tol)
