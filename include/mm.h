@@ -449,6 +449,11 @@ mm_status mm_batch_get_info(mm_batch batch, mm_batch_info* info);
  * at least one and at most max_slots. Results are written to the caller's
  * host buffers; completions are polled, out of order, with host timestamps.
  *
+ * Host: the scheduler thread polls the slots' events while any request is in
+ * flight, up to 500 times in a row with a yield in between (so that one host core
+ * is busy while short requests follow one another), then every 5 us or so of
+ * sleep; without requests it sleeps.
+ *
  * Resident coefficients (cache_rows > 0): the coefficients of each requested
  * asset over the request's window at its cutoff stay on the device (rows of
  * N_max + 1, least recently used evicted first), and a later request with
